@@ -10,9 +10,9 @@
 // of 128 ReLU units; a linear output of C x 64 values, the residual in noise
 // units: refined = c + s x output.  FP32 weights and arithmetic.  The layers are GEMMs
 // over a batch of groups (k_gemm: 64 x 64 output tiles, 16-deep slabs in
-// shared memory, 4 x 4 outputs per thread); the weight gradients reduce
-// over the batch with a split of the reduction and a fixed-order sum of the
-// parts, so training is deterministic.
+// shared memory, 8 x 4 outputs per thread); the weight gradients (k_wgrad)
+// reduce over the batch with a split of the reduction and a fixed-order sum
+// of the parts, so training is deterministic.
 //
 // Denoising (hts_denoise_ra): the mean patch of every group (k_group_means),
 // its coordinates, the network with the call's estimated sigma, the refined
@@ -50,11 +50,12 @@ struct hts_fcn {
     size_t cap = 0;                       // samples the activation buffers hold
     float *X = nullptr;                   // features [n][din]
     float *act[3] = {};                   // layer outputs [n][nout[l]]
-    float *d0 = nullptr, *d1 = nullptr;   // gradients of layer outputs [n][HID or dout]
-    size_t cap_part = 0;
-    float *part = nullptr;                // split-reduction parts
-    double *loss = nullptr;               // accumulated loss
+    size_t cap_train = 0;                 // samples the training buffers hold
+    float *dy[3] = {};                    // gradients of the layer outputs [n][nout[l]]
     double *lpart = nullptr;              // per-block loss parts
+    size_t cap_part = 0;
+    float *part = nullptr;                // split-reduction parts, each a parameter vector
+    double *loss = nullptr;               // accumulated loss
     float *sig = nullptr;                 // the call's sigma for the features (denoising)
 };
 
@@ -75,81 +76,212 @@ hts_status cu(cudaError_t e, const char *what) {
     return report(e == cudaErrorMemoryAllocation ? HTS_ENOMEM : HTS_ECUDA, buf);
 }
 
-// C(m, n) = sum_k A(m, k) B(n, k), A(m, k) = A[m * am + k * ak], B(n, k) = B[n * bn + k * bk].
-// parts == nullptr: Cout[m * ldc + n] = act(C + bias[n]) (act: 1 = ReLU, 2 = times (mask[m * ldc + n] > 0));
-// else the reduction range [z * kchunk, (z + 1) * kchunk) of block z goes to parts[z][m][n] as it is.
-__global__ void __launch_bounds__(256) k_gemm(const float *__restrict__ A, long am, long ak, const float *__restrict__ B,
-                                              long bn, long bk, int M, int N, int K, int kchunk,
-                                              const float *__restrict__ bias, int act, const float *__restrict__ mask,
-                                              float *__restrict__ Cout, int ldc, float *__restrict__ parts) {
-    __shared__ float sA[TK][TM + 4], sB[TK][TN + 4];
+// C(m, n) = sum_k A(m, k) B(n, k) over a 64 x 64 tile, FP32, k in ascending order.  Bound by FP32 issue at large
+// M and by load latency at small M: a block of 128 threads holds 8 x 4 outputs per thread (3 shared-memory float4
+// reads per 32 FMAs), and the next 16-deep slab travels global memory -> registers while the current one is
+// multiplied (two shared buffers, one barrier per slab).  AK / BK: the operand is contiguous along k (A[m * lda +
+// k]), else along m / n (A[k * lda + m]); either way a thread loads float4s along the contiguous axis, which is why
+// the leading dimensions and N (for BK false) are multiples of 4.  Before (4 x 4 outputs, scalar loads that strode
+// over rows in the forward pass, no overlap): 38 us per GEMM of a 4096-sample training step, now 16 (between events).
+constexpr int GT = 128;      // threads
+constexpr int SLD = TM + 4;  // row stride of a shared slab (float4-aligned, 2-way conflicts at worst)
+enum { EPI_BIAS = 0, EPI_BIAS_RELU = 1, EPI_MASK = 2, EPI_LOSS = 3, EPI_PART = 4 };
+
+struct GemmArgs {
+    const float *A, *B;
+    int lda, ldb, M, N, K;
+    const float *bias;  // EPI_BIAS, EPI_BIAS_RELU, EPI_LOSS
+    const float *mask;  // EPI_MASK: times (mask > 0)
+    float *out;         // [M][N]; EPI_LOSS: the gradient of the loss; EPI_PART: this block's part
+    // EPI_LOSS: target (clean - noisy) / (sigma * rsqrt_k), loss parts per block
+    const float *noisy, *clean, *sigma;
+    float rsqrt_k, total;
+    double *lpart;
+    float *bsum;  // EPI_PART: the part's bias gradients (sums of A over k), written by the blocks with n0 = 0
+};
+
+template <bool KC>
+__device__ __forceinline__ void load_slab(const float *__restrict__ P, int ld, int r0, int R, int k0, int k1, int tid,
+                                          float4 (&v)[2]) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int e = tid + i * GT;
+        const int r = r0 + (KC ? e >> 2 : (e & 15) * 4), k = k0 + (KC ? (e & 3) * 4 : e >> 4);
+        const bool in = r < R && k < k1;
+        v[i] = in ? *reinterpret_cast<const float4 *>(P + (KC ? (size_t)r * ld + k : (size_t)k * ld + r))
+                  : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+}
+
+template <bool KC>
+__device__ __forceinline__ void store_slab(float (&S)[TK][SLD], int tid, const float4 (&v)[2]) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int e = tid + i * GT;
+        if (KC) {
+            const int r = e >> 2, k = (e & 3) * 4;
+            S[k][r] = v[i].x;
+            S[k + 1][r] = v[i].y;
+            S[k + 2][r] = v[i].z;
+            S[k + 3][r] = v[i].w;
+        } else {
+            *reinterpret_cast<float4 *>(&S[e >> 4][(e & 15) * 4]) = v[i];
+        }
+    }
+}
+
+template <bool AK, bool BK, int EPI>
+__device__ __forceinline__ void gemm_tile(const GemmArgs &g, int m0, int n0, int k0, int k1, int lblock) {
+    __shared__ __align__(16) float sA[2][TK][SLD], sB[2][TK][SLD];
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
-    const int k0 = blockIdx.z * kchunk, k1 = min(K, k0 + kchunk);
-    float acc[4][4] = {};
+    float acc[8][4] = {}, bs[8] = {};
+    float4 va[2], vb[2];
+    load_slab<AK>(g.A, g.lda, m0, g.M, k0, k1, tid, va);
+    load_slab<BK>(g.B, g.ldb, n0, g.N, k0, k1, tid, vb);
+    store_slab<AK>(sA[0], tid, va);
+    store_slab<BK>(sB[0], tid, vb);
+    __syncthreads();
+    int cur = 0;
     for (int kb = k0; kb < k1; kb += TK) {
-        for (int e = tid; e < TK * TM; e += 256) {
-            const int kk = e / TM, mm = e - kk * TM;  // consecutive threads: consecutive m
-            const int gm = m0 + mm, gk = kb + kk;
-            sA[kk][mm] = (gm < M && gk < k1) ? A[(long)gm * am + (long)gk * ak] : 0.f;
+        const bool more = kb + TK < k1;
+        if (more) {
+            load_slab<AK>(g.A, g.lda, m0, g.M, kb + TK, k1, tid, va);
+            load_slab<BK>(g.B, g.ldb, n0, g.N, kb + TK, k1, tid, vb);
         }
-        for (int e = tid; e < TK * TN; e += 256) {
-            const int kk = e / TN, nn = e - kk * TN;
-            const int gn = n0 + nn, gk = kb + kk;
-            sB[kk][nn] = (gn < N && gk < k1) ? B[(long)gn * bn + (long)gk * bk] : 0.f;
-        }
-        __syncthreads();
 #pragma unroll
         for (int kk = 0; kk < TK; ++kk) {
-            float a[4], b[4];
+            float a[8], b[4];
+            *reinterpret_cast<float4 *>(a) = *reinterpret_cast<const float4 *>(&sA[cur][kk][ty * 8]);
+            *reinterpret_cast<float4 *>(a + 4) = *reinterpret_cast<const float4 *>(&sA[cur][kk][ty * 8 + 4]);
+            *reinterpret_cast<float4 *>(b) = *reinterpret_cast<const float4 *>(&sB[cur][kk][tx * 4]);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                a[i] = sA[kk][ty * 4 + i];
-                b[i] = sB[kk][tx * 4 + i];
-            }
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < 8; ++i)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
+            if (EPI == EPI_PART && n0 == 0) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int gm = m0 + ty * 4 + i;
-        if (gm >= M) continue;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int gn = n0 + tx * 4 + j;
-            if (gn >= N) continue;
-            if (parts) {
-                parts[((long)blockIdx.z * M + gm) * N + gn] = acc[i][j];
-            } else {
-                float r = acc[i][j] + (bias ? bias[gn] : 0.f);
-                if (act == 1) r = fmaxf(r, 0.f);
-                if (act == 2) r = mask[(long)gm * ldc + gn] > 0.f ? r : 0.f;
-                Cout[(long)gm * ldc + gn] = r;
+                for (int i = 0; i < 8; ++i) bs[i] += a[i];
             }
         }
+        if (more) {  // the other buffer: its last readers passed the barrier of the previous slab
+            cur ^= 1;
+            store_slab<AK>(sA[cur], tid, va);
+            store_slab<BK>(sB[cur], tid, vb);
+            __syncthreads();
+        }
+    }
+    const int gn = n0 + tx * 4;
+    float4 bias = make_float4(0.f, 0.f, 0.f, 0.f);
+    if ((EPI == EPI_BIAS || EPI == EPI_BIAS_RELU || EPI == EPI_LOSS) && gn < g.N)
+        bias = *reinterpret_cast<const float4 *>(g.bias + gn);
+    // EPI_LOSS: sum of squared errors, a double-float (FP64 runs at a 64th of the rate), and in FP64 what FP32
+    // squares could not hold
+    float ls = 0.f, lc = 0.f;
+    double ld = 0.0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int gm = m0 + ty * 8 + i;
+        if (gm >= g.M || gn >= g.N) continue;
+        const size_t o = (size_t)gm * g.N + gn;
+        float r[4] = {acc[i][0], acc[i][1], acc[i][2], acc[i][3]};
+        if (EPI == EPI_BIAS || EPI == EPI_BIAS_RELU || EPI == EPI_LOSS) {
+            r[0] += bias.x;
+            r[1] += bias.y;
+            r[2] += bias.z;
+            r[3] += bias.w;
+        }
+        if (EPI == EPI_BIAS_RELU) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) r[j] = fmaxf(r[j], 0.f);
+        }
+        if (EPI == EPI_MASK) {
+            const float4 mk = *reinterpret_cast<const float4 *>(g.mask + o);
+            r[0] = mk.x > 0.f ? r[0] : 0.f;
+            r[1] = mk.y > 0.f ? r[1] : 0.f;
+            r[2] = mk.z > 0.f ? r[2] : 0.f;
+            r[3] = mk.w > 0.f ? r[3] : 0.f;
+        }
+        if (EPI == EPI_LOSS) {  // the caller's tensors: 4-byte alignment only
+            const float unit = g.sigma[gm] * g.rsqrt_k;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float e = r[j] - (g.clean[o + j] - g.noisy[o + j]) / unit;
+                r[j] = 2.f * e / g.total;
+                if (fabsf(e) > 1e-12f && fabsf(e) < 1e12f) {
+                    const float p = __fmul_rn(e, e), pe = __fmaf_rn(e, e, -p);  // e^2 = p + pe exactly
+                    const float s = __fadd_rn(ls, p), t = __fsub_rn(s, ls);
+                    lc = __fadd_rn(lc, __fadd_rn(__fadd_rn(__fsub_rn(ls, __fsub_rn(s, t)), __fsub_rn(p, t)), pe));
+                    ls = s;
+                } else {
+                    ld += (double)e * e;
+                }
+            }
+        }
+        *reinterpret_cast<float4 *>(g.out + o) = make_float4(r[0], r[1], r[2], r[3]);
+    }
+    if (EPI == EPI_PART && n0 == 0 && tx == 0) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (m0 + ty * 8 + i < g.M) g.bsum[m0 + ty * 8 + i] = bs[i];
+    }
+    if (EPI == EPI_LOSS) {
+        __shared__ double red[GT / 32];
+        double s = ((double)ls + (double)lc) + ld;
+#pragma unroll
+        for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if ((tid & 31) == 0) red[tid >> 5] = s;
+        __syncthreads();
+        if (tid == 0) g.lpart[lblock] = (red[0] + red[1]) + (red[2] + red[3]);
     }
 }
 
-// out[e] += sum over z of parts[z][e], in z order.
-__global__ void k_sum_parts(const float *__restrict__ parts, int nz, long ne, float *__restrict__ out) {
-    for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < ne; e += (long)gridDim.x * blockDim.x) {
-        float s = 0.f;
-        for (int z = 0; z < nz; ++z) s += parts[(long)z * ne + e];
-        out[e] += s;
-    }
+// blockIdx = (n tile, m tile)
+template <bool BK, int EPI>
+__global__ void __launch_bounds__(GT) k_gemm(const GemmArgs g) {
+    gemm_tile<true, BK, EPI>(g, blockIdx.y * TM, blockIdx.x * TN, 0, g.K, blockIdx.y * gridDim.x + blockIdx.x);
 }
 
-// db[o] += sum over n of dY[n][o], n in order.
-__global__ void k_bias_grad(const float *__restrict__ dY, int n, int o, float *__restrict__ db) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= o) return;
+// The weight and bias gradients of every layer in one launch: dW[m][n] = sum over the samples of dY[k][m] X[k][n],
+// db[m] = sum dY[k][m].  Block (t, z): tile t of the layers' tiles over samples [z kchunk, (z + 1) kchunk); its sums
+// go to part z, which has the layout of the parameter vector, so that one pass adds the parts in z order.  Three
+// launches of their own (and a bias kernel of one thread per column: 107 us each) left most SMs idle.
+struct WgradArgs {
+    GemmArgs l[NL];  // A = dY, B = the layer's input, out / bsum: the layer's place in part 0
+    int tile0[NL + 1], nt[NL];
+    int kchunk, nparams;
+};
+__global__ void __launch_bounds__(GT) k_wgrad(const __grid_constant__ WgradArgs w) {
+    int l = 0;
+    while ((int)blockIdx.x >= w.tile0[l + 1]) ++l;
+    const int t = blockIdx.x - w.tile0[l];
+    GemmArgs g = w.l[l];
+    g.out += (size_t)blockIdx.y * w.nparams;
+    g.bsum += (size_t)blockIdx.y * w.nparams;
+    const int k0 = blockIdx.y * w.kchunk;
+    gemm_tile<false, false, EPI_PART>(g, (t / w.nt[l]) * TM, (t % w.nt[l]) * TN, k0, min(g.K, k0 + w.kchunk), 0);
+}
+
+// grad[e] += sum over z of parts[z][e], in z order; the last block adds the loss parts (a fixed order: 32 strided
+// chains, then a tree).
+__global__ void __launch_bounds__(256) k_sum_parts(const float *__restrict__ parts, int nz, int ne,
+                                                   float *__restrict__ grad, const double *__restrict__ lpart, int nl,
+                                                   double total, double *loss) {
+    if (blockIdx.x == gridDim.x - 1) {
+        if (threadIdx.x < 32) {
+            double t = 0.0;
+            for (int b = threadIdx.x; b < nl; b += 32) t += lpart[b];
+#pragma unroll
+            for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (threadIdx.x == 0) *loss += t / total;
+        }
+        return;
+    }
+    const int e = blockIdx.x * 256 + threadIdx.x;
+    if (e >= ne) return;
     float s = 0.f;
-    for (int i = 0; i < n; ++i) s += dY[(long)i * o + j];
-    db[j] += s;
+#pragma unroll 8
+    for (int z = 0; z < nz; ++z) s += parts[(size_t)z * ne + e];
+    grad[e] += s;
 }
 
 // Mean patch of group r (channel t, pixel (u, v)) over its K members, members in order.
@@ -190,37 +322,6 @@ __global__ void k_features(const float *__restrict__ coords, const float *__rest
 
 // sigma of the call (double in the state) as a float for the features.
 __global__ void k_state_sigma(const DevState *st, float *out) { *out = (float)st->sigma_hat; }
-
-// Loss parts: block b sums (out - (clean - noisy) / s)^2 over its stride (s = sigma / sqrt(K) of the
-// sample, d values per sample); dout = 2 (out - target) / total.
-__global__ void __launch_bounds__(256) k_fcn_loss(const float *__restrict__ out, const float *__restrict__ noisy,
-                                                  const float *__restrict__ clean, const float *__restrict__ sigma,
-                                                  int d, float rsqrt_k, long total, float *__restrict__ dout,
-                                                  double *lpart) {
-    __shared__ double red[8];
-    double s = 0.0;
-    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
-        const float e = out[i] - (clean[i] - noisy[i]) / (sigma[i / d] * rsqrt_k);
-        dout[i] = 2.f * e / (float)total;
-        s += (double)e * e;
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < 8; ++w) t += red[w];
-        lpart[blockIdx.x] = t;
-    }
-}
-
-__global__ void k_loss_sum(const double *lpart, int nb, long total, double *loss) {
-    if (threadIdx.x != 0) return;
-    double t = 0.0;
-    for (int b = 0; b < nb; ++b) t += lpart[b];
-    *loss += t / (double)total;
-}
 
 __global__ void k_fcn_adam(float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
                            float *__restrict__ v, int n, float lr, float c1, float c2) {
@@ -393,8 +494,6 @@ __global__ void __launch_bounds__(64) k_coefs_to_patch(const float *__restrict__
     }
 }
 
-constexpr int LOSS_BLOCKS = 304;
-
 void layout(hts_fcn *f) {
     f->din = (f->C * 64 + 1 + 15) / 16 * 16;
     f->dout = f->C * 64;
@@ -416,16 +515,37 @@ hts_status ensure(hts_fcn *f, size_t n) {
             cudaFree(p);
             p = nullptr;
         }
-        cudaFree(f->d0);
-        cudaFree(f->d1);
-        f->X = f->d0 = f->d1 = nullptr;
+        f->X = nullptr;
         f->cap = 0;
         HTS_TRY(cu(dev_malloc(&f->X, n * f->din * sizeof(float)), "cudaMalloc(fcn)"));
         for (int l = 0; l < NL; ++l) HTS_TRY(cu(dev_malloc(&f->act[l], n * f->nout[l] * sizeof(float)), "cudaMalloc(fcn)"));
-        const size_t wd = std::max(HID, f->dout);
-        HTS_TRY(cu(dev_malloc(&f->d0, n * wd * sizeof(float)), "cudaMalloc(fcn)"));
-        HTS_TRY(cu(dev_malloc(&f->d1, n * wd * sizeof(float)), "cudaMalloc(fcn)"));
         f->cap = n;
+    }
+    return HTS_OK;
+}
+
+// The buffers only training needs, for n samples in `nz` parts.
+hts_status ensure_train(hts_fcn *f, size_t n, int nz) {
+    if (n > f->cap_train) {
+        for (float *&p : f->dy) {
+            cudaFree(p);
+            p = nullptr;
+        }
+        cudaFree(f->lpart);
+        f->lpart = nullptr;
+        f->cap_train = 0;
+        for (int l = 0; l < NL; ++l) HTS_TRY(cu(dev_malloc(&f->dy[l], n * f->nout[l] * sizeof(float)), "cudaMalloc(fcn)"));
+        const size_t blocks = ((n + TM - 1) / TM) * ((f->dout + TN - 1) / TN);
+        HTS_TRY(cu(dev_malloc(&f->lpart, blocks * sizeof(double)), "cudaMalloc(fcn)"));
+        f->cap_train = n;
+    }
+    const size_t need = (size_t)nz * f->nparams;
+    if (need > f->cap_part) {
+        cudaFree(f->part);
+        f->part = nullptr;
+        f->cap_part = 0;
+        HTS_TRY(cu(dev_malloc(&f->part, need * sizeof(float)), "cudaMalloc(fcn)"));
+        f->cap_part = need;
     }
     return HTS_OK;
 }
@@ -437,55 +557,58 @@ int nsm() {
     return n;
 }
 
-hts_status gemm(const float *A, long am, long ak, const float *B, long bn, long bk, int M, int N, int K,
-                const float *bias, int act, const float *mask, float *Cout, int ldc, cudaStream_t s) {
-    dim3 grid((N + TN - 1) / TN, (M + TM - 1) / TM, 1);
+template <bool BK, int EPI>
+hts_status gemm(const GemmArgs &g, cudaStream_t s) {
+    const dim3 grid((g.N + TN - 1) / TN, (g.M + TM - 1) / TM);
     {
         KTimer kt("k_fcn_gemm", s);
-        k_gemm<<<grid, 256, 0, s>>>(A, am, ak, B, bn, bk, M, N, K, K, bias, act, mask, Cout, ldc, nullptr);
+        k_gemm<BK, EPI><<<grid, GT, 0, s>>>(g);
     }
     return check_launch("k_fcn_gemm");
 }
 
-// out[M][N] += sum_k A(m, k) B(n, k) with the reduction split over blocks and summed in a fixed order.
-hts_status gemm_acc(hts_fcn *f, const float *A, long am, long ak, const float *B, long bn, long bk, int M, int N,
-                    int K, float *out, cudaStream_t s) {
-    const int tiles = ((N + TN - 1) / TN) * ((M + TM - 1) / TM);
-    int nz = std::max(1, std::min((2 * nsm() + tiles - 1) / tiles, (K + 255) / 256));
-    const int kchunk = ((K + nz - 1) / nz + TK - 1) / TK * TK;
-    nz = (K + kchunk - 1) / kchunk;
-    const size_t need = (size_t)nz * M * N;
-    if (need > f->cap_part) {
-        cudaFree(f->part);
-        f->part = nullptr;
-        f->cap_part = 0;
-        HTS_TRY(cu(dev_malloc(&f->part, need * sizeof(float)), "cudaMalloc(fcn)"));
-        f->cap_part = need;
-    }
-    dim3 grid((N + TN - 1) / TN, (M + TM - 1) / TM, nz);
-    {
-        KTimer kt("k_fcn_gemm", s);
-        k_gemm<<<grid, 256, 0, s>>>(A, am, ak, B, bn, bk, M, N, K, kchunk, nullptr, 0, nullptr, nullptr, 0, f->part);
-    }
-    HTS_TRY(check_launch("k_fcn_gemm"));
-    const long ne = (long)M * N;
-    {
-        KTimer kt("k_sum_parts", s);
-        k_sum_parts<<<(unsigned)std::min<long>((ne + 255) / 256, 1024), 256, 0, s>>>(f->part, nz, ne, out);
-    }
-    return check_launch("k_sum_parts");
-}
-
-// Forward of n samples whose features are in f->X; output in f->act[2].
-hts_status forward(hts_fcn *f, int n, cudaStream_t s) {
+// Forward of n samples whose features are in f->X; output in f->act[2], or, with a target (noisy, clean, sigma of
+// each), the loss gradient in f->dy[2] and the loss parts in f->lpart.
+hts_status forward(hts_fcn *f, int n, cudaStream_t s, const float *noisy = nullptr, const float *clean = nullptr,
+                   const float *sigma = nullptr) {
     const float *in = f->X;
     for (int l = 0; l < NL; ++l) {
-        HTS_TRY(gemm(in, f->nin[l], 1, f->w + f->off[l], f->nin[l], 1, n, f->nout[l], f->nin[l],
-                     f->w + f->off[l] + f->nout[l] * f->nin[l], l < NL - 1 ? 1 : 0, nullptr, f->act[l], f->nout[l],
-                     s));
+        GemmArgs g{};
+        g.A = in;
+        g.B = f->w + f->off[l];
+        g.lda = g.ldb = g.K = f->nin[l];
+        g.M = n;
+        g.N = f->nout[l];
+        g.bias = f->w + f->off[l] + f->nout[l] * f->nin[l];
+        g.out = f->act[l];
+        if (l < NL - 1) {
+            HTS_TRY((gemm<true, EPI_BIAS_RELU>(g, s)));
+        } else if (!noisy) {
+            HTS_TRY((gemm<true, EPI_BIAS>(g, s)));
+        } else {
+            g.out = f->dy[l];
+            g.noisy = noisy;
+            g.clean = clean;
+            g.sigma = sigma;
+            g.rsqrt_k = 1.f / std::sqrt((float)f->K);
+            g.total = (float)((long)n * f->dout);
+            g.lpart = f->lpart;
+            HTS_TRY((gemm<true, EPI_LOSS>(g, s)));
+        }
         in = f->act[l];
     }
     return HTS_OK;
+}
+
+// Tiles of layer l's weight gradient.
+int wgrad_tiles(const hts_fcn *f, int l) { return (f->nout[l] + TM - 1) / TM * ((f->nin[l] + TN - 1) / TN); }
+
+// Samples per part of the weight gradients: about four blocks per SM over all the layers' tiles, and at least 64.
+int wgrad_chunk(const hts_fcn *f, int n) {
+    long tiles = 0;
+    for (int l = 0; l < NL; ++l) tiles += wgrad_tiles(f, l);
+    const long c = ((long)n * tiles + 4 * nsm() - 1) / (4 * nsm());
+    return (int)((std::max(c, 64l) + TK - 1) / TK * TK);
 }
 
 hts_status features(hts_fcn *f, const float *means, const float *sigma, int sstride, int n, cudaStream_t s) {
@@ -507,8 +630,9 @@ hts_status upload(hts_fcn *f, const float *host) {
 
 void free_fcn(hts_fcn *f) {
     if (!f) return;
-    for (float *p : {f->w, f->grad, f->m, f->v, f->X, f->d0, f->d1, f->part}) cudaFree(p);
+    for (float *p : {f->w, f->grad, f->m, f->v, f->X, f->part}) cudaFree(p);
     for (float *p : f->act) cudaFree(p);
+    for (float *p : f->dy) cudaFree(p);
     cudaFree(f->loss);
     cudaFree(f->lpart);
     cudaFree(f->sig);
@@ -600,7 +724,6 @@ extern "C" hts_status hts_fcn_create(int C, int K, uint64_t seed, hts_fcn **out)
         if (st == HTS_OK) st = cu(dev_malloc(p, f->nparams * sizeof(float)), "cudaMalloc(fcn)");
     if (st == HTS_OK) st = cu(dev_malloc(&f->loss, sizeof(double)), "cudaMalloc(fcn)");
     if (st == HTS_OK) st = cu(cudaMemset(f->loss, 0, sizeof(double)), "cudaMemset");
-    if (st == HTS_OK) st = cu(dev_malloc(&f->lpart, LOSS_BLOCKS * sizeof(double)), "cudaMalloc(fcn)");
     if (st == HTS_OK) st = cu(dev_malloc(&f->sig, sizeof(float)), "cudaMalloc(fcn)");
     if (st != HTS_OK) {
         free_fcn(f);
@@ -689,32 +812,48 @@ extern "C" hts_status hts_fcn_accumulate_grad(hts_fcn *f, const float *noisy_mea
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     HTS_TRY(ensure(f, n));
     HTS_TRY(features(f, noisy_means, sigma, 1, n, s));
-    HTS_TRY(forward(f, n, s));
-    const long total = (long)n * f->dout;
+    const int kchunk = wgrad_chunk(f, n), nz = (n + kchunk - 1) / kchunk;
+    HTS_TRY(ensure_train(f, n, nz));
+    HTS_TRY(forward(f, n, s, noisy_means, clean_means, sigma));
+    // dX = (dY W) * (X > 0), the ReLU of the layer below
+    for (int l = NL - 1; l > 0; --l) {
+        GemmArgs g{};
+        g.A = f->dy[l];
+        g.B = f->w + f->off[l];
+        g.lda = g.K = f->nout[l];
+        g.ldb = g.N = f->nin[l];
+        g.M = n;
+        g.mask = f->act[l - 1];
+        g.out = f->dy[l - 1];
+        HTS_TRY((gemm<false, EPI_MASK>(g, s)));
+    }
+    WgradArgs w{};
+    w.kchunk = kchunk;
+    w.nparams = f->nparams;
+    for (int l = 0; l < NL; ++l) {
+        GemmArgs &g = w.l[l];
+        g.A = f->dy[l];
+        g.B = l == 0 ? f->X : f->act[l - 1];
+        g.lda = g.M = f->nout[l];
+        g.ldb = g.N = f->nin[l];
+        g.K = n;
+        g.out = f->part + f->off[l];
+        g.bsum = g.out + f->nout[l] * f->nin[l];
+        w.nt[l] = (f->nin[l] + TN - 1) / TN;
+        w.tile0[l + 1] = w.tile0[l] + wgrad_tiles(f, l);
+    }
     {
-        KTimer kt("k_fcn_loss", s);
-        k_fcn_loss<<<LOSS_BLOCKS, 256, 0, s>>>(f->act[NL - 1], noisy_means, clean_means, sigma, f->dout,
-                                               1.f / std::sqrt((float)f->K), total, f->d0, f->lpart);
-        k_loss_sum<<<1, 32, 0, s>>>(f->lpart, LOSS_BLOCKS, total, f->loss);
+        KTimer kt("k_fcn_wgrad", s);
+        k_wgrad<<<dim3(w.tile0[NL], nz), GT, 0, s>>>(w);
     }
-    HTS_TRY(check_launch("k_fcn_loss"));
-    // layer l: dY (n x nout) in dcur; dW += dY^T X_l, db += column sums, dX = (dY W) * (X_l > 0)
-    float *dcur = f->d0, *dnext = f->d1;
-    for (int l = NL - 1; l >= 0; --l) {
-        const float *xin = l == 0 ? f->X : f->act[l - 1];
-        const int ni = f->nin[l], no = f->nout[l];
-        HTS_TRY(gemm_acc(f, dcur, 1, no, xin, 1, ni, no, ni, n, f->grad + f->off[l], s));
-        {
-            KTimer kt("k_fcn_bias_grad", s);
-            k_bias_grad<<<(no + 127) / 128, 128, 0, s>>>(dcur, n, no, f->grad + f->off[l] + no * ni);
-        }
-        HTS_TRY(check_launch("k_fcn_bias_grad"));
-        if (l > 0) {
-            HTS_TRY(gemm(dcur, no, 1, f->w + f->off[l], 1, ni, n, ni, no, nullptr, 2, xin, dnext, ni, s));
-            std::swap(dcur, dnext);
-        }
+    HTS_TRY(check_launch("k_fcn_wgrad"));
+    {
+        KTimer kt("k_sum_parts", s);
+        k_sum_parts<<<(f->nparams + 255) / 256 + 1, 256, 0, s>>>(
+            f->part, nz, f->nparams, f->grad, f->lpart, ((n + TM - 1) / TM) * ((f->dout + TN - 1) / TN),
+            (double)n * f->dout, f->loss);
     }
-    return HTS_OK;
+    return check_launch("k_sum_parts");
 }
 
 extern "C" hts_status hts_fcn_take_loss(hts_fcn *f, double *loss_sum, void *stream) {
