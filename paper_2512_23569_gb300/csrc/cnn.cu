@@ -27,7 +27,7 @@
 //                   patch centre, as row sums then column sums (fixed order).
 // k_learned_partial/final  the map against the eigenvalue estimate: geometric
 //                   mean of the ratio, and the decision to use it.
-// k_adam            Adam with bias correction; refreshes the FP16 copy.
+// k_adam            Adam with bias correction; refreshes the FP16 copies.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -192,19 +192,32 @@ __global__ void k_reduce_grad(const float *__restrict__ part, int ntiles, int ne
     }
 }
 
-// Loss over the reference patches (one block): mean of (out[centre] - target)^2 added to *loss;
-// dout[centre] = 2 (out - target) / N_ref (dout zeroed before).
-__global__ void __launch_bounds__(1024) k_loss(const float *__restrict__ outm, int H, int W, int step, int nx,
-                                               int nref, const float *__restrict__ target, float *__restrict__ dout,
-                                               double *loss) {
-    __shared__ double red[32];
+// Loss over the reference patches: mean of (out[centre] - target)^2 added to *loss; dout = 2 (out - target) / N_ref at
+// the patch centres, zero elsewhere.  Bound by its launch and one pass over the map: a block takes rows of the image,
+// so that the zeros and the gradient are one coalesced write (a block of 1024 threads over all patches
+// and its memset took two launches and 13 us on a 256 x 256 crop, this 10 between events).  The last block to finish adds the blocks' parts in
+// block order.
+__global__ void __launch_bounds__(256) k_loss(const float *__restrict__ outm, int H, int W, int step, int nx, int ny,
+                                              const float *__restrict__ target, float *__restrict__ dout,
+                                              double *lpart, double *loss) {
+    __shared__ double red[8];
+    __shared__ bool last;
+    const int nref = nx * ny;
     double s = 0.0;
-    for (int r = threadIdx.x; r < nref; r += blockDim.x) {
-        const int gy = r / nx, gx = r - gy * nx;
-        const size_t o = (size_t)(grid_pos(gy, H, step) + PS / 2) * W + grid_pos(gx, W, step) + PS / 2;
-        const float d = outm[o] - target[r];
-        dout[o] = 2.f * d / (float)nref;
-        s += (double)d * d;
+    for (int y = blockIdx.x; y < H; y += gridDim.x) {
+        const int py = y - PS / 2;
+        const bool row = py >= 0 && py <= H - PS && (py % step == 0 || py == H - PS);
+        const int gy = py == H - PS ? ny - 1 : py / step;
+        for (int x = threadIdx.x; x < W; x += blockDim.x) {
+            const int px = x - PS / 2;
+            float d = 0.f;
+            if (row && px >= 0 && px <= W - PS && (px % step == 0 || px == W - PS)) {
+                const float e = outm[(size_t)y * W + x] - target[gy * nx + (px == W - PS ? nx - 1 : px / step)];
+                d = 2.f * e / (float)nref;
+                s += (double)e * e;
+            }
+            dout[(size_t)y * W + x] = d;
+        }
     }
 #pragma unroll
     for (int off = 16; off; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
@@ -212,13 +225,40 @@ __global__ void __launch_bounds__(1024) k_loss(const float *__restrict__ outm, i
     __syncthreads();
     if (threadIdx.x == 0) {
         double t = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-        *loss += t / nref;
+        for (int w = 0; w < 8; ++w) t += red[w];
+        lpart[blockIdx.x] = t;
+        __threadfence();
+        last = atomicInc(reinterpret_cast<unsigned *>(lpart + LOSS_BLOCKS), gridDim.x - 1) == gridDim.x - 1;
     }
+    __syncthreads();
+    if (!last || threadIdx.x >= 32) return;
+    __threadfence();
+    double t = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += 32) t += *(volatile double *)(lpart + b);
+#pragma unroll
+    for (int off = 16; off; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+    if (threadIdx.x == 0) *loss += t / nref;
+}
+
+// Where parameter i goes in the tensor-core kernels' weights (hts_cnn::wpk): its layer's forward entry, and for the
+// layers with a backward pass the flipped, transposed one (out channel = the layer's input channel, tap 8 - t).
+struct PackMap {
+    int off[DEPTH + 1], cin[DEPTH], cout[DEPTH], pf[DEPTH], pb[DEPTH];
+};
+__device__ __forceinline__ void pack_weight(const PackMap &m, int i, __half v, __half *__restrict__ wpk) {
+    int l = 0;
+    while (i >= m.off[l + 1]) ++l;
+    const int j = i - m.off[l], per = m.cin[l] * 9;
+    if (j >= m.cout[l] * per) return;  // a bias
+    const int co = j / per, rem = j - co * per, ci = rem / 9, tap = rem - ci * 9;
+    const int g = l == 0 ? 2 : 4, n = l == DEPTH - 1 ? 16 : 32;
+    wpk[m.pf[l] + ((tap * g + (ci >> 3)) * n + co) * 8 + (ci & 7)] = v;
+    if (l > 0) wpk[m.pb[l] + (((8 - tap) * (l == DEPTH - 1 ? 2 : 4) + (co >> 3)) * 32 + ci) * 8 + (co & 7)] = v;
 }
 
 __global__ void k_adam(float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
-                       float *__restrict__ v, __half *__restrict__ w16, int n, float lr, float c1, float c2) {
+                       float *__restrict__ v, __half *__restrict__ w16, const __grid_constant__ PackMap pm,
+                       __half *__restrict__ wpk, int n, float lr, float c1, float c2) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const float gi = g[i];
         const float mi = ADAM_B1 * m[i] + (1.f - ADAM_B1) * gi;
@@ -228,12 +268,16 @@ __global__ void k_adam(float *__restrict__ p, const float *__restrict__ g, float
         const float pi = p[i] - lr * (mi * c1) / (sqrtf(vi * c2) + ADAM_EPS);
         p[i] = pi;
         w16[i] = __float2half_rn(pi);
+        pack_weight(pm, i, __float2half_rn(pi), wpk);
     }
 }
 
-__global__ void k_to_half(const float *__restrict__ p, __half *__restrict__ w16, int n) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+__global__ void k_to_half(const float *__restrict__ p, __half *__restrict__ w16, const __grid_constant__ PackMap pm,
+                          __half *__restrict__ wpk, int n) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         w16[i] = __float2half_rn(p[i]);
+        pack_weight(pm, i, __float2half_rn(p[i]), wpk);
+    }
 }
 
 // Window of a reference patch along one axis: [c - S/2, c - S/2 + S) cut to [0, n), c = centre.
@@ -316,14 +360,11 @@ __global__ void k_learned_final(int nref, double factor, DevState *st) {
 
 }  // namespace
 
-// The training loss over the reference patches and its gradient map (dout: H x W, zeroed here), for the
-// tensor-core training path (cnn_tc.cu).
-hts_status cnn_loss(const float *map, int H, int W, const Geom &g, const float *target, float *dout, double *loss,
+hts_status cnn_loss(hts_cnn *n, const float *map, int H, int W, const Geom &g, const float *target, float *dout,
                     cudaStream_t s) {
-    HTS_TRY(cu(cudaMemsetAsync(dout, 0, (size_t)H * W * sizeof(float), s), "cudaMemsetAsync"));
     {
         KTimer kt("k_loss", s);
-        k_loss<<<1, 1024, 0, s>>>(map, H, W, g.step, g.nx, g.nref, target, dout, loss);
+        k_loss<<<std::min(H, LOSS_BLOCKS), 256, 0, s>>>(map, H, W, g.step, g.nx, g.ny, target, dout, n->lpart, n->loss);
     }
     return check_launch("k_loss");
 }
@@ -440,6 +481,27 @@ void layout(hts_cnn *n) {
         o += n->cout[l] * n->cin[l] * 9 + n->cout[l];
     }
     n->nparams = o;
+    o = 0;
+    for (int l = 0; l < DEPTH; ++l) {
+        n->pf[l] = o;
+        o += 9 * (l == 0 ? 2 : 4) * (l == DEPTH - 1 ? 16 : 32) * 8;
+        n->pb[l] = o;
+        if (l > 0) o += 9 * (l == DEPTH - 1 ? 2 : 4) * 32 * 8;
+    }
+    n->npk = o;
+}
+
+PackMap pack_map(const hts_cnn *n) {
+    PackMap m;
+    for (int l = 0; l < DEPTH; ++l) {
+        m.off[l] = n->off[l];
+        m.cin[l] = n->cin[l];
+        m.cout[l] = n->cout[l];
+        m.pf[l] = n->pf[l];
+        m.pb[l] = n->pb[l];
+    }
+    m.off[DEPTH] = n->nparams;
+    return m;
 }
 
 hts_status upload(hts_cnn *n, const float *host) {
@@ -448,7 +510,7 @@ hts_status upload(hts_cnn *n, const float *host) {
     HTS_TRY(cu(cudaMemset(n->v, 0, n->nparams * sizeof(float)), "cudaMemset"));
     HTS_TRY(cu(cudaMemset(n->grad, 0, n->nparams * sizeof(float)), "cudaMemset"));
     n->t = 0;
-    k_to_half<<<(n->nparams + 255) / 256, 256>>>(n->master, n->w16, n->nparams);
+    k_to_half<<<(n->nparams + 255) / 256, 256>>>(n->master, n->w16, pack_map(n), n->wpk, n->nparams);
     count_launch();
     HTS_TRY(check_launch("k_to_half"));
     return cu(cudaDeviceSynchronize(), "cudaDeviceSynchronize");
@@ -461,6 +523,8 @@ void free_net(hts_cnn *n) {
     cudaFree(n->m);
     cudaFree(n->v);
     cudaFree(n->w16);
+    cudaFree(n->wpk);
+    cudaFree(n->lpart);
     for (int l = 0; l < DEPTH; ++l) cudaFree(n->act[l]);
     cudaFree(n->d0);
     cudaFree(n->d1);
@@ -472,8 +536,7 @@ void free_net(hts_cnn *n) {
     cudaFree(n->rows);
     cudaFree(n->err);
     for (int i = 0; i < 4; ++i) cudaFree(n->tr_act[i]);
-    for (int i = 0; i < 2; ++i) cudaFree(n->tr_dy[i]);
-    cudaFree(n->tr_wt);
+    for (int i = 0; i < 4; ++i) cudaFree(n->tr_dy[i]);
     cudaFree(n->tr_map);
     cudaFree(n->tr_d0);
     cudaFree(n->tr_part);
@@ -556,6 +619,10 @@ extern "C" hts_status hts_cnn_create(int C, uint64_t seed, hts_cnn **out) {
     for (float **p : {&n->master, &n->grad, &n->m, &n->v})
         if (st == HTS_OK) st = cu(dev_malloc(p, b), "cudaMalloc(cnn)");
     if (st == HTS_OK) st = cu(dev_malloc(&n->w16, n->nparams * sizeof(__half)), "cudaMalloc(cnn)");
+    if (st == HTS_OK) st = cu(dev_malloc(&n->wpk, n->npk * sizeof(__half)), "cudaMalloc(cnn)");
+    if (st == HTS_OK) st = cu(cudaMemset(n->wpk, 0, n->npk * sizeof(__half)), "cudaMemset");  // the padding channels
+    if (st == HTS_OK) st = cu(dev_malloc(&n->lpart, (LOSS_BLOCKS + 1) * sizeof(double)), "cudaMalloc(cnn)");
+    if (st == HTS_OK) st = cu(cudaMemset(n->lpart, 0, (LOSS_BLOCKS + 1) * sizeof(double)), "cudaMemset");
     if (st == HTS_OK) st = cu(dev_malloc(&n->loss, sizeof(double)), "cudaMalloc(cnn)");
     if (st == HTS_OK) st = cu(cudaMemset(n->loss, 0, sizeof(double)), "cudaMemset");
     if (st == HTS_OK) st = cu(dev_malloc(&n->err, sizeof(int)), "cudaMalloc(cnn)");
@@ -609,9 +676,7 @@ extern "C" hts_status hts_cnn_log_sigma_map(hts_cnn *net, const float *img, int 
     if (!map_out) return report(HTS_EINVAL, "NULL pointer");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     HTS_TRY(cnn_ensure_infer(net, H, W, 1));
-    HTS_TRY(cnn_forward_tc(net, img, H, W, s));
-    return cu(cudaMemcpyAsync(map_out, net->map, (size_t)H * W * sizeof(float), cudaMemcpyDeviceToDevice, s),
-              "cudaMemcpyAsync");
+    return cnn_forward_tc_into(net, img, H, W, net->h16[0], net->h16[1], map_out, s);
 }
 
 extern "C" hts_status hts_cnn_sigma_refs(hts_cnn *net, const float *img, int H, int W, const hts_params *p,
@@ -647,15 +712,8 @@ extern "C" hts_status hts_cnn_accumulate_grad(hts_cnn *net, const float *img, in
     if (net->train_tc) return cnn_grad_tc(net, img, H, W, g, target_log_sigma, s);
     HTS_TRY(ensure_ws(net, H, W));
     HTS_TRY(forward(net, img, H, W, s));
-    const size_t px = (size_t)H * W;
     // loss and its gradient map (in d0)
-    HTS_TRY(cu(cudaMemsetAsync(net->d0, 0, px * sizeof(float), s), "cudaMemsetAsync"));
-    {
-        KTimer kt("k_loss", s);
-        k_loss<<<1, 1024, 0, s>>>(net->act[DEPTH - 1], H, W, g.step, g.nx, g.nref, target_log_sigma, net->d0,
-                                  net->loss);
-    }
-    HTS_TRY(check_launch("k_loss"));
+    HTS_TRY(cnn_loss(net, net->act[DEPTH - 1], H, W, g, target_log_sigma, net->d0, s));
     // layer 4 (linear) back to layer 0; each bwd_data output is masked by the ReLU of its layer
     float *dcur = net->d0, *dnext = net->d1;
     HTS_TRY(bwd_weight<1>(net, DEPTH - 1, net->act[DEPTH - 2], 1.f, dcur, H, W, s));
@@ -695,7 +753,7 @@ extern "C" hts_status hts_cnn_adam_step(hts_cnn *net, float lr, void *stream) {
     {
         KTimer kt("k_adam", s);
         k_adam<<<(net->nparams + 255) / 256, 256, 0, s>>>(net->master, net->grad, net->m, net->v, net->w16,
-                                                          net->nparams, lr, c1, c2);
+                                                          pack_map(net), net->wpk, net->nparams, lr, c1, c2);
     }
     return check_launch("k_adam");
 }

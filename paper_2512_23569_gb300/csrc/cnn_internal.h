@@ -14,6 +14,11 @@ struct hts_cnn {
     int off[5] = {}, cin[5] = {}, cout[5] = {};  // per layer: parameter offset, input / output channels
     float *master = nullptr, *grad = nullptr, *m = nullptr, *v = nullptr;  // FP32 parameters, Adam state
     __half *w16 = nullptr;                                                  // FP16 copy used by the kernels
+    // the tensor-core kernels' weights, FP16, laid out as their shared memory holds them ([tap][plane][n][8], zero
+    // outside the layer's channels): layer l's at wpk + pf[l], and for l >= 1 the flipped, transposed ones of the
+    // backward pass at wpk + pb[l]; written with w16
+    __half *wpk = nullptr;
+    int pf[5] = {}, pb[5] = {}, npk = 0;
     size_t cap_px = 0;
     float *act[5] = {};                   // FP32 activations (planar CHW) of the training forward
     float *d0 = nullptr, *d1 = nullptr;   // gradient maps; d0 also holds the readout's row sums
@@ -25,11 +30,12 @@ struct hts_cnn {
     float *map = nullptr;   // its log-sigma map (H x W)
     float *rows = nullptr;  // row sums of the readout window (H x reference columns)
     int *err = nullptr;     // set by a tensor-core forward whose wait gave up (the map is then NaN)
-    // tensor-core training (cnn_tc.cu): per-layer FP16 activations, FP16 input gradients (ping-pong), the
-    // map and its loss gradient, per-block weight-gradient sums, the flipped weights of the backward passes
+    double *lpart = nullptr;  // the loss kernel's per-block parts (LOSS_BLOCKS), then its block counter
+    // tensor-core training (cnn_tc.cu): per-layer FP16 activations, the FP16 gradients of the hidden layers'
+    // outputs, the map and its loss gradient, per-block weight-gradient sums
     int train_tc = 1;  // 1: hts_cnn_accumulate_grad runs on the tensor cores (FP16); 0: the FP32 kernels
-    size_t tr_cap_px = 0, tr_cap_part = 0, tr_cap_wt = 0;
-    __half *tr_act[4] = {}, *tr_dy[2] = {}, *tr_wt = nullptr;
+    size_t tr_cap_px = 0, tr_cap_part = 0;
+    __half *tr_act[4] = {}, *tr_dy[4] = {};
     float *tr_map = nullptr, *tr_d0 = nullptr, *tr_part = nullptr;
 };
 
@@ -47,9 +53,10 @@ hts_status cnn_ensure_infer(hts_cnn *net, int H, int W, int nx);
 hts_status cnn_forward_tc_into(hts_cnn *net, const float *img, int H, int W, __half *h0, __half *h1, float *map,
                                cudaStream_t s);
 struct Geom;
-// Training loss (added to *loss) and its gradient map (dout, zeroed first) over the reference patches.
-hts_status cnn_loss(const float *map, int H, int W, const Geom &g, const float *target, float *dout, double *loss,
+// Training loss (added to net->loss) of the map over the reference patches and its gradient map (dout, every pixel).
+hts_status cnn_loss(hts_cnn *net, const float *map, int H, int W, const Geom &g, const float *target, float *dout,
                     cudaStream_t s);
+constexpr int LOSS_BLOCKS = 304;
 // One image's loss and gradient (added to net->grad) on the tensor cores: FP16 activations and input
 // gradients (loss scale 2^(floor(log2 N_ref) + 2)), FP32 accumulation of the weight gradients.
 hts_status cnn_grad_tc(hts_cnn *net, const float *img, int H, int W, const Geom &g, const float *target,

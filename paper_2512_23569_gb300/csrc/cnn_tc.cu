@@ -52,6 +52,17 @@ constexpr size_t MIN_SMEM = 80 * 1024;
 // (backward: the gradient of a layer's input, zero where the activation is zero).
 constexpr int EPI_RELU = 0, EPI_MAP = 1, EPI_MASK = 2;
 
+// The layer's weights B[tap][g][n][k] = w[n][8 g + k][tap], laid out so in global memory, and its biases, into shared
+// memory (gathering them from [n][ci][tap] took 2-byte loads with four divisions each: half of a small layer's time).
+template <int CING, int NOUT, int EPI>
+__device__ __forceinline__ void stage_weights(const __half *__restrict__ wp, const __half *__restrict__ wbias, int cout,
+                                              __half *sB, float *sBias, int tid) {
+    for (int e = tid; e < 9 * CING * NOUT; e += NTH)
+        reinterpret_cast<uint4 *>(sB)[e] = __ldg(reinterpret_cast<const uint4 *>(wp) + e);
+    if (EPI != EPI_MASK)
+        for (int n = tid; n < NOUT; n += NTH) sBias[n] = n < cout ? __half2float(wbias[n]) : 0.f;
+}
+
 // One tile row of the epilogue: thread m of lane quarter q holds output pixel (oy, ox); r: its NOUT
 // accumulator columns (read by the caller).
 template <int NOUT, int EPI>
@@ -103,8 +114,8 @@ struct ConvTcLayout {
 template <int CING, int NOUT, bool IN_F32, int EPI>
 __global__ void __launch_bounds__(NTH, 2)
     k_conv_tc(const float *__restrict__ img, int C, float in_scale, const __half *__restrict__ hin, int H, int W,
-              const __half *__restrict__ wt, int cin, int cout, __half *__restrict__ hout, float *__restrict__ map,
-              const __half *__restrict__ hmask, int *err) {
+              const __half *__restrict__ wp, const __half *__restrict__ wbias, int cout, __half *__restrict__ hout,
+              float *__restrict__ map, const __half *__restrict__ hmask, int *err) {
     using L = ConvTcLayout<CING, NOUT>;
     extern __shared__ __align__(1024) unsigned char smem[];
     uint4 *sA = reinterpret_cast<uint4 *>(smem);
@@ -114,14 +125,7 @@ __global__ void __launch_bounds__(NTH, 2)
     uint32_t *slot = reinterpret_cast<uint32_t *>(smem + L::slot_off);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-    // weights B[tap][g][n][k] = w[n][8 g + k][tap], zero outside the layer's channels
-    for (int e = tid; e < 9 * CING * NOUT * 8; e += NTH) {
-        const int k = e & 7, rest = e >> 3;
-        const int n = rest % NOUT, g = (rest / NOUT) % CING, tap = rest / (NOUT * CING);
-        const int ci = g * 8 + k;
-        sB[e] = (n < cout && ci < cin) ? wt[(n * cin + ci) * 9 + tap] : __float2half_rn(0.f);
-    }
-    for (int n = tid; n < NOUT; n += NTH) sBias[n] = n < cout ? __half2float(wt[cout * cin * 9 + n]) : 0.f;
+    stage_weights<CING, NOUT, EPI>(wp, wbias, cout, sB, sBias, tid);
     if (tid == 0) {
         tc::bar_init(bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;");
@@ -253,8 +257,9 @@ struct ConvTmaLayout {
 
 template <int NOUT, int EPI>
 __global__ void __launch_bounds__(NTH, 2)
-    k_conv_tma(const __grid_constant__ CUtensorMap tmap, int H, int W, const __half *__restrict__ wt, int cin, int cout,
-               __half *__restrict__ hout, float *__restrict__ map, const __half *__restrict__ hmask, int *err) {
+    k_conv_tma(const __grid_constant__ CUtensorMap tmap, int H, int W, const __half *__restrict__ wp,
+               const __half *__restrict__ wbias, int cout, __half *__restrict__ hout, float *__restrict__ map,
+               const __half *__restrict__ hmask, int *err) {
     using L = ConvTmaLayout<NOUT>;
     extern __shared__ __align__(1024) unsigned char smem[];
     __half *sB = reinterpret_cast<__half *>(smem + L::b_off);
@@ -264,13 +269,7 @@ __global__ void __launch_bounds__(NTH, 2)
     uint32_t *slot = reinterpret_cast<uint32_t *>(full + NBH + 1);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-    for (int e = tid; e < 9 * CING_H * NOUT * 8; e += NTH) {
-        const int k = e & 7, rest = e >> 3;
-        const int n = rest % NOUT, g = (rest / NOUT) % CING_H, tap = rest / (NOUT * CING_H);
-        const int ci = g * 8 + k;
-        sB[e] = (n < cout && ci < cin) ? wt[(n * cin + ci) * 9 + tap] : __float2half_rn(0.f);
-    }
-    for (int n = tid; n < NOUT; n += NTH) sBias[n] = n < cout ? __half2float(wt[cout * cin * 9 + n]) : 0.f;
+    stage_weights<CING_H, NOUT, EPI>(wp, wbias, cout, sB, sBias, tid);
     const int nsx = (W + SXH - 1) / SXH, nstrip = ((H + SY - 1) / SY) * nsx;
     if (tid == 0) {
         for (int k = 0; k <= NBH; ++k) tc::bar_init(&full[k], 1);
@@ -363,8 +362,10 @@ __global__ void __launch_bounds__(NTH, 2)
     if (warp == 0) tc::tmem_dealloc(tbase, L::tcols);
 }
 
-// The network's FP16 weights of layer l with its channel counts, as conv_tc / conv_tma take them.
-#define LW(n, l) (n)->w16 + (n)->off[l], (n)->cin[l], (n)->cout[l]
+// The network's weights of layer l, its biases and their number, as conv_tc / conv_tma take them.
+#define LW(n, l) (n)->wpk + (n)->pf[l], (n)->w16 + (n)->off[l] + (n)->cout[l] * (n)->cin[l] * 9, (n)->cout[l]
+// The flipped weights of a backward pass through layer l (no biases).
+#define LWB(n, l) (n)->wpk + (n)->pb[l], nullptr, 0
 
 // After a forward whose wait gave up: the whole map becomes NaN.
 __global__ void k_map_poison(float *map, size_t n, const int *err) {
@@ -373,9 +374,9 @@ __global__ void k_map_poison(float *map, size_t n, const int *err) {
         map[i] = __int_as_float(0x7fc00000);
 }
 
-// wt: FP16 weights [cout][cin][3][3] then cout biases (the network's, or the flipped ones of a backward pass).
+// wp: the layer's packed weights (the network's, or the flipped ones of a backward pass).
 template <int CING, int NOUT, bool IN_F32, int EPI>
-hts_status conv_tc(const hts_cnn *n, const __half *wt, int cin, int cout, const float *img, int C, float in_scale,
+hts_status conv_tc(const hts_cnn *n, const __half *wp, const __half *wbias, int cout, const float *img, int C, float in_scale,
                    const __half *hin, int H, int W, __half *hout, float *map, const __half *hmask, int nsm,
                    cudaStream_t s) {
     using L = ConvTcLayout<CING, NOUT>;
@@ -386,7 +387,7 @@ hts_status conv_tc(const hts_cnn *n, const __half *wt, int cin, int cout, const 
     const int grid = std::max(1, std::min(nstrip, 2 * nsm));
     {
         KTimer kt("k_conv_tc", s);
-        k_conv_tc<CING, NOUT, IN_F32, EPI><<<grid, NTH, L::total, s>>>(img, C, in_scale, hin, H, W, wt, cin, cout,
+        k_conv_tc<CING, NOUT, IN_F32, EPI><<<grid, NTH, L::total, s>>>(img, C, in_scale, hin, H, W, wp, wbias, cout,
                                                                       hout, map, hmask, n->err);
     }
     return check_launch("k_conv_tc");
@@ -395,7 +396,7 @@ hts_status conv_tc(const hts_cnn *n, const __half *wt, int cin, int cout, const 
 // A hidden layer with the TMA-staged input: the tensor map describes hin as [plane][y][x][8 halves], read
 // as 8-byte elements (3-D, innermost first: 2 W, H, 4 planes) with the box of one strip's staged input.
 template <int NOUT, int EPI>
-hts_status conv_tma(const hts_cnn *n, const __half *wt, int cin, int cout, const __half *hin, int H, int W,
+hts_status conv_tma(const hts_cnn *n, const __half *wp, const __half *wbias, int cout, const __half *hin, int H, int W,
                     __half *hout, float *map, const __half *hmask, int nsm, cudaStream_t s) {
     using L = ConvTmaLayout<NOUT>;
     const auto enc = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(tensor_map_encoder());
@@ -417,67 +418,74 @@ hts_status conv_tma(const hts_cnn *n, const __half *wt, int cin, int cout, const
     const int grid = std::max(1, std::min(nstrip, 2 * nsm));
     {
         KTimer kt("k_conv_tma", s);
-        k_conv_tma<NOUT, EPI><<<grid, NTH, L::total, s>>>(tmap, H, W, wt, cin, cout, hout, map, hmask, n->err);
+        k_conv_tma<NOUT, EPI><<<grid, NTH, L::total, s>>>(tmap, H, W, wp, wbias, cout, hout, map, hmask, n->err);
     }
     return check_launch("k_conv_tma");
 }
 
 // ------------------------------------------------------------------ training (backward) on the tensor cores
 
-// Weight and bias gradient of one 3x3 layer: dW[co][ci][ky][kx] = sum_p dY[co](p) X[ci](p + (ky - 1, kx - 1)),
-// db[co] = sum_p dY[co](p), a contraction over the pixels: D[(tap, ci)][co] = sum_p A[(tap, ci)][p] B[co][p]
-// with the pixels as the MMA's K.  A block takes strips of 8 x 64 pixels, stages X with a one-pixel halo and
-// dY as planes of 8 FP16 channels, and per strip row (64 pixels, four K steps) copies the 64 pixel vectors of
-// every (tap, plane) into a 1 KB group of a chunk buffer, so that the 8-row groups of A (8 channels of one
-// plane at one tap) lie 1 KB apart: A is MN-major (8 channels per 16-byte pixel vector), M = 128 rows = 16
-// groups per tile; one extra group holds ones (its rows give the bias gradient).  B is the staged dY row,
-// MN-major as well (core matrices of 8 pixels, planes 8 KB apart).  The block accumulates every strip it
-// takes in tensor memory and writes its sums once; k_wgrad_reduce adds the blocks' sums in block order.
+// Weight and bias gradients of every layer in one launch: per layer dW[co][ci][ky][kx] = sum_p dY[co](p) X[ci](p +
+// (ky - 1, kx - 1)), db[co] = sum_p dY[co](p), a contraction over the pixels (the MMA's K): D_kx[(ky, ci)][co] +=
+// A_kx[(ky, ci)][p] B[co][p].  A block takes strips of 8 x 64 pixels of one layer and stages X with a one-pixel halo
+// as [row][plane][column] vectors of 8 channels and dY as planes.  In that order the 8-row groups (ky, plane) of A at
+// a given kx lie one staged row piece (PX vectors) apart, so the descriptor of tap column kx, strip row r and 16
+// pixels is the staged region itself (MN-major, M = 128: three ky, the rest of the rows multiply whatever follows
+// and are not read back): no copy per tap, and every MMA of a strip issued at once.  An all-ones operand (its groups
+// overlapping in 512 bytes) gives the bias gradient.  B is the staged dY row, MN-major as well (core matrices of 8
+// pixels, planes 8 KB apart).  Every block accumulates its strips in tensor memory, rows then 16-pixel steps, and
+// writes its sums once; k_wgrad_reduce adds the blocks' sums in block order.
+// Bound by latency at the training crops' size (128 strips a layer): staging, about 4 us of MMAs whose 4 KB A
+// operands come from shared memory, the read-back.  Three blocks per SM and the five layers side by side hide them:
+// 256 x 256 x 3, between events, 33 us for the layers together (before, a launch per layer with a copy of every tap
+// and a wait per strip row: 96 us); the reduction in one coalesced launch: 27 us (before 116).
 constexpr int WSY = 8;            // strip rows
 constexpr int WPY = WSY + 2;      // staged X rows
-constexpr int WCH = SX;           // pixels per chunk (one strip row)
+constexpr int WCH = SX;           // strip columns
+constexpr int NWG = 5;            // layers
 
-template <int CINX, int NPLY>
-struct WgradLayout {
-    static constexpr int NG = 9 * CINX + 1;        // (tap, plane) groups and the ones group
-    static constexpr int NTILE = (NG + 15) / 16;   // M tiles of 16 groups
-    static constexpr int N = NPLY * 8;             // MMA N: the output channels
-    static constexpr int ROWS = 9 * CINX * 8 + 1;  // rows written per block: (tap, ci), then the bias row
-    static constexpr size_t x_bytes = (size_t)CINX * WPY * PX * 16;
-    static constexpr size_t y_off = (x_bytes + 1023) / 1024 * 1024;
-    static constexpr size_t y_plane = (size_t)WSY * WCH * 16;
-    static constexpr size_t i_off = y_off + (size_t)NPLY * y_plane;
-    static constexpr size_t bar_off = i_off + (size_t)NTILE * 16 * 1024;
-    static constexpr size_t used = bar_off + 32;
-    static constexpr size_t total = used > MIN_SMEM ? used : MIN_SMEM;
-    static constexpr uint32_t tcols = NTILE * N <= 32 ? 32 : NTILE * N <= 64 ? 64 : NTILE * N <= 128 ? 128 : 256;
+struct WgLayer {
+    const void *x, *y;  // X: FP16 planes [cinx][H][W][8], or the FP32 image (planar, C channels; times 1/255);
+                        // dY: FP16 planes [nply][H][W][8], or the FP32 gradient map (one channel; times y_scale)
+    int x_f32, y_f32, C, cinx, nply;
+    int rows;           // 72 cinx + 1: (tap, ci), then the bias row
+    int cin, cout;
+    size_t part;        // the layer's parts [block][rows][8 nply]
+    float *grad;
 };
+struct WgradArgs {
+    WgLayer l[NWG];     // in launch order
+    int H, W, nblk;     // blocks per layer
+    float y_scale;      // the loss scale dY carries (applied here when dY is the FP32 map)
+    float *part;
+    int *err;
+};
+struct WgradLayout {
+    static constexpr size_t x_bytes = (size_t)4 * WPY * PX * 16;
+    static constexpr size_t y_off = x_bytes, y_plane = (size_t)WSY * WCH * 16;
+    static constexpr size_t one_off = y_off + 4 * y_plane;
+    static constexpr size_t bar_off = one_off + 512;
+    static constexpr size_t total = bar_off + 16;
+    static constexpr uint32_t tcols = 128;  // three tap columns and the ones, 32 each
+};
+static_assert(WgradLayout::y_off % 128 == 0 && 3 * (WgradLayout::total + 1024) <= 228 * 1024, "three blocks per SM");
+// the last MMA's A operand (16 groups from strip row 7, tap column 2, the last 16 pixels) stays in the staged bytes
+static_assert(((WSY - 1 + 15) * PX + 2 + WCH) * 16 <= WgradLayout::one_off &&
+                  (((WSY - 1) * 4 + 15) * PX + 2 + WCH) * 16 <= WgradLayout::one_off, "A stays in bounds");
 
-// X_F32: X is the FP32 image (planar, C channels) times 1/255, else FP16 planes xin[CINX][H][W][8].
-// Y_F32: dY is the FP32 gradient map (one channel) times y_scale, else FP16 planes yin[NPLY][H][W][8].
-template <int CINX, int NPLY, bool X_F32, bool Y_F32>
-__global__ void __launch_bounds__(NTH, 1)
-    k_conv_wgrad(const float *__restrict__ img, int C, const __half *__restrict__ xin, const float *__restrict__ ymap,
-                 float y_scale, const __half *__restrict__ yin, int H, int W, float *__restrict__ part,
-                 int *err) {
-    using L = WgradLayout<CINX, NPLY>;
+__global__ void __launch_bounds__(NTH, 3) k_conv_wgrad(const __grid_constant__ WgradArgs a) {
+    using L = WgradLayout;
     extern __shared__ __align__(1024) unsigned char smem[];
     uint4 *sX = reinterpret_cast<uint4 *>(smem);
     uint4 *sY = reinterpret_cast<uint4 *>(smem + L::y_off);
-    uint4 *sI = reinterpret_cast<uint4 *>(smem + L::i_off);
+    uint4 *s1 = reinterpret_cast<uint4 *>(smem + L::one_off);
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem + L::bar_off);
-    uint32_t *slot = reinterpret_cast<uint32_t *>(bar + 2);
+    uint32_t *slot = reinterpret_cast<uint32_t *>(bar + 1);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const WgLayer &l = a.l[blockIdx.y];
+    const int H = a.H, W = a.W, cinx = l.cinx, nply = l.nply;
     const size_t HW = (size_t)H * W;
-    // chunk buffer: groups past the (tap, plane) ones: the ones group, then zeros
-    for (int e = tid; e < (L::NTILE * 16 - 9 * CINX) * WCH; e += NTH) {
-        const int gr = 9 * CINX + e / WCH;
-        const __half one = __float2half_rn(gr == 9 * CINX ? 1.f : 0.f);
-        const __half2 h2 = __halves2half2(one, one);
-        uint4 v;
-        v.x = v.y = v.z = v.w = *reinterpret_cast<const uint32_t *>(&h2);
-        sI[gr * WCH + (e % WCH)] = v;
-    }
+    if (tid < 32) s1[tid] = make_uint4(0x3C003C00u, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u);  // FP16 ones
     if (tid == 0) {
         tc::bar_init(bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;");
@@ -487,173 +495,168 @@ __global__ void __launch_bounds__(NTH, 1)
     __syncthreads();
     tc::fence_after();
     const uint32_t tbase = *slot;
-    const uint32_t idesc = tc::idesc_f16(128, L::N, false) | (1u << 15) | (1u << 16);  // A and B MN-major
+    const uint32_t idesc = tc::idesc_f16(128, 8 * nply, false) | (1u << 15) | (1u << 16);  // A and B MN-major
     const int nsx = (W + WCH - 1) / WCH, nstrip = ((H + WSY - 1) / WSY) * nsx;
     uint32_t phase = 0;
     bool first = true, failed = false;
-    for (int strip = blockIdx.x; strip < nstrip && !failed; strip += gridDim.x) {
+    for (int strip = blockIdx.x; strip < nstrip; strip += gridDim.x) {
         const int y0 = (strip / nsx) * WSY, x0 = (strip % nsx) * WCH;
         // ---- stage X (halo, zero outside the image) and dY (zero outside)
-        for (int e = tid; e < CINX * WPY * PX; e += NTH) {
-            const int gp = e / (WPY * PX), r = e - gp * (WPY * PX), py = r / PX, px = r - py * PX;
+        for (int e = tid; e < cinx * WPY * PX; e += NTH) {
+            const int rg = e / PX, px = e - rg * PX, py = rg / cinx, gp = rg - py * cinx;
             const int y = y0 - 1 + py, x = x0 - 1 + px;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (y >= 0 && y < H && x >= 0 && x < W) {
-                if (X_F32) {
-                    __align__(16) __half h[8];
+            const bool in = y >= 0 && y < H && x >= 0 && x < W;
+            if (!l.x_f32) {
+                const uint4 *src = static_cast<const uint4 *>(l.x);
+                tc::cp_async16(sX + e, in ? src + ((size_t)gp * H + y) * W + x : src, in);
+            } else {
+                const float *img = static_cast<const float *>(l.x);
+                __align__(16) __half h[8];
 #pragma unroll
-                    for (int c = 0; c < 8; ++c)
-                        h[c] = __float2half_rn(c < C ? img[c * HW + (size_t)y * W + x] * (1.f / 255.f) : 0.f);
-                    v = *reinterpret_cast<const uint4 *>(h);
-                } else {
-                    v = reinterpret_cast<const uint4 *>(xin)[((size_t)gp * H + y) * W + x];
-                }
+                for (int c = 0; c < 8; ++c)
+                    h[c] = __float2half_rn(in && c < l.C ? img[c * HW + (size_t)y * W + x] * (1.f / 255.f) : 0.f);
+                sX[e] = *reinterpret_cast<const uint4 *>(h);
             }
-            sX[e] = v;
         }
-        for (int e = tid; e < NPLY * WSY * WCH; e += NTH) {
+        for (int e = tid; e < nply * WSY * WCH; e += NTH) {
             const int gp = e / (WSY * WCH), r = e - gp * (WSY * WCH), py = r / WCH, px = r - py * WCH;
             const int y = y0 + py, x = x0 + px;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (y < H && x < W) {
-                if (Y_F32) {
-                    if (gp == 0) {
-                        __align__(16) __half h[8];
-                        h[0] = __float2half_rn(ymap[(size_t)y * W + x] * y_scale);
-#pragma unroll
-                        for (int c = 1; c < 8; ++c) h[c] = __float2half_rn(0.f);
-                        v = *reinterpret_cast<const uint4 *>(h);
-                    }
-                } else {
-                    v = reinterpret_cast<const uint4 *>(yin)[((size_t)gp * H + y) * W + x];
-                }
-            }
-            sY[e] = v;
-        }
-        __syncthreads();
-        for (int r = 0; r < WSY; ++r) {
-            // ---- the chunk (strip row r): group (tap, plane) = the 64 staged X vectors of that tap's shift
-            for (int e = tid; e < 9 * CINX * WCH; e += NTH) {
-                const int gr = e / WCH, px = e - gr * WCH;
-                const int tap = gr / CINX, gp = gr - tap * CINX, ky = tap / 3, kx = tap - 3 * ky;
-                sI[gr * WCH + px] = sX[(gp * WPY + r + ky) * PX + px + kx];
-            }
-            tc::fence_async_smem();
-            __syncthreads();
-            if (tid == 0) {
-                tc::fence_after();
-                const uint32_t a0 = tc::su32(sI), b0 = tc::su32(sY) + (uint32_t)(r * WCH * 16);
-#pragma unroll
-                for (int t = 0; t < L::NTILE; ++t)
-#pragma unroll
-                    for (int kk = 0; kk < WCH / 16; ++kk) {
-                        const uint64_t ad = tc::sdesc(a0 + t * 16 * 1024 + kk * 256, 128, 1024);
-                        const uint64_t bd = tc::sdesc(b0 + kk * 256, 128, (uint32_t)L::y_plane);
-                        tc::mma_f16(tbase + t * L::N, ad, bd, idesc, (first && kk == 0) ? 0u : 1u);
-                    }
-                tc::mma_commit(bar);
-            }
-            const bool done = tc::bar_wait(bar, phase, SPIN);
-            if (__syncthreads_or(!done)) {
-                if (tid == 0) {
-                    tc::bar_wait(bar, phase, SPIN);  // the MMAs must end before the memory is released
-                    atomicExch(err, 1);
-                }
-                failed = true;
-                break;
-            }
-            phase ^= 1u;
-            tc::fence_after();
-            first = false;
-        }
-    }
-    // ---- the block's sums: row (tap, ci) or the bias row, N output channels
-    if (!failed && !first) {
-        const int q = warp & 3;
-        for (int t = warp >> 2; t < L::NTILE; t += NTH / 128) {
-            const int row = t * 128 + 32 * q + lane, gr = row >> 3, ch = row & 7;
-            uint32_t v[32];
-            const uint32_t taddr = tbase + ((uint32_t)(32 * q) << 16) + (uint32_t)(t * L::N);
-            if constexpr (L::N == 32) {
-                tc::tmem_ld32(taddr, v);
+            const bool in = y < H && x < W;
+            if (!l.y_f32) {
+                const uint4 *src = static_cast<const uint4 *>(l.y);
+                tc::cp_async16(sY + e, in ? src + ((size_t)gp * H + y) * W + x : src, in);
             } else {
-                tc::tmem_ld16(taddr, *reinterpret_cast<uint32_t(*)[16]>(v));
+                uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                if (in && gp == 0)
+                    v.x = __half_as_ushort(
+                        __float2half_rn(static_cast<const float *>(l.y)[(size_t)y * W + x] * a.y_scale));
+                sY[e] = v;
             }
+        }
+        tc::cp_async_wait();
+        tc::fence_async_smem();
+        __syncthreads();
+        if (tid == 0) {
+            tc::fence_after();
+            const uint32_t xa = tc::su32(sX), ya = tc::su32(sY);
+            const uint64_t od = tc::sdesc(tc::su32(s1), 128, 16);
+            for (int r = 0; r < WSY; ++r)
+#pragma unroll
+                for (int kk = 0; kk < WCH / 16; ++kk) {
+                    const uint64_t bd = tc::sdesc(ya + (uint32_t)(r * WCH + kk * 16) * 16, 128, (uint32_t)L::y_plane);
+                    const uint32_t acc = (first && r == 0 && kk == 0) ? 0u : 1u;
+#pragma unroll
+                    for (int kx = 0; kx < 3; ++kx)
+                        tc::mma_f16(tbase + kx * 32,
+                                    tc::sdesc(xa + (uint32_t)(r * cinx * PX + kx + kk * 16) * 16, 128, PX * 16), bd,
+                                    idesc, acc);
+                    tc::mma_f16(tbase + 96, od, bd, idesc, acc);
+                }
+            tc::mma_commit(bar);
+        }
+        const bool done = tc::bar_wait(bar, phase, SPIN);
+        if (__syncthreads_or(!done)) {
+            if (tid == 0) {
+                tc::bar_wait(bar, phase, SPIN);  // the MMAs must end before the memory is released
+                atomicExch(a.err, 1);
+            }
+            failed = true;
+            break;
+        }
+        phase ^= 1u;
+        tc::fence_after();
+        first = false;
+    }
+    // ---- the block's sums: row (tap, ci) or the bias row, 8 nply output channels
+    if (!failed) {
+        const int q = warp & 3, row = 32 * q + lane, gr = row >> 3, ch = row & 7;
+        const int ky = gr / cinx, gp = gr - ky * cinx;
+        for (int t = warp >> 2; t < 4; t += NTH / 128) {
+            uint32_t v[32];
+            tc::tmem_ld32(tbase + ((uint32_t)(32 * q) << 16) + (uint32_t)(t * 32), v);
             tc::tmem_wait_ld();
             int orow = -1;
-            if (gr < 9 * CINX) orow = gr * 8 + ch;                  // (tap, plane, channel) = tap * 8 CINX + ci
-            else if (gr == 9 * CINX && ch == 0) orow = L::ROWS - 1;  // the bias
+            if (t < 3) {
+                if (ky < 3) orow = ((ky * 3 + t) * cinx + gp) * 8 + ch;  // (tap, ci)
+            } else if (row == 0) {
+                orow = l.rows - 1;  // the bias
+            }
             if (orow >= 0) {
-                float *dst = part + ((size_t)blockIdx.x * L::ROWS + orow) * L::N;
+                uint4 *dst = reinterpret_cast<uint4 *>(a.part + l.part + ((size_t)blockIdx.x * l.rows + orow) * 8 * nply);
 #pragma unroll
-                for (int n = 0; n < L::N; ++n) dst[n] = __uint_as_float(v[n]);
+                for (int n = 0; n < 8; ++n)
+                    if (n < 2 * nply) dst[n] = make_uint4(v[4 * n], v[4 * n + 1], v[4 * n + 2], v[4 * n + 3]);
             }
         }
-    } else if (!failed) {  // a block without strips adds zeros
-        for (int e = tid; e < L::ROWS * L::N; e += NTH) part[(size_t)blockIdx.x * L::ROWS * L::N + e] = 0.f;
     }
     tc::fence_before();
     __syncthreads();
     if (warp == 0) tc::tmem_dealloc(tbase, L::tcols);
 }
 
-// grad[e] += (sum over the blocks, in block order, of their sums) / scale for every parameter of the layer
-// (cout x cin x 9 weights, then cout biases); NaN everywhere after a wait that gave up.
-__global__ void k_wgrad_reduce(const float *__restrict__ part, int nblk, int rows, int N, int cin, int cout,
-                               int cin_pad, float inv_scale, const int *err, float *__restrict__ grad) {
-    const int ne = cout * cin * 9 + cout;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < ne; e += gridDim.x * blockDim.x) {
-        int row, co;
-        if (e < cout * cin * 9) {
-            co = e / (cin * 9);
-            const int rem = e - co * cin * 9, ci = rem / 9, tap = rem - ci * 9;
-            row = tap * cin_pad + ci;
-        } else {
-            co = e - cout * cin * 9;
-            row = rows - 1;
-        }
-        float s = 0.f;
-        for (int b = 0; b < nblk; ++b) s += part[((size_t)b * rows + row) * N + co];
-        grad[e] = *err ? __int_as_float(0x7fc00000) : grad[e] + s * inv_scale;
-    }
+// grad[e] += (sum over the blocks, in block order, of their sums) / y_scale for every parameter of every layer
+// (cout x cin x 9 weights, then cout biases); NaN everywhere after a wait that gave up.  A thread per element of a
+// part, so that the reads are coalesced (the writes, one in nblk, scatter).
+__global__ void __launch_bounds__(256) k_wgrad_reduce(const __grid_constant__ WgradArgs a) {
+    const WgLayer &l = a.l[blockIdx.y];
+    const int N = 8 * l.nply, j = blockIdx.x * 256 + threadIdx.x;
+    if (j >= l.rows * N) return;
+    const int row = j / N, co = j - row * N, cp = 8 * l.cinx, tap = row / cp, ci = row - tap * cp;
+    const bool bias = row == l.rows - 1;
+    if (co >= l.cout || (!bias && ci >= l.cin)) return;
+    const float *p = a.part + l.part + j;
+    const size_t stride = (size_t)l.rows * N;
+    float s = 0.f;
+#pragma unroll 16
+    for (int b = 0; b < a.nblk; ++b) s += p[b * stride];
+    float *g = l.grad + (bias ? l.cout * l.cin * 9 + co : (co * l.cin + ci) * 9 + tap);
+    *g = *a.err ? __int_as_float(0x7fc00000) : *g + s * (1.f / a.y_scale);
 }
 
-// The flipped, transposed weights of a backward pass through layer l: out channel n = the layer's input
-// channel, input channel c = its output channel, tap 8 - t; biases zero.
-__global__ void k_wflip(const __half *__restrict__ w, int cout, int cin, __half *__restrict__ wt) {
-    const int ne = cin * cout * 9;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < ne + cin; e += gridDim.x * blockDim.x) {
-        if (e >= ne) {
-            wt[e] = __float2half_rn(0.f);
-            continue;
-        }
-        const int n = e / (cout * 9), rem = e - n * cout * 9, c = rem / 9, tap = rem - c * 9;
-        wt[e] = w[(c * cin + n) * 9 + (8 - tap)];
-    }
-}
+// Rows of a block's sums over all the layers, times their output channels.
+constexpr size_t WG_PART = (size_t)(72 + 1) * 32 + 3 * (size_t)(72 * 4 + 1) * 32 + (size_t)(72 * 4 + 1) * 16;
 
-// y_scale: the loss scale dY carries (applied here when dY is the FP32 map, by the caller otherwise); the
-// reduction divides it out.
-template <int CINX, int NPLY, bool X_F32, bool Y_F32>
-hts_status conv_wgrad(hts_cnn *n, int l, const float *img, const __half *xin, const float *ymap, float y_scale,
-                      const __half *yin, int H, int W, int nsm, cudaStream_t s) {
-    using L = WgradLayout<CINX, NPLY>;
-    const void *k = reinterpret_cast<const void *>(k_conv_wgrad<CINX, NPLY, X_F32, Y_F32>);
-    hts_status st = allow_smem(k, L::total);
+// Every layer's gradients: x[l] the layer's input (the image for layer 0), dy[l] the gradient of its output.
+hts_status conv_wgrad(hts_cnn *n, const float *img, __half *const *act, const float *d4, __half *const *dy,
+                      float y_scale, int H, int W, int nsm, cudaStream_t s) {
+    WgradArgs a{};
+    a.H = H;
+    a.W = W;
+    a.nblk = std::max(1, std::min(((H + WSY - 1) / WSY) * ((W + WCH - 1) / WCH), nsm));
+    a.y_scale = y_scale;
+    a.part = n->tr_part;
+    a.err = n->err;
+    size_t part = 0;
+    int most = 0;
+    for (int i = 0; i < NWG; ++i) {
+        const int l = (i + 1) % NWG;  // layer 0, the cheapest, last
+        WgLayer &w = a.l[i];
+        w.x = l == 0 ? static_cast<const void *>(img) : act[l - 1];
+        w.y = l == NWG - 1 ? static_cast<const void *>(d4) : dy[l];
+        w.x_f32 = l == 0;
+        w.y_f32 = l == NWG - 1;
+        w.C = n->C;
+        w.cinx = l == 0 ? 1 : 4;
+        w.nply = l == NWG - 1 ? 2 : 4;
+        w.rows = 72 * w.cinx + 1;
+        w.cin = n->cin[l];
+        w.cout = n->cout[l];
+        w.part = part;
+        w.grad = n->grad + n->off[l];
+        part += (size_t)a.nblk * w.rows * 8 * w.nply;
+        most = std::max(most, w.rows * 8 * w.nply);
+    }
+    hts_status st = allow_smem(reinterpret_cast<const void *>(k_conv_wgrad), WgradLayout::total);
     if (st != HTS_OK) return st;
-    const int nstrip = ((H + WSY - 1) / WSY) * ((W + WCH - 1) / WCH);
-    const int grid = std::max(1, std::min(nstrip, nsm));
     {
         KTimer kt("k_conv_wgrad", s);
-        k_conv_wgrad<CINX, NPLY, X_F32, Y_F32><<<grid, NTH, L::total, s>>>(img, n->C, xin, ymap, y_scale, yin, H, W,
-                                                                          n->tr_part, n->err);
+        k_conv_wgrad<<<dim3(a.nblk, NWG), NTH, WgradLayout::total, s>>>(a);
     }
     st = check_launch("k_conv_wgrad");
     if (st != HTS_OK) return st;
     {
         KTimer kt("k_wgrad_reduce", s);
-        k_wgrad_reduce<<<64, 256, 0, s>>>(n->tr_part, grid, L::ROWS, L::N, n->cin[l], n->cout[l], CINX * 8,
-                                          1.f / y_scale, n->err, n->grad + n->off[l]);
+        k_wgrad_reduce<<<dim3((most + 255) / 256, NWG), 256, 0, s>>>(a);
     }
     return check_launch("k_wgrad_reduce");
 }
@@ -719,10 +722,6 @@ hts_status cnn_forward_tc_into(hts_cnn *n, const float *img, int H, int W, __hal
 
 // ------------------------------------------------------------------ tensor-core training step
 
-namespace {
-constexpr int WG_ROWS_MAX = 9 * 4 * 8 + 1;
-}  // namespace
-
 hts_status cnn_train_ensure(hts_cnn *n, int H, int W, int nsm) {
     const size_t px = (size_t)H * W;
     if (px > n->tr_cap_px) {
@@ -730,7 +729,7 @@ hts_status cnn_train_ensure(hts_cnn *n, int H, int W, int nsm) {
             cudaFree(n->tr_act[i]);
             n->tr_act[i] = nullptr;
         }
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < 4; ++i) {
             cudaFree(n->tr_dy[i]);
             n->tr_dy[i] = nullptr;
         }
@@ -743,7 +742,7 @@ hts_status cnn_train_ensure(hts_cnn *n, int H, int W, int nsm) {
             cap = 0;
             if (grow_buf(n->tr_act[i], cap, px * 32) != HTS_OK) return HTS_ENOMEM;
         }
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < 4; ++i) {
             cap = 0;
             if (grow_buf(n->tr_dy[i], cap, px * 32) != HTS_OK) return HTS_ENOMEM;
         }
@@ -753,17 +752,15 @@ hts_status cnn_train_ensure(hts_cnn *n, int H, int W, int nsm) {
         if (grow_buf(n->tr_d0, cap, px) != HTS_OK) return HTS_ENOMEM;
         n->tr_cap_px = px;
     }
-    hts_status st = grow_buf(n->tr_part, n->tr_cap_part, (size_t)nsm * WG_ROWS_MAX * 32);
-    if (st != HTS_OK) return st;
-    return grow_buf(n->tr_wt, n->tr_cap_wt, (size_t)n->nparams + 5 * 32);
+    return grow_buf(n->tr_part, n->tr_cap_part, (size_t)nsm * WG_PART);
 }
 
 // One image's loss and gradient on the tensor cores: the forward of cnn_forward_tc keeping every layer's
 // FP16 activations, the loss gradient map 2 (out - target) / N_ref times the loss scale 2^(floor(log2 N_ref)
-// + 2) (so (4, 8] times the error, well inside FP16's range) rounded to FP16, then per layer from the last:
-// the weight and bias gradients (k_conv_wgrad, FP32 accumulation, the scale divided out) and the gradient of
-// the layer input (the forward kernels with the flipped, transposed weights, times the ReLU mask of the
-// stored activation, FP16).
+// + 2) (so (4, 8] times the error, well inside FP16's range) rounded to FP16, then from the last layer down the
+// gradient of the layer input (the forward kernels with the flipped, transposed weights, times the ReLU mask of
+// the stored activation, FP16), and every layer's weight and bias gradients at once (k_conv_wgrad, FP32
+// accumulation, the scale divided out).
 hts_status cnn_grad_tc(hts_cnn *n, const float *img, int H, int W, const Geom &g, const float *target,
                        cudaStream_t s) {
     int dev = 0, nsm = 152;
@@ -782,34 +779,13 @@ hts_status cnn_grad_tc(hts_cnn *n, const float *img, int H, int W, const Geom &g
     for (int l = 1; l < 4 && st == HTS_OK; ++l)
         st = conv_tma<32, EPI_RELU>(n, LW(n, l), a[l - 1], H, W, a[l], nullptr, nullptr, nsm, s);
     if (st == HTS_OK) st = conv_tma<16, EPI_MAP>(n, LW(n, 4), a[3], H, W, nullptr, n->tr_map, nullptr, nsm, s);
-    if (st == HTS_OK) st = cnn_loss(n->tr_map, H, W, g, target, n->tr_d0, n->loss, s);
-    if (st != HTS_OK) return st;
-    // flipped weights of layers 1..4 (layer l's at n->off[l] + 32 l: its cin biases follow its weights)
-    for (int l = 1; l < 5; ++l) {
-        {
-            KTimer kt("k_wflip", s);
-            k_wflip<<<64, 256, 0, s>>>(n->w16 + n->off[l], n->cout[l], n->cin[l], n->tr_wt + n->off[l] + 32 * l);
-        }
-        st = check_launch("k_wflip");
-        if (st != HTS_OK) return st;
-    }
-    auto wf = [&](int l) { return n->tr_wt + n->off[l] + 32 * l; };
-    // layer 4 (linear): its gradients from the loss map, then the gradient of its input
-    st = conv_wgrad<4, 2, false, true>(n, 4, nullptr, a[3], n->tr_d0, S, nullptr, H, W, nsm, s);
+    if (st == HTS_OK) st = cnn_loss(n, n->tr_map, H, W, g, target, n->tr_d0, s);
+    __half **dy = n->tr_dy;
     if (st == HTS_OK)
-        st = conv_tc<2, 32, true, EPI_MASK>(n, wf(4), n->cout[4], n->cin[4], n->tr_d0, 1, S, nullptr, H, W,
-                                            n->tr_dy[0], nullptr, a[3], nsm, s);
-    int cur = 0;
-    for (int l = 3; l >= 1 && st == HTS_OK; --l) {
-        st = conv_wgrad<4, 4, false, false>(n, l, nullptr, a[l - 1], nullptr, S, n->tr_dy[cur], H, W, nsm, s);
-        if (st == HTS_OK)
-            st = conv_tma<32, EPI_MASK>(n, wf(l), n->cout[l], n->cin[l], n->tr_dy[cur], H, W, n->tr_dy[cur ^ 1],
-                                        nullptr, a[l - 1], nsm, s);
-        cur ^= 1;
-    }
-    if (st == HTS_OK)
-        st = conv_wgrad<1, 4, true, false>(n, 0, img, nullptr, nullptr, S, n->tr_dy[cur], H, W, nsm, s);
-    return st;
+        st = conv_tc<2, 32, true, EPI_MASK>(n, LWB(n, 4), n->tr_d0, 1, S, nullptr, H, W, dy[3], nullptr, a[3], nsm, s);
+    for (int l = 3; l >= 1 && st == HTS_OK; --l)
+        st = conv_tma<32, EPI_MASK>(n, LWB(n, l), dy[l], H, W, dy[l - 1], nullptr, a[l - 1], nsm, s);
+    return st == HTS_OK ? conv_wgrad(n, img, a, n->tr_d0, dy, S, H, W, nsm, s) : st;
 }
 
 }  // namespace hts
