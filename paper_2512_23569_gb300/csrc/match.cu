@@ -24,6 +24,8 @@
 // same operation order as the definition and ranked by (D, index).  When the
 // candidate set exceeds what a warp handles (flat, noiseless inputs with
 // massive ties), the reference goes to an exhaustive FP64 pass.
+#include <algorithm>
+
 #include "hts_internal.h"
 
 namespace hts {
@@ -160,6 +162,53 @@ __device__ int gcp_green_fast(const float *__restrict__ img, int W, size_t HW, i
     if (lhs > rhs * (1.f + 1e-5f) && lhs > 0.f) return 1;
     if (lhs < rhs * (1.f - 1e-5f)) return 0;
     return gcp_green(img, W, HW, y, x, gamma, lane);
+}
+
+// The group of one reference from the m >= K - 1 collected candidates (plist, any order): sorted; certified, or
+// re-ranked in FP64; written to out[1 ..].  One warp; psort and pd64 hold PMAX entries each.
+template <int K>
+__device__ void settle_group(const MatchArgs &a, const Bound &bd, const uint64_t *plist, uint64_t *psort, double *pd64,
+                             int m, int yr, int xr, int green, int lane, int32_t *out) {
+    const size_t HW = (size_t)a.H * a.W;
+    // rank sort of the collected keys (unique: the raster index is part of the key)
+    for (int e = lane; e < m; e += 32) {
+        const uint64_t key = plist[e];
+        int rank = 0;
+        for (int j = 0; j < m; ++j) rank += (plist[j] < key) ? 1 : 0;
+        psort[rank] = key;
+    }
+    __syncwarp();
+    bool ok = true;
+    for (int i = lane; i < K - 1; i += 32)
+        if (i + 1 < m) ok = ok && (bd.upper(key_dist(psort[i])) < bd.lower(key_dist(psort[i + 1])));
+    if (__all_sync(FULL, ok)) {
+        for (int i = lane; i < K - 1; i += 32) out[1 + i] = key_idx(psort[i]);
+        return;
+    }
+    // uncertain order: FP64 re-rank of every entry that may belong to the K-1 nearest
+    const float thr = bd.upper(key_dist(psort[K - 2]));
+    int mp = 0;
+    for (int i = 0; i < m; ++i) {
+        if (bd.lower(key_dist(psort[i])) > thr) break;
+        mp = i + 1;
+    }
+    for (int i = lane; i < mp; i += 32) {
+        const int id = key_idx(psort[i]);
+        pd64[i] = exact_dist(a.img, a.W, HW, a.C, green, yr, xr, id / a.W, id % a.W);
+    }
+    __syncwarp();
+    for (int i = lane; i < mp; i += 32) {
+        const double di = pd64[i];
+        const int ii = key_idx(psort[i]);
+        int rank = 0;
+        for (int j = 0; j < mp; ++j) {
+            const double dj = pd64[j];
+            const int ij = key_idx(psort[j]);
+            rank += (dj < di || (dj == di && ij < ii)) ? 1 : 0;
+        }
+        if (rank < K - 1) out[1 + rank] = ii;
+    }
+    if (lane == 0) atomicAdd(&a.st->match_reranked, 1);
 }
 
 template <int K>
@@ -319,45 +368,309 @@ __global__ void __launch_bounds__(MW * 32) k_match(MatchArgs a) {
         return;
     }
     __syncwarp();
-    // rank sort of the collected keys (unique: the raster index is part of the key)
-    for (int e = lane; e < m; e += 32) {
-        const uint64_t key = plist[e];
-        int rank = 0;
-        for (int j = 0; j < m; ++j) rank += (plist[j] < key) ? 1 : 0;
-        psort[rank] = key;
-    }
-    __syncwarp();
-    bool ok = true;
-    for (int i = lane; i < K - 1; i += 32)
-        if (i + 1 < m) ok = ok && (bd.upper(key_dist(psort[i])) < bd.lower(key_dist(psort[i + 1])));
-    if (__all_sync(FULL, ok)) {
-        for (int i = lane; i < K - 1; i += 32) out[1 + i] = key_idx(psort[i]);
-        return;
-    }
-    // uncertain order: FP64 re-rank of every entry that may belong to the K-1 nearest
-    const float thr = bd.upper(key_dist(psort[K - 2]));
-    int mp = 0;
-    for (int i = 0; i < m; ++i) {
-        if (bd.lower(key_dist(psort[i])) > thr) break;
-        mp = i + 1;
-    }
-    for (int i = lane; i < mp; i += 32) {
-        const int id = key_idx(psort[i]);
-        pd64[i] = exact_dist(a.img, a.W, HW, a.C, green, yr, xr, id / a.W, id % a.W);
-    }
-    __syncwarp();
-    for (int i = lane; i < mp; i += 32) {
-        const double di = pd64[i];
-        const int ii = key_idx(psort[i]);
-        int rank = 0;
-        for (int j = 0; j < mp; ++j) {
-            const double dj = pd64[j];
-            const int ij = key_idx(psort[j]);
-            rank += (dj < di || (dj == di && ij < ii)) ? 1 : 0;
+    settle_group<K>(a, bd, plist, psort, pd64, m, yr, xr, green, lane, out);
+}
+
+// ---- the default grid step (4): 4 x 4 cells shared by neighbouring references
+//
+// Two references 4 pixels apart share half their patches, and at one offset (dy, dx) the squared differences of the
+// shared pixels are the same numbers: with the plane cut into 4 x 4 cells on the reference grid, a reference's
+// distance at an offset is the sum of four cells' sums, and a cell's sum serves four references.  A block takes a
+// tile of up to 8 x nry references; a thread takes an offset row dy and four consecutive dx, walks the tile's cell
+// rows with the candidate row pieces sliding through registers (per cell and pixel row one 16-byte load of the
+// reference, broadcast, and one of the candidates, conflict-free, for 32 operations), adds horizontally adjacent
+// cells, keeps the row of these pairs in registers and adds the next one: about 43 operations a candidate where the
+// distance alone took 128.  A row of references' distances goes to shared memory, and each warp settles a reference:
+// a bound on the (K-1)-th distance from the two smallest of every lane (a sort of 32 values per list, no rounds of
+// warp minima), the candidates under it, then as k_match.  Bound by FP32 issue (about 2/3 of it the distances).
+// Tiles are cut where the grid is: the last row / column of references, where H - 8 / W - 8 is no multiple of 4, are
+// tiles of their own.
+// Error: a term passes 2 roundings (difference, squared), at most 16 of the cell's chain and 2 of the cells' sums,
+// 20 u together; Bound takes 32 u.
+constexpr int CX = 8;          // references per tile row
+constexpr int CT = 256;        // most threads: (2R + 1) * ceil((R4 + R + 1) / 4) <= 256, R4 = R rounded up to 4 (R <= 15)
+constexpr float CEPS = 32.f * U32;
+
+struct CellArgs {
+    MatchArgs m;
+    int R4, G;                 // dx = 4 g + t - R4, g < G
+    int nry;                   // reference rows per tile
+    int rx, ry;                // references on the regular grid per row / column
+    int ntx, nty;              // regular tiles
+    int ncp;                   // floats per reference of the distance rows
+    int rows, cols;            // staged region
+};
+
+// Ascending sort of one value per lane.
+__device__ __forceinline__ float warp_sort(float v, int lane) {
+#pragma unroll
+    for (int k = 2; k <= 32; k <<= 1)
+#pragma unroll
+        for (int j = k >> 1; j; j >>= 1) {
+            const float o = __shfl_xor_sync(FULL, v, j);
+            const bool up = (lane & k) == 0 || k == 32, low = (lane & j) == 0;
+            v = (up == low) ? fminf(v, o) : fmaxf(v, o);
         }
-        if (rank < K - 1) out[1 + rank] = ii;
+    return v;
+}
+
+template <int K>
+__global__ void __launch_bounds__(CT, 3) k_match_cells(const __grid_constant__ CellArgs c) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const MatchArgs &a = c.m;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
+    const int npl = a.C == 3 ? 2 : 1, rw = c.cols;
+    float *plane0 = reinterpret_cast<float *>(smem_raw);              // [npl][rows][cols]: gray or green, R + G + B
+    float *dbuf = plane0 + (size_t)npl * c.rows * rw;                 // [CX][ncp] distances of a row of references
+    uint64_t *plist = reinterpret_cast<uint64_t *>(dbuf + (size_t)CX * c.ncp) + warp * PMAX;
+    __shared__ unsigned s_tmax;
+    __shared__ unsigned s_use[2][8];  // per plane and reference row of the tile: the references that use it
+    // ---- the tile: references (gy0 + i, gx0 + j) at (ya + 4 i, xa + 4 j), i < ni, j < nj
+    const size_t HW = (size_t)a.H * a.W;
+    int b = blockIdx.x, gy0, gx0, ni, nj;
+    const int nreg = c.nty * c.ntx, nlc = a.nx > c.rx ? c.nty : 0, nlr = a.ny > c.ry ? c.ntx : 0;
+    if (b < nreg) {
+        gy0 = b / c.ntx * c.nry;
+        gx0 = b % c.ntx * CX;
+        ni = min(c.nry, c.ry - gy0);
+        nj = min(CX, c.rx - gx0);
+    } else if (b < nreg + nlc) {  // the last column, off the grid
+        gy0 = (b - nreg) * c.nry;
+        gx0 = c.rx;
+        ni = min(c.nry, c.ry - gy0);
+        nj = 1;
+    } else {  // the last row, off the grid, and its corner
+        gy0 = c.ry;
+        gx0 = b < nreg + nlc + nlr ? (b - nreg - nlc) * CX : c.rx;
+        ni = 1;
+        nj = b < nreg + nlc + nlr ? min(CX, c.rx - gx0) : 1;
     }
-    if (lane == 0) atomicAdd(&a.st->match_reranked, 1);
+    const int ya = grid_pos(gy0, a.H, 4), xa = grid_pos(gx0, a.W, 4);
+    const int y0 = ya - a.R, x0 = xa - c.R4;  // region origin (may lie outside the image: zeros)
+    if (tid == 0) s_tmax = 0u;
+    if (tid < 16) s_use[tid >> 3][tid & 7] = 0u;
+    for (int e = tid; e < CX * c.ncp; e += blockDim.x) dbuf[e] = __int_as_float(0x7f800000);  // the padding stays
+    __syncthreads();
+    float tmax = 0.f;
+    const int nrow = 4 * (ni + 1) + 2 * a.R;
+#pragma unroll 4
+    for (int e = tid; e < nrow * rw; e += blockDim.x) {
+        const int yy = e / rw, xx = e - yy * rw, y = y0 + yy, x = x0 + xx;
+        const bool in = y >= 0 && y < a.H && x >= 0 && x < a.W;
+        const size_t o = in ? (size_t)y * a.W + x : 0;
+        if (a.C == 1) {
+            plane0[e] = in ? __ldg(a.img + o) : 0.f;
+        } else {
+            const float r = __ldg(a.img + o), g = __ldg(a.img + HW + o), bl = __ldg(a.img + 2 * HW + o);
+            plane0[e] = in ? g : 0.f;
+            plane0[c.rows * rw + e] = in ? __fadd_rn(__fadd_rn(r, g), bl) : 0.f;
+            if (in) tmax = fmaxf(tmax, fabsf(r) + fabsf(g) + fabsf(bl));
+        }
+    }
+    tmax = warp_max_f(tmax);
+    if (lane == 0) atomicMax(&s_tmax, __float_as_uint(tmax));  // non-negative floats order as their bits
+    for (int q = warp; q < ni * nj; q += nw) {  // Eq. 9 flags
+        const int i = q / nj, j = q - i * nj;
+        const int green = a.C == 3 ? gcp_green_fast(a.img, a.W, HW, ya + 4 * i, xa + 4 * j, a.gamma, lane) : 1;
+        if (lane == 0) {
+            if (a.green) a.green[(size_t)(gy0 + i) * a.nx + gx0 + j] = (uint8_t)green;
+            atomicOr(&s_use[green ? 0 : 1][i], 1u << j);
+        }
+    }
+    __syncthreads();
+    const float T3 = __uint_as_float(s_tmax);
+    // ---- this thread's offsets: row ky (dy = ky - R), columns 4 g .. 4 g + 3
+    const int ky = tid / c.G, g = tid - ky * c.G;
+    const bool item = ky <= 2 * a.R;
+    unsigned vt = 0u;  // its offsets inside the window, without the reference itself
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        const int dx = 4 * g + t - c.R4;
+        if (item && dx >= -a.R && dx <= a.R && !(ky == a.R && dx == 0)) vt |= 1u << t;
+    }
+    const int wrow = 4 * c.G;
+    for (int pass = 0; pass < npl; ++pass) {
+        unsigned used = 0u;  // rows with a reference of this plane
+        for (int i = 0; i < ni; ++i) used |= s_use[pass][i] ? 1u << i : 0u;
+        if (!used) continue;
+        const float *pa = plane0 + (size_t)pass * c.rows * rw + a.R * rw + c.R4;
+        const float *pb = plane0 + (size_t)pass * c.rows * rw + (item ? ky * rw + 4 * g : 0);
+        Bound bd;
+        bd.eps = CEPS;
+        bd.beta = pass == 0 ? 0.f : 72.f * U32 * T3;
+        bd.g0 = (pass == 0 ? 0.f : 1200.f * U32 * U32 * T3 * T3) + 1e-30f;
+        float4 hp[CX];  // the previous cell row's horizontal pairs
+#pragma unroll
+        for (int j = 0; j < CX; ++j) hp[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int cr = 0; cr <= ni; ++cr) {
+            if (!(((used << 1) | used) >> cr & 1u)) continue;  // no reference of rows cr - 1, cr needs this cell row
+            const bool emit = cr > 0 && (used >> (cr - 1) & 1u);
+            const int cy = ya + 4 * (cr - 1) + ky - a.R;
+            const unsigned vr = (cy >= 0 && cy <= a.H - PS) ? vt : 0u;
+            if (item) {
+                const float *ra = pa + 4 * cr * rw, *rb = pb + 4 * cr * rw;
+                float4 bl[4], sp = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) bl[u] = *reinterpret_cast<const float4 *>(rb + u * rw);
+#pragma unroll
+                for (int k = 0; k <= CX; ++k) {
+                    if (k > nj) break;
+                    float s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const float4 av = *reinterpret_cast<const float4 *>(ra + u * rw + 4 * k);
+                        const float4 bh = *reinterpret_cast<const float4 *>(rb + u * rw + 4 * k + 4);
+                        const float aa[4] = {av.x, av.y, av.z, av.w};
+                        const float bb[8] = {bl[u].x, bl[u].y, bl[u].z, bl[u].w, bh.x, bh.y, bh.z, bh.w};
+#pragma unroll
+                        for (int v = 0; v < 4; ++v)
+#pragma unroll
+                            for (int t = 0; t < 4; ++t) {
+                                const float e = __fsub_rn(aa[v], bb[v + t]);
+                                s[t] = __fmaf_rn(e, e, s[t]);
+                            }
+                        bl[u] = bh;
+                    }
+                    if (k > 0) {
+                        const float4 h = make_float4(sp.x + s[0], sp.y + s[1], sp.z + s[2], sp.w + s[3]);
+                        if (emit) {
+                            const float inf = __int_as_float(0x7f800000);
+                            const int cx = xa + 4 * (k - 1) + 4 * g - c.R4;  // the candidates' columns
+                            const float4 p = hp[k - 1];
+                            float4 d;
+                            d.x = (vr & 1u) && cx >= 0 && cx <= a.W - PS ? p.x + h.x : inf;
+                            d.y = (vr & 2u) && cx + 1 >= 0 && cx + 1 <= a.W - PS ? p.y + h.y : inf;
+                            d.z = (vr & 4u) && cx + 2 >= 0 && cx + 2 <= a.W - PS ? p.z + h.z : inf;
+                            d.w = (vr & 8u) && cx + 3 >= 0 && cx + 3 <= a.W - PS ? p.w + h.w : inf;
+                            *reinterpret_cast<float4 *>(dbuf + (k - 1) * c.ncp + ky * wrow + 4 * g) = d;
+                        }
+                        hp[k - 1] = h;
+                    }
+                    sp = make_float4(s[0], s[1], s[2], s[3]);
+                }
+            }
+            if (!emit) continue;
+            __syncthreads();
+            // ---- the row's references of this plane, a warp each
+            const unsigned use = s_use[pass][cr - 1];
+            for (int j = warp; j < nj; j += nw) {
+                if (!(use >> j & 1u)) continue;
+                float *db = dbuf + j * c.ncp;
+                const int r = (gy0 + cr - 1) * a.nx + gx0 + j, yr = ya + 4 * (cr - 1), xr = xa + 4 * j;
+                int32_t *out = a.idx + (size_t)r * K;
+                if (lane == 0) out[0] = yr * a.W + xr;
+                const int nch = (wrow * (2 * a.R + 1) + 31) >> 5;
+                // entry i of this lane: 32 i + ((lane + 7 i) mod 32), so that neighbouring rows' equal dx differ in lane
+                float m1 = __int_as_float(0x7f800000), m2 = m1;
+#pragma unroll 8
+                for (int i = 0; i < nch; ++i) {
+                    const float v = db[32 * i + ((lane + 7 * i) & 31)];
+                    m2 = fminf(m2, fmaxf(m1, v));
+                    m1 = fminf(m1, v);
+                }
+                // the K-1 smallest of two ascending lists are min(A[i], B[K-2-i]): the largest of them bounds the
+                // (K-1)-th distance
+                const float A = warp_sort(m1, lane), B = warp_sort(m2, lane);
+                const float bo = __shfl_sync(FULL, B, lane < K - 1 ? K - 2 - lane : 0);
+                float tau = __uint_as_float(__reduce_max_sync(FULL, lane < K - 1 ? __float_as_uint(fminf(A, bo)) : 0u));
+                float T = bd.upper(bd.upper(tau));
+                unsigned hit = 0u;
+                int m = 0;
+                float lo = 0.f;
+                for (int it = 0;; ++it) {
+                    hit = 0u;
+#pragma unroll 8
+                    for (int i = 0; i < nch; ++i) hit |= (db[32 * i + ((lane + 7 * i) & 31)] <= T ? 1u : 0u) << i;
+                    m = __reduce_add_sync(FULL, __popc(hit));
+                    if (m <= PMAX || it >= 24 || !(T < 3e38f)) break;
+                    // too many: halve the bound as long as it keeps K - 1 candidates
+                    int n = 0;
+                    float mid;
+                    for (;; ++it) {
+                        mid = 0.5f * (lo + tau);
+                        n = 0;
+                        for (int i = 0; i < nch; ++i) n += db[32 * i + lane] <= mid ? 1 : 0;
+                        n = __reduce_add_sync(FULL, n);
+                        if (n >= K - 1 || it >= 24) break;
+                        lo = mid;
+                    }
+                    if (n < K - 1) break;
+                    tau = mid;
+                    T = bd.upper(bd.upper(tau));
+                }
+                if (m > PMAX || m < K - 1 || !(T < 3e38f)) {  // the exhaustive FP64 pass
+                    if (lane == 0) a.fb[atomicAdd(&a.st->match_fallback, 1)] = r;
+                    continue;
+                }
+                int pos = __popc(hit);
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int v = __shfl_up_sync(FULL, pos, o);
+                    if (lane >= o) pos += v;
+                }
+                pos -= __popc(hit);
+                for (; hit; hit &= hit - 1) {
+                    const int i = __ffs(hit) - 1, e = 32 * i + ((lane + 7 * i) & 31), ey = e / wrow;
+                    plist[pos++] = make_key(db[e], (yr + ey - a.R) * a.W + xr + (e - ey * wrow) - c.R4);
+                }
+                __syncwarp();
+                // the reference's distances are spent: their row holds the sorted keys and FP64 distances
+                settle_group<K>(a, bd, plist, reinterpret_cast<uint64_t *>(db), reinterpret_cast<double *>(db) + PMAX, m,
+                                yr, xr, pass == 0 ? 1 : 0, lane, out);
+                __syncwarp();
+                for (int e = wrow * (2 * a.R + 1) + lane; e < c.ncp; e += 32) db[e] = __int_as_float(0x7f800000);
+            }
+            __syncthreads();
+        }
+    }
+}
+
+// Offsets (threads) of the cell matcher's window.
+inline int cell_groups(int R, int *R4) {
+    *R4 = (R + 3) / 4 * 4;
+    return (*R4 + R + 4) / 4;
+}
+
+template <int K>
+hts_status launch_cells(const MatchArgs &a, cudaStream_t s) {
+    CellArgs c{};
+    c.m = a;
+    c.G = cell_groups(a.R, &c.R4);
+    const int items = (2 * a.R + 1) * c.G;
+    const int threads = std::max(64, (items + 31) / 32 * 32);
+    c.ry = (a.H - PS) / 4 + 1;
+    c.rx = (a.W - PS) / 4 + 1;
+    c.ntx = (c.rx + CX - 1) / CX;
+    c.ncp = std::max((items * 4 + 31) / 32 * 32, PMAX * 4);
+    c.cols = 4 * (CX + 1) + 4 * c.G;
+    auto smem_of = [&](int nry) {
+        return ((size_t)(a.C == 3 ? 2 : 1) * (4 * (nry + 1) + 2 * a.R) * c.cols + (size_t)CX * c.ncp) * sizeof(float) +
+               (size_t)(threads / 32) * PMAX * sizeof(uint64_t);
+    };
+    // rows per tile: more share cells (a tile of n rows sums n + 1 cell rows and settles n rows of references; about
+    // 11 and 5 thousand warp instructions, 6 to stage) but leave SMs idle on small images: the fewest waves' work
+    double best = 0.0;
+    for (int n : {8, 6, 4, 3, 2, 1}) {
+        const int slots = 152 * (int)std::max<size_t>(1, std::min<size_t>(2048 / threads, 233472 / (smem_of(n) + 1024)));
+        const long blocks = (long)c.ntx * ((c.ry + n - 1) / n);
+        const double w = (double)((blocks + slots - 1) / slots) * ((n + 1) * 11.0 + n * 5.0 + 6.0) *
+                         std::max(1.0, std::min<double>(blocks, slots) / 152.0);
+        if (best == 0.0 || w < best) {
+            best = w;
+            c.nry = n;
+        }
+    }
+    c.nty = (c.ry + c.nry - 1) / c.nry;
+    c.rows = 4 * (c.nry + 1) + 2 * a.R;
+    const int blocks = c.ntx * c.nty + (a.nx > c.rx ? c.nty : 0) + (a.ny > c.ry ? c.ntx : 0) +
+                       (a.nx > c.rx && a.ny > c.ry ? 1 : 0);
+    const hts_status st0 = allow_smem(reinterpret_cast<const void *>(k_match_cells<K>), smem_of(c.nry));
+    if (st0 != HTS_OK) return st0;
+    {
+        KTimer kt("k_match", s);
+        k_match_cells<K><<<blocks, threads, smem_of(c.nry), s>>>(c);
+    }
+    return check_launch("k_match");
 }
 
 // Exhaustive FP64 matching of the references listed by k_match.
@@ -548,8 +861,9 @@ __global__ void __launch_bounds__(128) k_match_rescue(MatchArgs a) {
     }
 }
 
+// The grid step the cells are cut for, and windows whose offsets fit a block; else a reference per warp.
 template <int K>
-hts_status launch_k(const MatchArgs &a, cudaStream_t s) {
+hts_status launch_direct(const MatchArgs &a, cudaStream_t s) {
     const int RHM = a.step + 2 * a.R + PS;
     const int NCM = (2 * a.R + 1) * (2 * a.R + 1);
     const size_t smem = (size_t)MW * 3 * PMAX * 8 + (size_t)(a.C == 3 ? 2 : 1) * RHM * RHM * sizeof(float) +
@@ -563,7 +877,14 @@ hts_status launch_k(const MatchArgs &a, cudaStream_t s) {
         KTimer kt("k_match", s);
         k_match<K><<<blocks, MW * 32, smem, s>>>(a);
     }
-    hts_status st = check_launch("k_match");
+    return check_launch("k_match");
+}
+
+template <int K>
+hts_status launch_k(const MatchArgs &a, cudaStream_t s) {
+    int R4;
+    const bool cells = a.step == 4 && (2 * a.R + 1) * cell_groups(a.R, &R4) <= CT;
+    const hts_status st = cells ? launch_cells<K>(a, s) : launch_direct<K>(a, s);
     if (st != HTS_OK) return st;
     {
         KTimer kt("k_match_fallback", s);
