@@ -1,5 +1,8 @@
 // Grouping step of Haar-tSVD (Eq. 9, Alg. 1 step 1) on sm_103a.
 //
+// At the default grid step k_match_cells (below) shares the squared differences
+// of neighbouring references; for other steps and windows above 31, k_match:
+//
 // A block of four warps takes a 2x2 block of reference patches and stages the
 // union of their search regions of the matching planes in shared memory
 // (gray image; for colour both the green channel and the channel sum R+G+B,
@@ -164,47 +167,88 @@ __device__ int gcp_green_fast(const float *__restrict__ img, int W, size_t HW, i
     return gcp_green(img, W, HW, y, x, gamma, lane);
 }
 
-// The group of one reference from the m >= K - 1 collected candidates (plist, any order): sorted; certified, or
-// re-ranked in FP64; written to out[1 ..].  One warp; psort and pd64 hold PMAX entries each.
+// A warp's collected candidates: FP32 distances and raster indices, and the same sorted; PMAX entries each.
+struct CandList {
+    float *d, *sd;  // 16-byte aligned
+    int *i, *si;
+    double *d64;
+    __device__ __forceinline__ CandList(void *list, void *scratch)
+        : d(static_cast<float *>(list)), sd(static_cast<float *>(scratch)), i(reinterpret_cast<int *>(d + PMAX)),
+          si(reinterpret_cast<int *>(sd + PMAX)), d64(reinterpret_cast<double *>(si + PMAX)) {}
+    static constexpr int LIST = PMAX * 8, SCRATCH = PMAX * 16;  // bytes
+};
+
+// The group of one reference from its m collected candidates (K - 1 <= m <= PMAX, any order): sorted and, where the
+// order is certain, written to out[1 ..] (returns 0); else the number of entries of c.si that may belong to the K-1
+// nearest, for rerank_group.  One warp.
 template <int K>
-__device__ void settle_group(const MatchArgs &a, const Bound &bd, const uint64_t *plist, uint64_t *psort, double *pd64,
-                             int m, int yr, int xr, int green, int lane, int32_t *out) {
-    const size_t HW = (size_t)a.H * a.W;
-    // rank sort of the collected keys (unique: the raster index is part of the key)
-    for (int e = lane; e < m; e += 32) {
-        const uint64_t key = plist[e];
-        int rank = 0;
-        for (int j = 0; j < m; ++j) rank += (plist[j] < key) ? 1 : 0;
-        psort[rank] = key;
+__device__ __forceinline__ int settle_group(const Bound &bd, const CandList &c, int m, int lane, int32_t *out) {
+    if (lane < 4 && m + lane < PMAX) c.d[m + lane] = __int_as_float(0x7f800000);  // up to a multiple of 4
+    __syncwarp();
+    // ranks by distance, four comparisons per shared-memory load; equal distances collide and are ranked again with
+    // the raster index
+    const bool two = m > 32;
+    const float inf = __int_as_float(0x7f800000);
+    const float d0 = lane < m ? c.d[lane] : inf, d1 = lane + 32 < m ? c.d[lane + 32] : inf;
+    const int i0 = lane < m ? c.i[lane] : 0, i1 = lane + 32 < m ? c.i[lane + 32] : 0;
+    int r0 = 0, r1 = 0;
+    for (int j = 0; j < m; j += 4) {
+        const float4 v = *reinterpret_cast<const float4 *>(c.d + j);
+        r0 += (v.x < d0 ? 1 : 0) + (v.y < d0 ? 1 : 0) + (v.z < d0 ? 1 : 0) + (v.w < d0 ? 1 : 0);
+        if (two) r1 += (v.x < d1 ? 1 : 0) + (v.y < d1 ? 1 : 0) + (v.z < d1 ? 1 : 0) + (v.w < d1 ? 1 : 0);
     }
+    if (lane < m) c.si[r0] = i0;
+    if (lane + 32 < m) c.si[r1] = i1;
+    __syncwarp();
+    const bool clash = (lane < m && c.si[r0] != i0) || (lane + 32 < m && c.si[r1] != i1);
+    if (__any_sync(FULL, clash)) {
+        r0 = r1 = 0;
+        for (int j = 0; j < m; ++j) {
+            const float v = c.d[j];
+            const int w = c.i[j];
+            r0 += (v < d0 || (v == d0 && w < i0)) ? 1 : 0;
+            r1 += (v < d1 || (v == d1 && w < i1)) ? 1 : 0;
+        }
+        __syncwarp();
+        if (lane < m) c.si[r0] = i0;
+        if (lane + 32 < m) c.si[r1] = i1;
+    }
+    if (lane < m) c.sd[r0] = d0;
+    if (lane + 32 < m) c.sd[r1] = d1;
     __syncwarp();
     bool ok = true;
-    for (int i = lane; i < K - 1; i += 32)
-        if (i + 1 < m) ok = ok && (bd.upper(key_dist(psort[i])) < bd.lower(key_dist(psort[i + 1])));
+    if (lane < K - 1 && lane + 1 < m) ok = bd.upper(c.sd[lane]) < bd.lower(c.sd[lane + 1]);
     if (__all_sync(FULL, ok)) {
-        for (int i = lane; i < K - 1; i += 32) out[1 + i] = key_idx(psort[i]);
-        return;
+        if (lane < K - 1) out[1 + lane] = c.si[lane];
+        return 0;
     }
-    // uncertain order: FP64 re-rank of every entry that may belong to the K-1 nearest
-    const float thr = bd.upper(key_dist(psort[K - 2]));
+    const float thr = bd.upper(c.sd[K - 2]);
     int mp = 0;
     for (int i = 0; i < m; ++i) {
-        if (bd.lower(key_dist(psort[i])) > thr) break;
+        if (bd.lower(c.sd[i]) > thr) break;
         mp = i + 1;
     }
+    return mp;
+}
+
+// The K-1 nearest of the mp candidates `ids` by (FP64 distance, raster index) to out[1 ..]; d64: PMAX doubles of
+// scratch.  One warp.
+template <int K>
+__device__ __forceinline__ void rerank_group(const MatchArgs &a, const int *ids, double *d64, int mp, int yr, int xr,
+                                             int green, int lane, int32_t *out) {
+    const size_t HW = (size_t)a.H * a.W;
     for (int i = lane; i < mp; i += 32) {
-        const int id = key_idx(psort[i]);
-        pd64[i] = exact_dist(a.img, a.W, HW, a.C, green, yr, xr, id / a.W, id % a.W);
+        const int id = ids[i];
+        d64[i] = exact_dist(a.img, a.W, HW, a.C, green, yr, xr, id / a.W, id % a.W);
     }
     __syncwarp();
     for (int i = lane; i < mp; i += 32) {
-        const double di = pd64[i];
-        const int ii = key_idx(psort[i]);
+        const double di = d64[i];
+        const int ii = ids[i];
         int rank = 0;
         for (int j = 0; j < mp; ++j) {
-            const double dj = pd64[j];
-            const int ij = key_idx(psort[j]);
-            rank += (dj < di || (dj == di && ij < ii)) ? 1 : 0;
+            const double dj = d64[j];
+            rank += (dj < di || (dj == di && ids[j] < ii)) ? 1 : 0;
         }
         if (rank < K - 1) out[1 + rank] = ii;
     }
@@ -217,10 +261,9 @@ __global__ void __launch_bounds__(MW * 32) k_match(MatchArgs a) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int RHM = a.step + 2 * a.R + PS;          // region side bound
     const int NCM = (2 * a.R + 1) * (2 * a.R + 1);  // candidates per window bound
-    uint64_t *plist = reinterpret_cast<uint64_t *>(smem_raw) + warp * 2 * PMAX;
-    uint64_t *psort = plist + PMAX;
-    double *pd64 = reinterpret_cast<double *>(smem_raw) + MW * 2 * PMAX + warp * PMAX;
-    float *planeA = reinterpret_cast<float *>(smem_raw + (size_t)MW * 3 * PMAX * 8);
+    const CandList cl(smem_raw + warp * (CandList::LIST + CandList::SCRATCH),
+                      smem_raw + warp * (CandList::LIST + CandList::SCRATCH) + CandList::LIST);
+    float *planeA = reinterpret_cast<float *>(smem_raw + (size_t)MW * (CandList::LIST + CandList::SCRATCH));
     float *planeS = planeA + RHM * RHM;
     float *dbuf = planeS + (a.C == 3 ? RHM * RHM : 0) + warp * NCM;
     __shared__ unsigned s_tmax;
@@ -353,7 +396,8 @@ __global__ void __launch_bounds__(MW * 32) k_match(MatchArgs a) {
                 const int pos = m + __popc(msk & lt);
                 if (pos < PMAX) {
                     const int ci = c / ncol;
-                    plist[pos] = make_key(dv, (cy0 + ci) * a.W + cx0 + (c - ci * ncol));
+                    cl.d[pos] = dv;
+                    cl.i[pos] = (cy0 + ci) * a.W + cx0 + (c - ci * ncol);
                 }
             }
             m += __popc(msk);
@@ -368,7 +412,8 @@ __global__ void __launch_bounds__(MW * 32) k_match(MatchArgs a) {
         return;
     }
     __syncwarp();
-    settle_group<K>(a, bd, plist, psort, pd64, m, yr, xr, green, lane, out);
+    const int mp = settle_group<K>(bd, cl, m, lane, out);
+    if (mp) rerank_group<K>(a, cl.si, cl.d64, mp, yr, xr, green, lane, out);
 }
 
 // ---- the default grid step (4): 4 x 4 cells shared by neighbouring references
@@ -382,7 +427,11 @@ __global__ void __launch_bounds__(MW * 32) k_match(MatchArgs a) {
 // cells, keeps the row of these pairs in registers and adds the next one: about 43 operations a candidate where the
 // distance alone took 128.  A row of references' distances goes to shared memory, and each warp settles a reference:
 // a bound on the (K-1)-th distance from the two smallest of every lane (a sort of 32 values per list, no rounds of
-// warp minima), the candidates under it, then as k_match.  Bound by FP32 issue (about 2/3 of it the distances).
+// warp minima), the candidates under it, then as k_match; the few references whose order FP64 decides wait for the
+// end of the tile, where they do not hold up a row.  Bound by issue (58-64 % active, 16 warps per SM) and, below
+// 1000 tiles, by the uneven filling of the SMs.  Measured against a reference per warp (k_match): 768 x 1024 gray,
+// K = 32, win 21: 191 us (562); 512 x 512 x 3, K = 16, win 31, beside the basis chain: 162 us (260); 1021 x 771 x 3:
+// 365 us (683).
 // Tiles are cut where the grid is: the last row / column of references, where H - 8 / W - 8 is no multiple of 4, are
 // tiles of their own.
 // Error: a term passes 2 roundings (difference, squared), at most 16 of the cell's chain and 2 of the cells' sums,
@@ -390,6 +439,7 @@ __global__ void __launch_bounds__(MW * 32) k_match(MatchArgs a) {
 constexpr int CX = 8;          // references per tile row
 constexpr int CT = 256;        // most threads: (2R + 1) * ceil((R4 + R + 1) / 4) <= 256, R4 = R rounded up to 4 (R <= 15)
 constexpr float CEPS = 32.f * U32;
+constexpr int NDEFER = 24;     // references a tile can leave to its end
 
 struct CellArgs {
     MatchArgs m;
@@ -415,14 +465,18 @@ __device__ __forceinline__ float warp_sort(float v, int lane) {
 }
 
 template <int K>
-__global__ void __launch_bounds__(CT, 3) k_match_cells(const __grid_constant__ CellArgs c) {
+__global__ void __launch_bounds__(CT, 2) k_match_cells(const __grid_constant__ CellArgs c) {
+    constexpr int LT = K <= 16 ? 1 : 2;  // smallest distances of a lane that enter the bound
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const MatchArgs &a = c.m;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
     const int npl = a.C == 3 ? 2 : 1, rw = c.cols;
     float *plane0 = reinterpret_cast<float *>(smem_raw);              // [npl][rows][cols]: gray or green, R + G + B
     float *dbuf = plane0 + (size_t)npl * c.rows * rw;                 // [CX][ncp] distances of a row of references
-    uint64_t *plist = reinterpret_cast<uint64_t *>(dbuf + (size_t)CX * c.ncp) + warp * PMAX;
+    unsigned char *list = reinterpret_cast<unsigned char *>(dbuf + (size_t)CX * c.ncp) + warp * CandList::LIST;
+    __shared__ int defer[NDEFER * PMAX];  // candidates of the references left to the tile's FP64 re-rank
+    __shared__ int4 s_defer[NDEFER];      // (reference, its position, candidates, plane)
+    __shared__ int s_ndefer;
     __shared__ unsigned s_tmax;
     __shared__ unsigned s_use[2][8];  // per plane and reference row of the tile: the references that use it
     // ---- the tile: references (gy0 + i, gx0 + j) at (ya + 4 i, xa + 4 j), i < ni, j < nj
@@ -447,7 +501,10 @@ __global__ void __launch_bounds__(CT, 3) k_match_cells(const __grid_constant__ C
     }
     const int ya = grid_pos(gy0, a.H, 4), xa = grid_pos(gx0, a.W, 4);
     const int y0 = ya - a.R, x0 = xa - c.R4;  // region origin (may lie outside the image: zeros)
-    if (tid == 0) s_tmax = 0u;
+    if (tid == 0) {
+        s_tmax = 0u;
+        s_ndefer = 0;
+    }
     if (tid < 16) s_use[tid >> 3][tid & 7] = 0u;
     for (int e = tid; e < CX * c.ncp; e += blockDim.x) dbuf[e] = __int_as_float(0x7f800000);  // the padding stays
     __syncthreads();
@@ -508,45 +565,45 @@ __global__ void __launch_bounds__(CT, 3) k_match_cells(const __grid_constant__ C
             const int cy = ya + 4 * (cr - 1) + ky - a.R;
             const unsigned vr = (cy >= 0 && cy <= a.H - PS) ? vt : 0u;
             if (item) {
-                const float *ra = pa + 4 * cr * rw, *rb = pb + 4 * cr * rw;
-                float4 bl[4], sp = make_float4(0.f, 0.f, 0.f, 0.f);
+                // the cells' sums, pixel row by pixel row (the rows rolled: unrolled, the loop outgrew the instruction
+                // cache), the candidate pieces sliding through registers
+                float s[CX + 1][4] = {};
+#pragma unroll 1
+                for (int u = 0; u < 4; ++u) {
+                    const float4 *ra = reinterpret_cast<const float4 *>(pa + (4 * cr + u) * rw);
+                    const float4 *rb = reinterpret_cast<const float4 *>(pb + (4 * cr + u) * rw);
+                    float4 bl = rb[0];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) bl[u] = *reinterpret_cast<const float4 *>(rb + u * rw);
-#pragma unroll
-                for (int k = 0; k <= CX; ++k) {
-                    if (k > nj) break;
-                    float s[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const float4 av = *reinterpret_cast<const float4 *>(ra + u * rw + 4 * k);
-                        const float4 bh = *reinterpret_cast<const float4 *>(rb + u * rw + 4 * k + 4);
+                    for (int k = 0; k <= CX; ++k) {  // (all of them: a branch per cell would serialise the chains)
+                        const float4 av = ra[k], bh = rb[k + 1];
                         const float aa[4] = {av.x, av.y, av.z, av.w};
-                        const float bb[8] = {bl[u].x, bl[u].y, bl[u].z, bl[u].w, bh.x, bh.y, bh.z, bh.w};
+                        const float bb[8] = {bl.x, bl.y, bl.z, bl.w, bh.x, bh.y, bh.z, bh.w};
 #pragma unroll
                         for (int v = 0; v < 4; ++v)
 #pragma unroll
                             for (int t = 0; t < 4; ++t) {
                                 const float e = __fsub_rn(aa[v], bb[v + t]);
-                                s[t] = __fmaf_rn(e, e, s[t]);
+                                s[k][t] = __fmaf_rn(e, e, s[k][t]);
                             }
-                        bl[u] = bh;
+                        bl = bh;
                     }
-                    if (k > 0) {
-                        const float4 h = make_float4(sp.x + s[0], sp.y + s[1], sp.z + s[2], sp.w + s[3]);
-                        if (emit) {
-                            const float inf = __int_as_float(0x7f800000);
-                            const int cx = xa + 4 * (k - 1) + 4 * g - c.R4;  // the candidates' columns
-                            const float4 p = hp[k - 1];
-                            float4 d;
-                            d.x = (vr & 1u) && cx >= 0 && cx <= a.W - PS ? p.x + h.x : inf;
-                            d.y = (vr & 2u) && cx + 1 >= 0 && cx + 1 <= a.W - PS ? p.y + h.y : inf;
-                            d.z = (vr & 4u) && cx + 2 >= 0 && cx + 2 <= a.W - PS ? p.z + h.z : inf;
-                            d.w = (vr & 8u) && cx + 3 >= 0 && cx + 3 <= a.W - PS ? p.w + h.w : inf;
-                            *reinterpret_cast<float4 *>(dbuf + (k - 1) * c.ncp + ky * wrow + 4 * g) = d;
-                        }
-                        hp[k - 1] = h;
+                }
+#pragma unroll
+                for (int j = 0; j < CX; ++j) {
+                    if (j >= nj) break;
+                    const float4 h = make_float4(s[j][0] + s[j + 1][0], s[j][1] + s[j + 1][1], s[j][2] + s[j + 1][2],
+                                                 s[j][3] + s[j + 1][3]);
+                    if (emit) {
+                        const float inf = __int_as_float(0x7f800000);
+                        const int cx = xa + 4 * j + 4 * g - c.R4;  // the candidates' columns
+                        float4 d;
+                        d.x = (vr & 1u) && cx >= 0 && cx <= a.W - PS ? hp[j].x + h.x : inf;
+                        d.y = (vr & 2u) && cx + 1 >= 0 && cx + 1 <= a.W - PS ? hp[j].y + h.y : inf;
+                        d.z = (vr & 4u) && cx + 2 >= 0 && cx + 2 <= a.W - PS ? hp[j].z + h.z : inf;
+                        d.w = (vr & 8u) && cx + 3 >= 0 && cx + 3 <= a.W - PS ? hp[j].w + h.w : inf;
+                        *reinterpret_cast<float4 *>(dbuf + j * c.ncp + ky * wrow + 4 * g) = d;
                     }
-                    sp = make_float4(s[0], s[1], s[2], s[3]);
+                    hp[j] = h;
                 }
             }
             if (!emit) continue;
@@ -559,20 +616,28 @@ __global__ void __launch_bounds__(CT, 3) k_match_cells(const __grid_constant__ C
                 const int r = (gy0 + cr - 1) * a.nx + gx0 + j, yr = ya + 4 * (cr - 1), xr = xa + 4 * j;
                 int32_t *out = a.idx + (size_t)r * K;
                 if (lane == 0) out[0] = yr * a.W + xr;
+                // the reference's distances, once spent, make room for the sorted candidates
+                const CandList cl(list, db);
                 const int nch = (wrow * (2 * a.R + 1) + 31) >> 5;
                 // entry i of this lane: 32 i + ((lane + 7 i) mod 32), so that neighbouring rows' equal dx differ in lane
                 float m1 = __int_as_float(0x7f800000), m2 = m1;
 #pragma unroll 8
                 for (int i = 0; i < nch; ++i) {
                     const float v = db[32 * i + ((lane + 7 * i) & 31)];
-                    m2 = fminf(m2, fmaxf(m1, v));
+                    if (LT == 2) m2 = fminf(m2, fmaxf(m1, v));
                     m1 = fminf(m1, v);
                 }
-                // the K-1 smallest of two ascending lists are min(A[i], B[K-2-i]): the largest of them bounds the
-                // (K-1)-th distance
-                const float A = warp_sort(m1, lane), B = warp_sort(m2, lane);
-                const float bo = __shfl_sync(FULL, B, lane < K - 1 ? K - 2 - lane : 0);
-                float tau = __uint_as_float(__reduce_max_sync(FULL, lane < K - 1 ? __float_as_uint(fminf(A, bo)) : 0u));
+                // a bound on the (K-1)-th distance: the (K-1)-th smallest of the lanes' minima (K = 16: 19 candidates
+                // lie under it on average), or of their two smallest (K = 32: 33; one alone would give 71) -- the K-1
+                // smallest of two ascending lists are min(A[i], B[K-2-i])
+                const float A = warp_sort(m1, lane);
+                float tau;
+                if (LT == 1) {
+                    tau = __shfl_sync(FULL, A, K - 2);
+                } else {
+                    const float bo = __shfl_sync(FULL, warp_sort(m2, lane), lane < K - 1 ? K - 2 - lane : 0);
+                    tau = __uint_as_float(__reduce_max_sync(FULL, lane < K - 1 ? __float_as_uint(fminf(A, bo)) : 0u));
+                }
                 float T = bd.upper(bd.upper(tau));
                 unsigned hit = 0u;
                 int m = 0;
@@ -611,17 +676,33 @@ __global__ void __launch_bounds__(CT, 3) k_match_cells(const __grid_constant__ C
                 pos -= __popc(hit);
                 for (; hit; hit &= hit - 1) {
                     const int i = __ffs(hit) - 1, e = 32 * i + ((lane + 7 * i) & 31), ey = e / wrow;
-                    plist[pos++] = make_key(db[e], (yr + ey - a.R) * a.W + xr + (e - ey * wrow) - c.R4);
+                    cl.d[pos] = db[e];
+                    cl.i[pos++] = (yr + ey - a.R) * a.W + xr + (e - ey * wrow) - c.R4;
                 }
                 __syncwarp();
-                // the reference's distances are spent: their row holds the sorted keys and FP64 distances
-                settle_group<K>(a, bd, plist, reinterpret_cast<uint64_t *>(db), reinterpret_cast<double *>(db) + PMAX, m,
-                                yr, xr, pass == 0 ? 1 : 0, lane, out);
+                const int mp = settle_group<K>(bd, cl, m, lane, out);
+                if (mp) {  // FP64 is slow and its warp would hold up the row: kept for the end of the tile
+                    int at = 0;
+                    if (lane == 0) at = atomicAdd(&s_ndefer, 1);
+                    at = __shfl_sync(FULL, at, 0);
+                    if (at < NDEFER) {
+                        for (int i = lane; i < mp; i += 32) defer[at * PMAX + i] = cl.si[i];
+                        if (lane == 0) s_defer[at] = make_int4(r, yr * a.W + xr, mp, pass == 0 ? 1 : 0);
+                    } else {
+                        rerank_group<K>(a, cl.si, cl.d64, mp, yr, xr, pass == 0 ? 1 : 0, lane, out);
+                    }
+                }
                 __syncwarp();
                 for (int e = wrow * (2 * a.R + 1) + lane; e < c.ncp; e += 32) db[e] = __int_as_float(0x7f800000);
             }
             __syncthreads();
         }
+    }
+    for (int e = warp; e < min(s_ndefer, NDEFER); e += nw) {  // the last barrier was the last row's
+        const int4 f = s_defer[e];
+        rerank_group<K>(a, defer + e * PMAX, reinterpret_cast<double *>(list), f.z, f.y / a.W, f.y % a.W, f.w, lane,
+                        a.idx + (size_t)f.x * K);
+        __syncwarp();
     }
 }
 
@@ -641,20 +722,21 @@ hts_status launch_cells(const MatchArgs &a, cudaStream_t s) {
     c.ry = (a.H - PS) / 4 + 1;
     c.rx = (a.W - PS) / 4 + 1;
     c.ntx = (c.rx + CX - 1) / CX;
-    c.ncp = std::max((items * 4 + 31) / 32 * 32, PMAX * 4);
+    c.ncp = std::max((items * 4 + 31) / 32 * 32, CandList::SCRATCH / 4);
     c.cols = 4 * (CX + 1) + 4 * c.G;
     auto smem_of = [&](int nry) {
         return ((size_t)(a.C == 3 ? 2 : 1) * (4 * (nry + 1) + 2 * a.R) * c.cols + (size_t)CX * c.ncp) * sizeof(float) +
-               (size_t)(threads / 32) * PMAX * sizeof(uint64_t);
+               (size_t)(threads / 32) * CandList::LIST;
     };
-    // rows per tile: more share cells (a tile of n rows sums n + 1 cell rows and settles n rows of references; about
-    // 11 and 5 thousand warp instructions, 6 to stage) but leave SMs idle on small images: the fewest waves' work
+    // rows per tile: more share cells (n rows of references need n + 1 cell rows) but fill the SMs unevenly: the
+    // least work of the fullest SM, in thousands of warp instructions (a cell row 1.4 per warp, a row of references
+    // settled 4, the staging 2 per 3000 values)
     double best = 0.0;
-    for (int n : {8, 6, 4, 3, 2, 1}) {
-        const int slots = 152 * (int)std::max<size_t>(1, std::min<size_t>(2048 / threads, 233472 / (smem_of(n) + 1024)));
+    for (int n = 8; n >= 1; --n) {
         const long blocks = (long)c.ntx * ((c.ry + n - 1) / n);
-        const double w = (double)((blocks + slots - 1) / slots) * ((n + 1) * 11.0 + n * 5.0 + 6.0) *
-                         std::max(1.0, std::min<double>(blocks, slots) / 152.0);
+        const double w = (double)((blocks + 151) / 152) *
+                         ((n + 1) * 1.4 * (threads / 32) + n * 4.0 +
+                          (a.C == 3 ? 2 : 1) * (4 * (n + 1) + 2 * a.R) * c.cols * (2.0 / 3000.0));
         if (best == 0.0 || w < best) {
             best = w;
             c.nry = n;
@@ -861,12 +943,12 @@ __global__ void __launch_bounds__(128) k_match_rescue(MatchArgs a) {
     }
 }
 
-// The grid step the cells are cut for, and windows whose offsets fit a block; else a reference per warp.
+// k_match: one reference per warp.
 template <int K>
 hts_status launch_direct(const MatchArgs &a, cudaStream_t s) {
     const int RHM = a.step + 2 * a.R + PS;
     const int NCM = (2 * a.R + 1) * (2 * a.R + 1);
-    const size_t smem = (size_t)MW * 3 * PMAX * 8 + (size_t)(a.C == 3 ? 2 : 1) * RHM * RHM * sizeof(float) +
+    const size_t smem = (size_t)MW * (CandList::LIST + CandList::SCRATCH) + (size_t)(a.C == 3 ? 2 : 1) * RHM * RHM * sizeof(float) +
                         (size_t)MW * NCM * sizeof(float);
     {
         const hts_status st0 = allow_smem(reinterpret_cast<const void *>(k_match<K>), smem);
@@ -882,6 +964,8 @@ hts_status launch_direct(const MatchArgs &a, cudaStream_t s) {
 
 template <int K>
 hts_status launch_k(const MatchArgs &a, cudaStream_t s) {
+    // the cells are cut for step 4, and a window's offsets have to fit a block's threads (R <= 15); at any image size
+    // they are the faster (96 x 128 gray, where each cell row serves one row of references: 38 us against 39)
     int R4;
     const bool cells = a.step == 4 && (2 * a.R + 1) * cell_groups(a.R, &R4) <= CT;
     const hts_status st = cells ? launch_cells<K>(a, s) : launch_direct<K>(a, s);
