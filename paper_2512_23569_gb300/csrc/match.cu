@@ -816,130 +816,193 @@ __global__ void __launch_bounds__(128) k_match_fallback(MatchArgs a) {
     }
 }
 
-// Exhaustive matching, in FP32, of the references the tensor-core matcher
-// listed in a.fb (count in a.st->match_fallback): one block of four warps per
-// reference, its search region staged in shared memory as FP32 plane values
-// ((R + G) + B for the channel sum), distances as FP32 fused multiply-adds
-// in the definition's (u, v) order -- the arithmetic of the tensor-core
-// matcher's re-rank -- and the K-1 nearest by (distance, raster index).  The
-// matching plane comes from a.green (Eq. 9 flags already decided).
+// Exhaustive matching, in FP32, of the references the tensor-core matcher listed in a.fb (count in
+// a.st->match_fallback): distances as FP32 fused multiply-adds in the definition's (u, v) order on the FP32 plane
+// ((R + G) + B for the channel sum) -- the arithmetic of the tensor-core matcher's re-rank -- and the K-1 nearest by
+// (distance, raster index).  The matching plane comes from a.green (Eq. 9 flags already decided).  A few references
+// in a thousand on most images, over half of them on images full of gratings, whose equally good candidates crowd the
+// matcher's bins.  One warp per reference: the region staged in shared memory, four consecutive candidates per lane
+// and item with the reference in registers (three 16-byte loads of candidates, conflict-free, for 64 operations),
+// distances to shared memory, then the bound from the lanes' minima and a sort of the few candidates under it.
+// Bound by FP32 issue.  Before (a block per reference, two loads per pixel and candidate, per-thread insertion lists
+// merged by one thread): 27 references / us at 1536 x 2048 x 3, now 96.
+constexpr unsigned NONE = 0xffffffffu;  // no candidate: above every distance's bits
+constexpr int RW = 4;                   // warps per block
+
+struct RescueShape {
+    int R4, G, cols, rows, ncp;  // as CellArgs; ncp: candidates, padded to whole chunks of 32
+    __host__ __device__ explicit RescueShape(int R)
+        : R4((R + 3) / 4 * 4), G((R4 + R + 4) / 4), cols(4 * G + 8), rows(2 * R + PS),
+          ncp(((2 * R + 1) * 4 * G + 31) / 32 * 32) {}
+    __host__ __device__ size_t floats() const { return (size_t)cols * rows + ncp + 4 * PMAX; }  // per warp
+};
+
+__device__ __forceinline__ unsigned warp_sort_u(unsigned v, int lane) {
+#pragma unroll
+    for (int k = 2; k <= 32; k <<= 1)
+#pragma unroll
+        for (int j = k >> 1; j; j >>= 1) {
+            const unsigned o = __shfl_xor_sync(FULL, v, j);
+            const bool up = (lane & k) == 0, low = (lane & j) == 0;
+            v = (up == low) ? min(v, o) : max(v, o);
+        }
+    return v;
+}
+
 template <int K>
-__global__ void __launch_bounds__(128) k_match_rescue(MatchArgs a) {
+__global__ void __launch_bounds__(RW * 32) k_match_rescue(MatchArgs a) {
     constexpr int L = K - 1;
-    extern __shared__ float rs_plane[];  // (2R + 8)^2 region values, then the warps' lists
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int LT = K <= 16 ? 1 : 2;  // smallest distances of a lane that enter the bound (as k_match_cells)
+    extern __shared__ __align__(16) float rs_smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int count = *(volatile int *)&a.st->match_fallback;
     const size_t HW = (size_t)a.H * a.W;
-    const int side = 2 * a.R + PS;
-    float *wd = rs_plane + (size_t)side * side;  // [4][L]
-    int *wi = reinterpret_cast<int *>(wd + 4 * L);  // [4][L]
-    for (int f = blockIdx.x; f < count; f += gridDim.x) {
+    const RescueShape S(a.R);
+    float *plane = rs_smem + warp * S.floats();                                // [rows][cols]
+    unsigned *db = reinterpret_cast<unsigned *>(plane + S.cols * S.rows);      // [ncp] distances' bits, raster order
+    unsigned *cd = db + S.ncp;                                                 // [PMAX] collected distances
+    int *ci = reinterpret_cast<int *>(cd + PMAX), *si = ci + PMAX;             // and indices; sorted indices
+    const int wrow = 4 * S.G, items = (2 * a.R + 1) * S.G, nch = S.ncp / 32;
+    const unsigned below = (1u << lane) - 1u;
+    for (int f = blockIdx.x * RW + warp; f < count; f += gridDim.x * RW) {
         const int r = a.fb[f];
         const int yr = grid_pos(r / a.nx, a.H, a.step), xr = grid_pos(r % a.nx, a.W, a.step);
         const int green = (a.C == 3) ? (int)a.green[r] : 1;
-        const int cy0 = max(0, yr - a.R), cy1 = min(a.H - PS, yr + a.R);
-        const int cx0 = max(0, xr - a.R), cx1 = min(a.W - PS, xr + a.R);
-        const int ncol = cx1 - cx0 + 1, ncand = (cy1 - cy0 + 1) * ncol;
-        const int rw = ncol + PS - 1, rh = cy1 - cy0 + PS;  // staged rows and columns
-        __syncthreads();  // the previous reference's lists are read
-        for (int e = tid; e < rw * rh; e += 128) {
-            const int y = e / rw, x = e - y * rw;
-            const size_t o = (size_t)(cy0 + y) * a.W + cx0 + x;
-            float v;
-            if (a.C == 1) v = __ldg(a.img + o);
-            else if (green) v = __ldg(a.img + HW + o);
-            else v = (__ldg(a.img + o) + __ldg(a.img + HW + o)) + __ldg(a.img + 2 * HW + o);
-            rs_plane[e] = v;
-        }
-        __syncthreads();
-        const float *ref = rs_plane + (size_t)(yr - cy0) * rw + (xr - cx0);
-        float dl[L];
-        int il[L];
+        const int y0 = yr - a.R, x0 = xr - S.R4;
+        __syncwarp();  // the previous reference's values are read
+        {  // the region, 16 elements in flight per lane (columns and rows advanced by 32 elements, no divisions)
+            const bool one = a.C == 1 || green;  // the plane is one channel
+            const float *ch = a.img + (a.C == 3 && green ? HW : 0);
+            const int dq = 32 / S.cols, dr = 32 - dq * S.cols;
+            int x = x0 + lane % S.cols, y = y0 + lane / S.cols;
+            for (int e0 = lane; e0 < S.rows * S.cols; e0 += 16 * 32) {
+                float v[16];
 #pragma unroll
-        for (int i = 0; i < L; ++i) {
-            dl[i] = __builtin_huge_valf();
-            il[i] = 0x7fffffff;
-        }
-        for (int c = tid; c < ncand; c += 128) {
-            const int cy = c / ncol, cx = c - cy * ncol;
-            if (cy0 + cy == yr && cx0 + cx == xr) continue;
-            const float *cand = rs_plane + (size_t)cy * rw + cx;
-            float D = 0.f;
-            for (int u = 0; u < PS; ++u)
-#pragma unroll
-                for (int v = 0; v < PS; ++v) {
-                    const float d = ref[u * rw + v] - cand[u * rw + v];
-                    D = fmaf(d, d, D);
-                }
-            const int id = (cy0 + cy) * a.W + cx0 + cx;
-            if (D > dl[L - 1] || (D == dl[L - 1] && id > il[L - 1])) continue;
-#pragma unroll
-            for (int i = L - 1; i > 0; --i) {
-                const bool shift = (dl[i - 1] > D) || (dl[i - 1] == D && il[i - 1] > id);
-                const bool here = !shift && ((dl[i] > D) || (dl[i] == D && il[i] > id));
-                if (shift) {
-                    dl[i] = dl[i - 1];
-                    il[i] = il[i - 1];
-                } else if (here) {
-                    dl[i] = D;
-                    il[i] = id;
-                }
-            }
-            if ((dl[0] > D) || (dl[0] == D && il[0] > id)) {
-                dl[0] = D;
-                il[0] = id;
-            }
-        }
-        // each warp: the L smallest of its lanes' lists (L rounds of a warp arg-min over the list heads)
-        for (int j = 0; j < L; ++j) {
-            float bd = dl[0];
-            int bi = il[0];
-#pragma unroll
-            for (int o = 16; o; o >>= 1) {
-                const float od = __shfl_xor_sync(FULL, bd, o);
-                const int oi = __shfl_xor_sync(FULL, bi, o);
-                if (od < bd || (od == bd && oi < bi)) {
-                    bd = od;
-                    bi = oi;
-                }
-            }
-            if (lane == 0) {
-                wd[warp * L + j] = bd;
-                wi[warp * L + j] = bi;
-            }
-            if (il[0] == bi && dl[0] == bd) {
-#pragma unroll
-                for (int t = 0; t < L - 1; ++t) {
-                    dl[t] = dl[t + 1];
-                    il[t] = il[t + 1];
-                }
-                dl[L - 1] = __builtin_huge_valf();
-                il[L - 1] = 0x7fffffff;
-            }
-        }
-        __syncthreads();
-        if (tid == 0) {  // merge of the four warps' sorted lists
-            int h[4] = {0, 0, 0, 0};
-            int32_t *out = a.idx + (size_t)r * K;
-            out[0] = yr * a.W + xr;
-            for (int j = 0; j < L; ++j) {
-                int bw = -1;
-                float bd = 0.f;
-                int bi = 0x7fffffff;
-                for (int w = 0; w < 4; ++w) {
-                    if (h[w] >= L) continue;
-                    const float dv = wd[w * L + h[w]];
-                    const int iv = wi[w * L + h[w]];
-                    if (bw < 0 || dv < bd || (dv == bd && iv < bi)) {
-                        bw = w;
-                        bd = dv;
-                        bi = iv;
+                for (int i = 0; i < 16; ++i) {
+                    const bool in = e0 + 32 * i < S.rows * S.cols && y >= 0 && y < a.H && x >= 0 && x < a.W;
+                    const size_t o = in ? (size_t)y * a.W + x : 0;
+                    v[i] = in ? __ldg(ch + o) : 0.f;
+                    if (!one && in) v[i] = (v[i] + __ldg(a.img + HW + o)) + __ldg(a.img + 2 * HW + o);
+                    x += dr;
+                    y += dq;
+                    if (x >= x0 + S.cols) {
+                        x -= S.cols;
+                        ++y;
                     }
                 }
-                ++h[bw];
-                out[1 + j] = (bi == 0x7fffffff) ? out[0] : bi;
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    if (e0 + 32 * i < S.rows * S.cols) plane[e0 + 32 * i] = v[i];
             }
         }
+        __syncwarp();
+        float ar[NPIX];
+#pragma unroll
+        for (int e = 0; e < NPIX; e += 4)
+            *reinterpret_cast<float4 *>(ar + e) =
+                *reinterpret_cast<const float4 *>(plane + (a.R + (e >> 3)) * S.cols + S.R4 + (e & 7));
+        unsigned m1 = NONE, m2 = NONE;  // this lane's two smallest
+        for (int it = lane; it < S.ncp / 4; it += 32) {
+            uint4 d = make_uint4(NONE, NONE, NONE, NONE);
+            if (it < items) {
+                const int ky = it / S.G, g = it - ky * S.G;
+                const float *row = plane + ky * S.cols + 4 * g;
+                float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int u = 0; u < PS; ++u) {
+                    float b[12];
+#pragma unroll
+                    for (int i = 0; i < 12; i += 4)
+                        *reinterpret_cast<float4 *>(b + i) = *reinterpret_cast<const float4 *>(row + u * S.cols + i);
+#pragma unroll
+                    for (int v = 0; v < PS; ++v)
+#pragma unroll
+                        for (int t = 0; t < 4; ++t) {
+                            const float e = ar[u * PS + v] - b[v + t];
+                            acc[t] = fmaf(e, e, acc[t]);
+                        }
+                }
+                const int cy = y0 + ky, cx = x0 + 4 * g, dx = 4 * g - S.R4;
+                const bool rowok = cy >= 0 && cy <= a.H - PS;
+                unsigned *dv = &d.x;
+#pragma unroll
+                for (int t = 0; t < 4; ++t)
+                    if (rowok && cx + t >= 0 && cx + t <= a.W - PS && dx + t >= -a.R && dx + t <= a.R &&
+                        !(ky == a.R && dx + t == 0))
+                        dv[t] = __float_as_uint(acc[t]);
+            }
+            *reinterpret_cast<uint4 *>(db + 4 * it) = d;
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const unsigned v = (&d.x)[t];
+                if (LT == 2) m2 = min(m2, max(m1, v));
+                m1 = min(m1, v);
+            }
+        }
+        __syncwarp();
+        // a bound on the L-th distance: the L-th smallest of the lanes' smallest (K = 32: of their two smallest; of
+        // two ascending lists the L smallest are min(A[i], B[L-1-i]))
+        const unsigned A = warp_sort_u(m1, lane);
+        unsigned T;
+        if (LT == 1) {
+            T = __shfl_sync(FULL, A, L - 1);
+        } else {
+            const unsigned bo = __shfl_sync(FULL, warp_sort_u(m2, lane), lane < L ? L - 1 - lane : 0);
+            T = __reduce_max_sync(FULL, lane < L ? min(A, bo) : 0u);
+        }
+        // candidates below T and, in raster order, at T; more than the list holds (ties, a clustered bound): the exact
+        // L-th distance by bisection, of which only the first ones in raster order can belong to the group
+        int m = 0, nless = 0;
+        for (int pass = 0; pass < 2; ++pass) {
+            m = nless = 0;
+            int cap = PMAX;  // of the candidates at T
+            if (pass == 1) {
+                unsigned lo = 0u, hi = T;  // count(<= hi) >= L
+                while (lo < hi) {
+                    const unsigned mid = lo + (hi - lo) / 2;
+                    int n = 0;
+                    for (int i = 0; i < nch; ++i) n += db[32 * i + lane] <= mid ? 1 : 0;
+                    if (__reduce_add_sync(FULL, n) >= L) hi = mid;
+                    else lo = mid + 1;
+                }
+                T = hi;
+                int n = 0;
+                for (int i = 0; i < nch; ++i) n += db[32 * i + lane] < T ? 1 : 0;
+                cap = L - __reduce_add_sync(FULL, n);  // fewer than L lie below
+            }
+            for (int i = 0; i < nch; ++i) {
+                const int e = 32 * i + lane;
+                const unsigned v = db[e];
+                const bool at = v == T && v != NONE;
+                const unsigned eq = __ballot_sync(FULL, at);
+                const bool ok = v < T || (at && nless + __popc(eq & below) < cap);
+                const unsigned msk = __ballot_sync(FULL, ok);
+                const int pos = m + __popc(msk & below);
+                if (ok && pos < PMAX) {
+                    const int ky = e / wrow;
+                    cd[pos] = v;
+                    ci[pos] = (y0 + ky) * a.W + x0 + (e - ky * wrow);
+                }
+                m += __popc(msk);
+                nless += __popc(eq);  // candidates at T so far
+            }
+            if (m <= PMAX) break;
+        }
+        __syncwarp();
+        // ranks by (distance, raster index): the collected entries are in raster order, so an equal distance ranks
+        // behind the ones collected before it
+        const unsigned d0 = lane < m ? cd[lane] : NONE, d1 = lane + 32 < m ? cd[lane + 32] : NONE;
+        int r0 = 0, r1 = 0;
+        for (int j = 0; j < m; ++j) {
+            const unsigned v = cd[j];
+            r0 += (v < d0 || (v == d0 && j < lane)) ? 1 : 0;
+            r1 += (v < d1 || (v == d1 && j < lane + 32)) ? 1 : 0;
+        }
+        if (lane < m) si[r0] = ci[lane];
+        if (lane + 32 < m) si[r1] = ci[lane + 32];
+        __syncwarp();
+        int32_t *out = a.idx + (size_t)r * K;
+        if (lane < K) out[lane] = lane == 0 || lane > m ? yr * a.W + xr : si[lane - 1];
     }
 }
 
@@ -1080,8 +1143,7 @@ hts_status launch_match_rescue(const float *img, const Geom &g, int32_t *idx, co
     a.green = const_cast<uint8_t *>(green);
     a.fb = fallback_list;
     a.st = st;
-    const size_t side = 2 * (size_t)g.R + PS;
-    const size_t smem = side * side * sizeof(float) + 4 * 32 * (sizeof(float) + sizeof(int));
+    const size_t smem = RW * RescueShape(g.R).floats() * sizeof(float);
     const void *fn = nullptr;
     switch (g.K) {
         case 2: fn = reinterpret_cast<const void *>(k_match_rescue<2>); break;
@@ -1095,15 +1157,15 @@ hts_status launch_match_rescue(const float *img, const Geom &g, int32_t *idx, co
         const hts_status st0 = allow_smem(fn, smem);
         if (st0 != HTS_OK) return st0;
     }
-    const int blocks = 4 * 152;
+    const int blocks = 4 * 152;  // as many as are resident
     {
         KTimer kt("k_match_rescue", s);
         switch (g.K) {
-            case 2: k_match_rescue<2><<<blocks, 128, smem, s>>>(a); break;
-            case 4: k_match_rescue<4><<<blocks, 128, smem, s>>>(a); break;
-            case 8: k_match_rescue<8><<<blocks, 128, smem, s>>>(a); break;
-            case 16: k_match_rescue<16><<<blocks, 128, smem, s>>>(a); break;
-            default: k_match_rescue<32><<<blocks, 128, smem, s>>>(a); break;
+            case 2: k_match_rescue<2><<<blocks, RW * 32, smem, s>>>(a); break;
+            case 4: k_match_rescue<4><<<blocks, RW * 32, smem, s>>>(a); break;
+            case 8: k_match_rescue<8><<<blocks, RW * 32, smem, s>>>(a); break;
+            case 16: k_match_rescue<16><<<blocks, RW * 32, smem, s>>>(a); break;
+            default: k_match_rescue<32><<<blocks, RW * 32, smem, s>>>(a); break;
         }
     }
     return check_launch("k_match_rescue");
