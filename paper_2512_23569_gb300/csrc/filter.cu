@@ -1270,17 +1270,26 @@ __global__ void __launch_bounds__(TPB, 1) k_filter_tile(FilterArgs a, TileArgs t
                     const int ly = py + row - ry0, lx = px - rx0;
                     if (ly >= 0 && ly < rh && lx >= 0 && lx + 7 < rw) {
                         const int o = ly * rw + lx;
+                        bool small = true;
 #pragma unroll
-                        for (int bb = 0; bb < 8; ++bb) {
+                        for (int bb = 0; bb < 8; ++bb)
 #pragma unroll
-                            for (int c = 0; c < C; ++c) {
-                                int qh, ql;
-                                fix16_split(out[c][bb], qh, ql);
-                                atomicAdd(acc_hi + c * RA + o + bb, qh);
-                                atomicAdd(acc_lo + c * RA + o + bb, ql);
+                            for (int c = 0; c < C; ++c) small = small && fabsf(out[c][bb]) < fc::SPLIT_MAX;
+                        auto add = [&](bool sm) {
+#pragma unroll
+                            for (int bb = 0; bb < 8; ++bb) {
+#pragma unroll
+                                for (int c = 0; c < C; ++c) {
+                                    int qh, ql;
+                                    fix16_split(out[c][bb], sm, qh, ql);
+                                    atomicAdd(acc_hi + c * RA + o + bb, qh);
+                                    atomicAdd(acc_lo + c * RA + o + bb, ql);
+                                }
+                                atomicAdd(acc_w + o + bb, 1);
                             }
-                            atomicAdd(acc_w + o + bb, 1);
-                        }
+                        };
+                        if (small) add(true);
+                        else add(false);
                     } else {
                         atomicExch(&a.st->error, 1);
                     }
@@ -1648,15 +1657,42 @@ hts_status launch_normalize(const long long *acc, const int *wcount, float *out,
     return check_launch("k_normalize");
 }
 
+// The tile shape of a call that no batch has tuned: the least time of the fullest SM, in batches of PPB / K groups; a
+// tile's sums to clear and flush cost half a batch and up to half of one more, by area.  The largest shape that fits,
+// taken before, left 128 of 152 SMs idle on a 96 x 128 image (24 tiles of 4 x 8 references; 2 x 4: 96): 76 us, now
+// 26; 512 x 512 x 3 (4 x 4 instead of 4 x 8: seven rounds of four batches for four of eight), with fix16_split's hoisted
+// test: 462 us, now 358.
+template <int C, int K>
+TileChoice model_tile(const Geom &g, int nsm) {
+    TileChoice best{0, 0};
+    double cost = 0.0;
+    for (int i = 0; i < NSHAPES; ++i) {
+        const int ty = SHAPES[i][0], tx = SHAPES[i][1];
+        int rh, rw;
+        if (tile_bytes(g, ty, tx, &rh, &rw) > tile_budget()) continue;
+        const long tiles = (long)((g.ny + ty - 1) / ty) * ((g.nx + tx - 1) / tx);
+        const int nb = (ty * tx * K + PPB - 1) / PPB;
+        const double w = (double)((tiles + nsm - 1) / nsm) * (nb + 0.5 + 0.5 * rh * rw / 3300.0);
+        if (best.ty == 0 || w < cost) {
+            best = {ty, tx};
+            cost = w;
+        }
+    }
+    return best;
+}
+
 template <int C, int K>
 hts_status launch_ck(const FilterArgs &a, const Geom &g, float *out, cudaStream_t s) {
     const size_t HW = (size_t)a.H * a.W;
-    // tile shape: forced (autotuning), tuned, or the largest that fits
+    int dev = 0, nsm = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    // tile shape: forced (autotuning), tuned, or the model's
     TileChoice ch;
     TileChoice cands[NSHAPES + 1];
     tile_candidates(g, cands, NSHAPES + 1);
     if (t_forced) ch = *t_forced;
-    else if (!tuned_tile(g, &ch)) ch = cands[0];
+    else if (!tuned_tile(g, &ch)) ch = model_tile<C, K>(g, nsm);
     if (ch.ty > 0 && tile_bytes(g, ch.ty, ch.tx) > tile_budget()) ch = cands[0];
     const size_t fixed = tile_fixed_smem<C, K>();
     TileArgs ta;
@@ -1676,9 +1712,6 @@ hts_status launch_ck(const FilterArgs &a, const Geom &g, float *out, cudaStream_
         if (st0 == HTS_OK) st0 = allow_smem(reinterpret_cast<const void *>(k_filter_exact<C, K>), sm_exact);
         if (st0 != HTS_OK) return st0;
     }
-    int dev = 0, nsm = 152;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     const int grid = std::max(1, std::min(ta.ntiles, nsm));
     {
         KTimer kt("k_filter", s);

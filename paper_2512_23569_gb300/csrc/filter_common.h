@@ -54,10 +54,13 @@ __device__ __forceinline__ long long fix16(float v) { return __float2ll_rn(v * 6
 // integer (ties to even) and leaves it in the low mantissa bits, for the
 // integer part and again for the 16-bit fraction; both steps are exact, so
 // hi * 2^16 + lo == fix16(v).
-__device__ __forceinline__ void fix16_split(float v, int &hi, int &lo) {
+// The caller tests once whether all its values are that small: as a branch per
+// value the 64-bit conversion was issued, predicated off, with every one.
+constexpr float SPLIT_MAX = 4194304.0f;
+__device__ __forceinline__ void fix16_split(float v, bool small, int &hi, int &lo) {
     constexpr float MAGIC = 12582912.0f;  // 1.5 * 2^23
     constexpr int MAGIC_BITS = 0x4B400000;
-    if (fabsf(v) < 4194304.0f) {
+    if (small) {
         const float t = v + MAGIC;
         hi = __float_as_int(t) - MAGIC_BITS;
         const float f = v - (t - MAGIC);  // v - round(v), exact
