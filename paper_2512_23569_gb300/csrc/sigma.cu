@@ -16,7 +16,9 @@
 // k_sigma_final: a strict majority divides sigma_est by beta (Eq. 23); then
 //                tau = tau_mult sigma sqrt(2 ln(c K ps^2)).
 #include <algorithm>
+#include <cmath>
 #include <cooperative_groups.h>
+#include <type_traits>
 
 #include "hts_internal.h"
 
@@ -151,6 +153,22 @@ __device__ void lambda64_partial(const float *__restrict__ img, int H, int W, co
     }
 }
 
+// One component's value, or two components' side by side: the packed operations round each half as the scalar ones
+// and issue once for both (the FP32 lanes are the same; it is the issue slots that bind the vote).
+__device__ __forceinline__ float vadd(float a, float b) { return a + b; }
+__device__ __forceinline__ float vsub(float a, float b) { return a - b; }
+__device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ float vneg(float a) { return -a; }
+__device__ __forceinline__ float vsum(float a) { return a; }
+__device__ __forceinline__ void vset(float &a, float c) { a = c; }
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 vsub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ float2 vfma(float2 a, float b, float2 c) { return __ffma2_rn(a, make_float2(b, b), c); }
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 vneg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float vsum(float2 a) { return a.x + a.y; }
+__device__ __forceinline__ void vset(float2 &a, float c) { a = make_float2(c, c); }
+
 // Half spectrum X_m, m = 0..N/2, of N real values x (N a power of two, 2..32), into re[m OS], im[m OS]:
 // one radix-2 split per level (a_k = x_k + x_{k+N/2} carries the even outputs, d_k = x_k - x_{k+N/2} the
 // odd ones), the odd outputs X_{2j+1} = sum_k d_k w^{(2j+1) k} evaluated directly, pairing d_k with
@@ -161,42 +179,42 @@ __device__ void lambda64_partial(const float *__restrict__ img, int H, int W, co
 // difference d, the pair, the twiddle's own rounding and at most N / 2^(L+2) - 1 steps of the chain,
 // i.e. at most N/4 + 2 roundings (N >= 4); for X_0, log2 N.  So |Re, Im error| <= gamma_(N/4 + 2)
 // sum_k |x_k|.
-template <int N, int OS, int NO>
-__device__ __forceinline__ void rdft_half(const float *x, float (&re)[NO], float (&im)[NO]) {
+template <int N, int OS, int NO, typename T>
+__device__ __forceinline__ void rdft_half(const T *x, T (&re)[NO], T (&im)[NO]) {
     if constexpr (N == 2) {
-        re[0] = x[0] + x[1];
-        im[0] = 0.f;
-        re[OS] = x[0] - x[1];
-        im[OS] = 0.f;
+        re[0] = vadd(x[0], x[1]);
+        vset(im[0], 0.f);
+        re[OS] = vsub(x[0], x[1]);
+        vset(im[OS], 0.f);
     } else {
         constexpr int n = N / 2;
-        float a[n], d[n];
+        T a[n], d[n];
 #pragma unroll
         for (int k = 0; k < n; ++k) {
-            a[k] = x[k] + x[k + n];
-            d[k] = x[k] - x[k + n];
+            a[k] = vadd(x[k], x[k + n]);
+            d[k] = vsub(x[k], x[k + n]);
         }
-        rdft_half<n, 2 * OS, NO>(a, re, im);
-        float dd[n / 2 > 0 ? n / 2 : 1], ss[n / 2 > 0 ? n / 2 : 1];
+        rdft_half<n, 2 * OS, NO, T>(a, re, im);
+        T dd[n / 2 > 0 ? n / 2 : 1], ss[n / 2 > 0 ? n / 2 : 1];
 #pragma unroll
         for (int k = 1; k < n / 2; ++k) {
-            dd[k] = d[k] - d[n - k];
-            ss[k] = d[k] + d[n - k];
+            dd[k] = vsub(d[k], d[n - k]);
+            ss[k] = vadd(d[k], d[n - k]);
         }
 #pragma unroll
         for (int j = 0; j < n / 2; ++j) {
-            float r = d[0], i = (j & 1) ? d[n / 2] : -d[n / 2];
+            T r = d[0], i = (j & 1) ? d[n / 2] : vneg(d[n / 2]);
 #pragma unroll
             for (int k = 1; k < n / 2; ++k) {
                 const int t = ((2 * j + 1) * k * (32 / N)) & 31;
                 // quarter turns: the twiddle parts are exactly 0 or +-1, the same sums without the products
-                if (t == 0) r += dd[k];
-                else if (t == 8) i -= ss[k];
-                else if (t == 16) r -= dd[k];
-                else if (t == 24) i += ss[k];
+                if (t == 0) r = vadd(r, dd[k]);
+                else if (t == 8) i = vsub(i, ss[k]);
+                else if (t == 16) r = vsub(r, dd[k]);
+                else if (t == 24) i = vadd(i, ss[k]);
                 else {
-                    r = fmaf(dd[k], c_twc[t], r);
-                    i = fmaf(ss[k], c_tws[t], i);
+                    r = vfma(dd[k], c_twc[t], r);
+                    i = vfma(ss[k], c_tws[t], i);
                 }
             }
             re[(2 * j + 1) * OS] = r;
@@ -210,43 +228,59 @@ __device__ __forceinline__ void rdft_half(const float *x, float (&re)[NO], float
 // the FP32 bound cannot settle is listed for k_vote_exact and counts 0 here).
 template <int C, int K>
 __device__ __forceinline__ int vote_group(const float *__restrict__ src, size_t plane, int rstride,
-                                          const int (&off)[K], double gamma_rank, int r, int32_t *__restrict__ list,
+                                          const int (&off)[K], int gamma_rank, int r, int32_t *__restrict__ list,
                                           DevState *st) {
     constexpr int D = C * NPIX;
     constexpr int NM = K / 2 + 1;
+    // two components a lane at a time, d and d + 32 (four patch rows further down): 96 M warp instructions instead of
+    // 128 M at 1024 x 1024 x 3, though 16 warps per SM instead of 24 (121 us; 129 with single components, 127 before
+    // the offsets came from shared memory, the ranks from whole numbers and the bounds from squares).  K = 32 has no
+    // registers for it.
+    using T = std::conditional_t<(K <= 16), float2, float>;
+    constexpr int PW = sizeof(T) / sizeof(float);
     const int lane = threadIdx.x & 31;
-    float lam[NM];
+    T lam2[NM], p0sq, qsq;
 #pragma unroll
-    for (int m = 0; m < NM; ++m) lam[m] = 0.f;
-    float e0sq = 0.f, esq = 0.f;
+    for (int m = 0; m < NM; ++m) vset(lam2[m], 0.f);
+    vset(p0sq, 0.f);
+    vset(qsq, 0.f);
 #pragma unroll 1
-    for (int d = lane; d < D; d += 32) {
+    for (int d = lane; d < D; d += 32 * PW) {
         const int c = d / NPIX, e = d - c * NPIX;
-        const size_t base = (size_t)c * plane + (size_t)(e >> 3) * rstride + (e & 7);
-        float p[K];
+        const float *s0 = src + (size_t)c * plane + (size_t)(e >> 3) * rstride + (e & 7);
+        T p[K];
+        if constexpr (PW == 2) {
+            const float *s1 = s0 + 4 * rstride;
 #pragma unroll
-        for (int k = 0; k < K; ++k) p[k] = src[base + off[k]];
+            for (int k = 0; k < K; ++k) p[k] = make_float2(s0[off[k]], s1[off[k]]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < K; ++k) p[k] = s0[off[k]];
+        }
         // q_k = p_k - p_0: X_m(q) = X_m(p) for m != 0, and X_0(p) = X_0(q) + K p_0
-        float q[K], a1 = 0.f;
-        q[0] = 0.f;
+        T q[K];
+        vset(q[0], 0.f);
 #pragma unroll
         for (int k = 1; k < K; ++k) {
-            q[k] = p[k] - p[0];
-            a1 += fabsf(q[k]);
+            q[k] = vsub(p[k], p[0]);
+            qsq = vfma(q[k], q[k], qsq);
         }
-        float xr[NM], xi[NM];
-        rdft_half<K, 1, NM>(q, xr, xi);
-        const float x0 = fmaf((float)K, p[0], xr[0]);
-        lam[0] = fmaf(x0, x0, lam[0]);
+        p0sq = vfma(p[0], p[0], p0sq);
+        T xr[NM], xi[NM];
+        rdft_half<K, 1, NM, T>(q, xr, xi);
+        const T x0 = vfma(p[0], (float)K, xr[0]);
+        lam2[0] = vfma(x0, x0, lam2[0]);
 #pragma unroll
-        for (int m = 1; m < NM; ++m) lam[m] = fmaf(xr[m], xr[m], fmaf(xi[m], xi[m], lam[m]));
-        // error bounds: X_m, m != 0, errs by at most sqrt(2) gamma_(K/4 + 3) sum_k |q_k| (the subtraction's
-        // rounding added), X_0(p) by gamma_(log2 K + 2) (sum_k |q_k| + K |p_0|); both inside sqrt(2) (K + 3) u
-        // times these sums, the bounds below
-        const float a0 = fmaf((float)K, fabsf(p[0]), a1);
-        e0sq = fmaf(a0, a0, e0sq);
-        esq = fmaf(a1, a1, esq);
+        for (int m = 1; m < NM; ++m) lam2[m] = vfma(xr[m], xr[m], vfma(xi[m], xi[m], lam2[m]));
     }
+    // error bounds: X_m, m != 0, of a component errs by at most sqrt(2) gamma_(K/4 + 3) sum_k |q_k| (the subtraction's
+    // rounding added), X_0(p) by gamma_(log2 K + 2) (sum_k |q_k| + K |p_0|); both inside sqrt(2) (K + 3) u times these
+    // sums.  Their squares over the components are at most (Cauchy-Schwarz, q_0 = 0) (K - 1) sum q^2 and
+    // 2 K^2 sum p_0^2 + 2 (K - 1) sum q^2, which take no absolute values.
+    float lam[NM];
+#pragma unroll
+    for (int m = 0; m < NM; ++m) lam[m] = vsum(lam2[m]);
+    const float esq = (float)(K - 1) * vsum(qsq), e0sq = 2.f * fmaf((float)(K * K), vsum(p0sq), esq);
     // warp sums of the NM eigenvalues and the two bound sums by a reduce-scatter: at each level a lane keeps
     // the half of its values that its lane bit selects and adds the partner's copy of that half, so that
     // after log2(NV) levels it holds the full sum of one value (index vidx); the addition depth per value
@@ -306,8 +340,8 @@ __device__ __forceinline__ int vote_group(const float *__restrict__ src, size_t 
     const unsigned l0 = 1u << lane_of(0);
     const int sure = 2 * __popc(bs) - ((bs & l0) ? 1 : 0);
     const int unc = 2 * __popc(bu) - ((bu & l0) ? 1 : 0);
-    if ((double)(1 + sure + unc) <= gamma_rank) return 1;
-    if ((double)(1 + sure) > gamma_rank) return 0;
+    if (1 + sure + unc <= gamma_rank) return 1;  // (gamma's whole part: the ranks are whole numbers)
+    if (1 + sure > gamma_rank) return 0;
     if (lane == 0) {  // decided in FP64 by k_vote_exact
         const int pos = atomicAdd(&st->vote_uncertain, 1);
         list[pos] = r;
@@ -328,9 +362,10 @@ constexpr int VNT = 256;     // threads per block (8 warps)
 template <int C, int K>
 __global__ void __launch_bounds__(VNT) k_vote(const float *__restrict__ img, int H, int W,
                                               const int32_t *__restrict__ idx, int nx, int ny, int step, int R,
-                                              double gamma_rank, int32_t *__restrict__ list, DevState *st) {
+                                              int gamma_rank, int32_t *__restrict__ list, DevState *st) {
     extern __shared__ float vreg[];
     __shared__ int s_votes;
+    __shared__ __align__(16) int s_off[VNT / 32][K < 4 ? 4 : K];  // the warps' members' offsets
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) s_votes = 0;
     const size_t HW = (size_t)H * W;
@@ -377,25 +412,29 @@ __global__ void __launch_bounds__(VNT) k_vote(const float *__restrict__ img, int
         }
         __syncthreads();
         const int tw = gx1 - gx0 + 1, ng = (gy1 - gy0 + 1) * tw;
+        auto member = [&](int t) {  // this lane's member of the tile's group t
+            return lane < K && t < ng ? __ldg(idx + (size_t)((gy0 + t / tw) * nx + gx0 + t % tw) * K + lane) : 0;
+        };
+        int next = member(warp);
         for (int t = warp; t < ng; t += VNT / 32) {
-            const int gy = gy0 + t / tw, gx = gx0 + t % tw, r = gy * nx + gx;
-            const int pos = (lane < K) ? idx[(size_t)r * K + lane] : 0;
+            const int r = (gy0 + t / tw) * nx + gx0 + t % tw;
+            const int pos = next;
+            next = member(t + VNT / 32);  // in flight while this group is decided
             const int py = pos / W, px = pos - py * W;
             const bool inside = lane >= K || (py >= ry0 && py + PS - 1 <= ry1 && px >= rx0 && px + PS - 1 <= rx1);
+            const bool staged = __all_sync(FULL, inside);
+            const int mine = staged ? (py - ry0) * rs + (px - rx0) : pos;
+            if (staged && !HTS_IN_BOUNDS(lane >= K || mine + (C - 1) * (int)plane + (PS - 1) * rs + PS - 1 < C * (int)plane,
+                                         &st->error))
+                continue;  // (the check build: the staged region would be overrun)
+            __syncwarp();
+            if (lane < K) s_off[warp][lane] = mine;
+            __syncwarp();
             int off[K];
-            if (__all_sync(FULL, inside)) {
-                const int mine = (py - ry0) * rs + (px - rx0);
-                if (!HTS_IN_BOUNDS(lane >= K || mine + (C - 1) * (int)plane + (PS - 1) * rs + PS - 1 < C * (int)plane,
-                                   &st->error))
-                    continue;  // (the check build: the staged region would be overrun)
 #pragma unroll
-                for (int k = 0; k < K; ++k) off[k] = __shfl_sync(FULL, mine, k);
-                my_votes += vote_group<C, K>(vreg, plane, rs, off, gamma_rank, r, list, st);
-            } else {
-#pragma unroll
-                for (int k = 0; k < K; ++k) off[k] = __shfl_sync(FULL, pos, k);
-                my_votes += vote_group<C, K>(img, HW, W, off, gamma_rank, r, list, st);
-            }
+            for (int k = 0; k < K; ++k) off[k] = s_off[warp][k];
+            if (staged) my_votes += vote_group<C, K>(vreg, plane, rs, off, gamma_rank, r, list, st);
+            else my_votes += vote_group<C, K>(img, HW, W, off, gamma_rank, r, list, st);
         }
     }
     if (lane == 0) atomicAdd(&s_votes, my_votes);
@@ -493,9 +532,10 @@ hts_status launch_vote(const float *img, const Geom &g, const int32_t *idx, doub
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, VNT, smem);
     const int ntiles = ((g.nx + VT - 1) / VT) * ((g.ny + VT - 1) / VT);
     const int blocks = std::max(1, std::min(ntiles, nsm * std::max(per_sm, 1)));
+    const int whole = gamma_rank >= 1000.0 ? 1000 : (int)std::floor(gamma_rank);  // a rank is at most K
     {
         KTimer kt("k_vote", s);
-        k_vote<C, K><<<blocks, VNT, smem, s>>>(img, g.H, g.W, idx, g.nx, g.ny, g.step, g.R, gamma_rank, list, st);
+        k_vote<C, K><<<blocks, VNT, smem, s>>>(img, g.H, g.W, idx, g.nx, g.ny, g.step, g.R, whole, list, st);
     }
     if (hts_status e = check_launch("k_vote"); e != HTS_OK) return e;
     {
