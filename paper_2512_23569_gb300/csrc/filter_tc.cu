@@ -115,9 +115,9 @@ __device__ __forceinline__ int a_off(int r, int k) {
 }
 
 // Row stride (elements) of the tile's staged region (FP16) and shared sums (int32): the region width rounded
-// up to 8 mod 64.  A warp reads or adds to 4 rows x 8 pixels of one patch: in the region four 16-byte row
-// pieces whose starts are 16 B apart modulo the banks' 128 bytes, in the sums four 32-byte row pieces 32 B
-// apart: distinct banks.
+// up to 8 mod 64.  A warp reads or adds to 4 rows x 8 pixels of one patch: in the region four 64-byte (gray
+// 16-byte) row pieces whose starts are 64 (16) B apart modulo the banks' 128 bytes, in the sums four 32-byte row
+// pieces 32 B apart: no two of the lanes served together meet in a bank.
 __host__ __device__ constexpr int acc_stride(int rw) { return rw + ((8 - rw) & 63); }
 
 // Fixed-point value * 2^8 rounded to the nearest integer (ties to even), as __float2int_rn(v * 256), for the
@@ -141,17 +141,20 @@ struct FtcLayout {
     static constexpr size_t a_off = 0;
     static constexpr size_t t_off = a_off + a_bytes;  // the transposed FP32 buffer [64][TS] of one slice
     static constexpr size_t b_off = t_off + (size_t)64 * TS * 4;
-    static constexpr size_t basis_off = b_off + (size_t)B_HALVES * 2;  // 6 x 64 FP32
-    static constexpr size_t misc_off = basis_off + (size_t)6 * 64 * 4;
+    static constexpr size_t basis_off = t_off;  // 6 x 64 FP32, only while the transforms are built
+    static constexpr size_t misc_off = b_off + (size_t)B_HALVES * 2;
     // misc: tau[2][32] float, off[2][MB] int, 4 mbarrier words (forward; inverse of slice 1; inverse of
-    // slices 2-3), tensor-memory slot
+    // slices 2-3), tensor-memory slot, detail flags
     static constexpr size_t job_off = misc_off + (size_t)2 * 32 * 4 + 2 * MB * 4 + 32 + 16;
-    // then the tile's sums [C][RA] int32 (per slice) and its staged region [C][RA] FP16 (per channel; RA =
-    // rows x acc_stride(width))
+    // then the tile's sums [C][RA] int32 (per slice) and its staged region [RA] of PXH FP16 values a pixel (RA =
+    // rows x acc_stride(width)): R, G, B and a pad, so that a pixel is one 8-byte load; one value for gray
+    static constexpr int PXH = (C == 3) ? 4 : 1;
     static constexpr size_t acc_off = job_off + 256;
-    static constexpr size_t bytes(int rh, int rw) { return acc_off + (size_t)C * rh * acc_stride(rw) * 6; }
+    static constexpr size_t bytes(int rh, int rw) { return acc_off + (size_t)rh * acc_stride(rw) * (C * 4 + PXH * 2); }
     static constexpr uint32_t tcols = (C == 3) ? 256 : 64;
 };
+// a tile of one reference fits with the largest window (MAX_WIN)
+static_assert(FtcLayout<3>::bytes(MAX_WIN - 1 + PS, MAX_WIN - 1 + PS) <= 227 * 1024, "every window has a tile");
 
 struct FtcArgs {
     const float *img;
@@ -212,12 +215,13 @@ __global__ void __launch_bounds__(NT, 1) k_filter_tc(const __grid_constant__ Ftc
     int *sOff = reinterpret_cast<int *>(sTau + 64);  // [2][MB] members' patch origins in the tile region (-1: none)
     uint64_t *bar = reinterpret_cast<uint64_t *>(sOff + 2 * MB);  // [3], 8-byte aligned
     uint32_t *slot = reinterpret_cast<uint32_t *>(bar + 4);
+    unsigned *sDet = slot + 1;  // bit 2 g + (slice > 0): group g of the batch kept a Haar detail coefficient
     int *accs = reinterpret_cast<int *>(smem + L::acc_off);
     FtcArgs *sjob = reinterpret_cast<FtcArgs *>(smem + L::job_off);
     const FtcArgs &a = BATCH ? *sjob : a0;  // the current job's arguments
     const int RA = BATCH ? bt.rh_max * acc_stride(bt.rw_max) : a0.rh_max * acc_stride(a0.rw_max);
     int *acc_v = accs;                                         // [C][RA] the tile's sums of value * 2^8
-    __half *sReg = reinterpret_cast<__half *>(accs + C * RA);  // [C][RA] the tile's region, FP16
+    __half *sReg = reinterpret_cast<__half *>(accs + C * RA);  // [RA][PXH] the tile's region, FP16
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // ---- bases (row-major 8x8, element (r, c) at r * 8 + c) and the transform F of the current job
     auto build_f = [&]() {
@@ -388,37 +392,43 @@ __global__ void __launch_bounds__(NT, 1) k_filter_tc(const __grid_constant__ Ftc
         const int rh = ry1 - ry0 + 1, rw = rx1 - rx0 + 1, rwp = acc_stride(rw);
         const int RP = rh * rwp;  // elements per channel plane of the region and of the sums
         for (int e = tid; e < C * RP; e += NT) acc_v[e] = 0;
-        // the tile's region, FP16: row y of channel c at (c * rh + y) * rwp; consecutive threads take consecutive
-        // pixels of a row, eight loads in flight per thread
+        // the tile's region, FP16: pixel (y, x) at y * rwp + x; consecutive threads take consecutive pixels of a row,
+        // eight loads in flight per thread (colour: twelve)
         {
-            // element e = tid + i NT: column x, region row `row` = channel c, row y; advanced by NT per step
+            constexpr int UN = (C == 3) ? 4 : 8;
+            // pixel e = tid + i NT at row y, column x; advanced by NT per step
             const int dq = NT / rw, dr = NT - dq * rw;
-            int row = tid / rw, x = tid - row * rw;
-            int c = row / rh, y = row - c * rh;
-            for (int e0 = 0; e0 < C * rh * rw; e0 += 8 * NT) {
-                float v[8];
-                int d[8];
+            int y = tid / rw, x = tid - y * rw;
+            for (int e0 = tid; e0 < rh * rw; e0 += UN * NT) {
+                float v[UN][C];
+                int d[UN];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const bool in = c < C;
-                    d[i] = in ? row * rwp + x : -1;
-                    v[i] = in ? __ldg(a.img + c * HW + (size_t)(ry0 + y) * a.W + rx0 + x) : 0.f;
+                for (int i = 0; i < UN; ++i) {
+                    const bool in = y < rh;
+                    d[i] = in ? y * rwp + x : -1;
+                    const float *src = a.img + (in ? (size_t)(ry0 + y) * a.W + rx0 + x : 0);
+#pragma unroll
+                    for (int c = 0; c < C; ++c) v[i][c] = in ? __ldg(src + c * HW) : 0.f;
                     x += dr;
-                    row += dq;
                     y += dq;
                     if (x >= rw) {
                         x -= rw;
-                        ++row;
                         ++y;
-                    }
-                    while (y >= rh) {
-                        y -= rh;
-                        ++c;
                     }
                 }
 #pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    if (d[i] >= 0) sReg[d[i]] = __float2half_rn(v[i]);
+                for (int i = 0; i < UN; ++i)
+                    if (d[i] >= 0) {
+                        if constexpr (C == 3) {
+                            const __half2 rg = __floats2half2_rn(v[i][0], v[i][1]), b0 = __floats2half2_rn(v[i][2], 0.f);
+                            uint2 w;
+                            w.x = *reinterpret_cast<const uint32_t *>(&rg);
+                            w.y = *reinterpret_cast<const uint32_t *>(&b0);
+                            reinterpret_cast<uint2 *>(sReg)[d[i]] = w;
+                        } else {
+                            sReg[d[i]] = __float2half_rn(v[i][0]);
+                        }
+                    }
             }
         }
         // the block's next tile's region into L2 while this tile runs (its staging then reads L2, not HBM):
@@ -484,14 +494,21 @@ __global__ void __launch_bounds__(NT, 1) k_filter_tc(const __grid_constant__ Ftc
                 int g, p, h;
                 slot_of(i, g, p, h);
                 const int *offs = sOff + MB * buf + g * K + h * KM;
-                const __half *src = sReg + (p >> 3) * rwp + (p & 7);
+                const __half *src = sReg + L::PXH * ((p >> 3) * rwp + (p & 7));
                 float v[KM][C];
 #pragma unroll
                 for (int j = 0; j < KM; ++j) {
                     const int o = offs[j];
                     const bool in = o >= 0 && HTS_IN_BOUNDS(o + (p >> 3) * rwp + (p & 7) < RP, &a.st->error);
-#pragma unroll
-                    for (int c = 0; c < C; ++c) v[j][c] = in ? __half2float(src[c * RP + o]) : 0.f;
+                    if constexpr (C == 3) {
+                        const uint2 w = in ? *reinterpret_cast<const uint2 *>(src + 4 * o) : make_uint2(0u, 0u);
+                        const float2 rg = __half22float2(*reinterpret_cast<const __half2 *>(&w.x));
+                        v[j][0] = rg.x;
+                        v[j][1] = rg.y;
+                        v[j][2] = __low2float(*reinterpret_cast<const __half2 *>(&w.y));
+                    } else {
+                        v[j][0] = in ? __half2float(src[o]) : 0.f;
+                    }
                 }
                 if constexpr (C == 3) {  // the channel DFT (Eq. 4-5), real orthonormal form: v[j][s] = slice value s
 #pragma unroll
@@ -538,6 +555,7 @@ __global__ void __launch_bounds__(NT, 1) k_filter_tc(const __grid_constant__ Ftc
         for (int b = 0; b < nbatch; ++b) {
             const int cur = b & 1;
             const float *bTau = sTau + 32 * cur;
+            if (tid == 0) *sDet = 0u;  // read last before the previous batch's last barrier
             commit(cur);
             if (b + 1 < nbatch) {  // the next batch's thresholds and member offsets (read after the next barrier)
                 if (tid < GPB) sTau[32 * (cur ^ 1) + tid] = tau_from(sigreg, svalid);
@@ -564,16 +582,21 @@ __global__ void __launch_bounds__(NT, 1) k_filter_tc(const __grid_constant__ Ftc
                 const float t2 = tau * tau * (float)(1 << l);
                 const float sc = (ra && k == 0) ? 0.f : __int_as_float((127 - l) << 23);  // 2^-l; RA: row 0 replaced
                 unsigned char *rowp = sA + (m >> 3) * SBO_A + ((m & 7) << 4);
+                unsigned det = 0u;  // kept a detail coefficient: slice 1, slices 2-3
                 {
                     uint32_t v[16];
                     tc::tmem_ld16(tbase + tlane + (uint32_t)(16 * wq), v);
                     tc::tmem_wait_ld();
                     __align__(16) __half2 hv[8];
+                    bool any = false;
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
                         const float x0 = __uint_as_float(v[2 * j]), x1 = __uint_as_float(v[2 * j + 1]);
-                        hv[j] = __floats2half2_rn(x0 * x0 >= t2 ? x0 * sc : 0.f, x1 * x1 >= t2 ? x1 * sc : 0.f);
+                        const bool k0 = x0 * x0 >= t2, k1 = x1 * x1 >= t2;
+                        any = any || k0 || k1;
+                        hv[j] = __floats2half2_rn(k0 ? x0 * sc : 0.f, k1 ? x1 * sc : 0.f);
                     }
+                    if (any && k > 0) det = 1u << (2 * (m / K));
                     const uint4 *hp = reinterpret_cast<const uint4 *>(hv);
                     *reinterpret_cast<uint4 *>(rowp + (2 * wq) * LBO_A) = hp[0];
                     *reinterpret_cast<uint4 *>(rowp + (2 * wq + 1) * LBO_A) = hp[1];
@@ -585,6 +608,7 @@ __global__ void __launch_bounds__(NT, 1) k_filter_tc(const __grid_constant__ Ftc
                     tc::tmem_wait_ld();
                     const float t2c = 2.f * t2;
                     __align__(16) __half2 hr[8], hi[8];
+                    bool any = false;
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
                         float o[2][2];
@@ -592,12 +616,14 @@ __global__ void __launch_bounds__(NT, 1) k_filter_tc(const __grid_constant__ Ftc
                         for (int e = 0; e < 2; ++e) {
                             const float re = __uint_as_float(vr[2 * j + e]), im = __uint_as_float(vi[2 * j + e]);
                             const bool keep = fmaf(re, re, im * im) >= t2c;
+                            any = any || keep;
                             o[0][e] = keep ? re * sc : 0.f;
                             o[1][e] = keep ? im * sc : 0.f;
                         }
                         hr[j] = __floats2half2_rn(o[0][0], o[0][1]);
                         hi[j] = __floats2half2_rn(o[1][0], o[1][1]);
                     }
+                    if (any && k > 0) det |= 2u << (2 * (m / K));
                     const uint4 *rp = reinterpret_cast<const uint4 *>(hr);
                     const uint4 *ip = reinterpret_cast<const uint4 *>(hi);
                     *reinterpret_cast<uint4 *>(rowp + BLK_A + (2 * wq) * LBO_A) = rp[0];
@@ -605,6 +631,8 @@ __global__ void __launch_bounds__(NT, 1) k_filter_tc(const __grid_constant__ Ftc
                     *reinterpret_cast<uint4 *>(rowp + 2 * BLK_A + (2 * wq) * LBO_A) = ip[0];
                     *reinterpret_cast<uint4 *>(rowp + 2 * BLK_A + (2 * wq + 1) * LBO_A) = ip[1];
                 }
+                det = __reduce_or_sync(0xffffffffu, det);
+                if (lane == 0 && det) atomicOr(sDet, det);
             }
             // ---- inverse transform (Eq. 21): E[row] = the slices' values of the group's thresholded Haar rows,
             //      slice 1 first (its own commit), so that its aggregation overlaps the rest
@@ -641,6 +669,39 @@ __global__ void __launch_bounds__(NT, 1) k_filter_tc(const __grid_constant__ Ftc
                     int g, p, h;
                     slot_of(i, g, p, h);
                     const float *colp = sT + p * TS + g * K;
+                    float mu = 0.f;  // first Haar row replaced (Eq. 24-25): the refined mean joins every member
+                    if (ra) {
+                        const int lg = b * GPB + g;
+                        const int gy = gy0 + lg / a.tx, gx = gx0 + lg % a.tx;
+                        if (lg < gpt && gy <= gy1 && gx <= gx1) {
+                            const float *mp = a.mean_est + (size_t)(gy * a.nx + gx) * (C * 64) + p;
+                            // slice c of the refined mean's pixel p
+                            if (C == 1) {
+                                mu = __ldg(mp);
+                            } else {
+                                const float r = __ldg(mp), gg = __ldg(mp + 64), bl = __ldg(mp + 128);
+                                mu = c == 0 ? K3F * (r + (gg + bl)) : c == 1 ? K23F * fmaf(-0.5f, gg + bl, r) : K12F * (bl - gg);
+                            }
+                        }
+                    }
+                    int *dst = acc_v + c * RP;
+                    // No detail coefficient of the group's slice was kept (the rule where the members match to within
+                    // the noise): the butterflies would add zeros, and every member gets the first row's value.  A
+                    // warp holds one group, so it takes this way as a whole.  (With the region's 8-byte pixels 20 % of
+                    // the warp instructions: 3840 x 2160 x 3, sigma 2 to 28: 3190 -> 2870 us; 1021 x 771 x 3, sigma
+                    // 30: 372 -> 335.  Barriers between the phases, 16 warps per SM in step, bind it now.)
+                    if (!(*sDet >> (2 * g + (c > 0 ? 1 : 0)) & 1u)) {
+                        float x0 = colp[0];
+                        if (ra) x0 += mu;
+                        const int fx = fix8(x0);
+                        if (fx != 0) {  // (chroma slices thresholded away)
+#pragma unroll
+                            for (int j = 0; j < KM; ++j)
+                                if (offs[i][j] >= 0 && HTS_IN_BOUNDS(offs[i][j] < RP, &a.st->error))
+                                    atomicAdd(dst + offs[i][j], fx);
+                        }
+                        continue;
+                    }
                     float x[KM];
                     if (TPP == 1) {
 #pragma unroll
@@ -668,23 +729,10 @@ __global__ void __launch_bounds__(NT, 1) k_filter_tc(const __grid_constant__ Ftc
                         }
                     }
                     haar_inv_u<KM>(x);
-                    if (ra) {  // first Haar row replaced (Eq. 24-25): the refined mean joins every member
-                        const int lg = b * GPB + g;
-                        const int gy = gy0 + lg / a.tx, gx = gx0 + lg % a.tx;
-                        if (lg < gpt && gy <= gy1 && gx <= gx1) {
-                            const float *mp = a.mean_est + (size_t)(gy * a.nx + gx) * (C * 64) + p;
-                            float mu;  // slice c of the refined mean's pixel p
-                            if (C == 1) {
-                                mu = __ldg(mp);
-                            } else {
-                                const float r = __ldg(mp), gg = __ldg(mp + 64), bl = __ldg(mp + 128);
-                                mu = c == 0 ? K3F * (r + (gg + bl)) : c == 1 ? K23F * fmaf(-0.5f, gg + bl, r) : K12F * (bl - gg);
-                            }
+                    if (ra) {
 #pragma unroll
-                            for (int j = 0; j < KM; ++j) x[j] += mu;
-                        }
+                        for (int j = 0; j < KM; ++j) x[j] += mu;
                     }
-                    int *dst = acc_v + c * RP;
 #pragma unroll
                     for (int j = 0; j < KM; ++j)
                         if (offs[i][j] >= 0 && HTS_IN_BOUNDS(offs[i][j] < RP, &a.st->error))
