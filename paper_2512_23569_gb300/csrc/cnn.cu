@@ -39,6 +39,7 @@
 
 #include "cnn_internal.h"
 #include "hts_internal.h"
+#include "tc_ptx.h"
 
 namespace hts {
 namespace {
@@ -204,6 +205,8 @@ __global__ void __launch_bounds__(256) k_loss(const float *__restrict__ outm, in
     __shared__ bool last;
     const int nref = nx * ny;
     double s = 0.0;
+    tc::grid_wait();
+    tc::grid_launch();
     for (int y = blockIdx.x; y < H; y += gridDim.x) {
         const int py = y - PS / 2;
         const bool row = py >= 0 && py <= H - PS && (py % step == 0 || py == H - PS);
@@ -362,11 +365,8 @@ __global__ void k_learned_final(int nref, double factor, DevState *st) {
 
 hts_status cnn_loss(hts_cnn *n, const float *map, int H, int W, const Geom &g, const float *target, float *dout,
                     cudaStream_t s) {
-    {
-        KTimer kt("k_loss", s);
-        k_loss<<<std::min(H, LOSS_BLOCKS), 256, 0, s>>>(map, H, W, g.step, g.nx, g.ny, target, dout, n->lpart, n->loss);
-    }
-    return check_launch("k_loss");
+    return launch_chained("k_loss", k_loss, dim3(std::min(H, LOSS_BLOCKS)), 256, 0, s, map, H, W, g.step, g.nx, g.ny,
+                          target, dout, n->lpart, n->loss);
 }
 
 namespace {

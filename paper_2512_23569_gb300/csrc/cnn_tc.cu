@@ -4,7 +4,7 @@
 //
 // A 3x3 convolution with zero padding is an implicit GEMM: for every tap
 // (ky, kx), out[p][n] += sum_c in[p + (ky - 1, kx - 1)][c] w[n][c][ky][kx].
-// A block takes a strip of 16 x 64 output pixels and stages its input with a
+// A block takes a strip of 16 x 64 (16) output pixels and stages its input with a
 // one-pixel halo in shared memory as planes of 8 channels: entry (g, py, px)
 // is the 16-byte vector of channels 8g .. 8g + 7 of one pixel.  Eight 16 x 8
 // pixel tiles of the strip are the MMA's M = 128 rows (tile row i = 8
@@ -38,9 +38,8 @@ namespace hts {
 namespace {
 
 constexpr int SY = 16;                   // output rows of a strip
-constexpr int MT = 8;                    // 16 x 8 pixel tiles (MMA M = 128) per strip
-constexpr int SX = 8 * MT;               // output columns of a strip
-constexpr int PY = SY + 2, PX = SX + 2;  // staged rows and columns (halo of one pixel)
+constexpr int PY = SY + 2;               // staged rows (halo of one pixel)
+constexpr int SX = 64, PX = SX + 2;      // output and staged columns of the weight gradient's strips
 constexpr int NTH = 256;                 // 8 warps; warp w reads tensor-memory lanes 32 (w % 4) .. + 31
 constexpr long long SPIN = 1ll << 22;
 // At least this much shared memory per block: at most two blocks per SM, so
@@ -93,8 +92,10 @@ __device__ __forceinline__ void epilogue_store(const uint32_t *r, const float *s
     }
 }
 
-template <int CING, int NOUT>
+// MT: 16 x 8 pixel tiles (MMA M = 128) per strip, side by side.
+template <int CING, int NOUT, int MT>
 struct ConvTcLayout {
+    static constexpr int SX = 8 * MT, PX = SX + 2;                  // output and staged columns of a strip
     static constexpr size_t a_bytes = (size_t)CING * PY * PX * 16;  // staged input planes
     static constexpr size_t b_off = a_bytes;
     static constexpr size_t b_bytes = (size_t)9 * CING * NOUT * 16;  // weights [tap][plane][n][8]
@@ -103,7 +104,7 @@ struct ConvTcLayout {
     static constexpr size_t slot_off = bar_off + 16;
     static constexpr size_t used = slot_off + 16;
     static constexpr size_t total = used > MIN_SMEM ? used : MIN_SMEM;
-    static constexpr uint32_t tcols = MT * NOUT;  // 256 or 128
+    static constexpr uint32_t tcols = MT * NOUT;  // 64 or 256
 };
 
 // CING: input planes of 8 channels (2 for layer 0, whose C <= 3 channels
@@ -111,12 +112,13 @@ struct ConvTcLayout {
 // IN_F32: the input is an FP32 planar C x H x W array (the image) times
 // in_scale (1/255); otherwise FP16 planes hin[g][y][x][8].  EPI: the
 // epilogue (EPI_RELU, EPI_MAP, EPI_MASK with the activation planes hmask).
-template <int CING, int NOUT, bool IN_F32, int EPI>
+template <int CING, int NOUT, int MT, bool IN_F32, int EPI>
 __global__ void __launch_bounds__(NTH, 2)
     k_conv_tc(const float *__restrict__ img, int C, float in_scale, const __half *__restrict__ hin, int H, int W,
               const __half *__restrict__ wp, const __half *__restrict__ wbias, int cout, __half *__restrict__ hout,
               float *__restrict__ map, const __half *__restrict__ hmask, int *err) {
-    using L = ConvTcLayout<CING, NOUT>;
+    using L = ConvTcLayout<CING, NOUT, MT>;
+    constexpr int SX = L::SX, PX = L::PX;
     extern __shared__ __align__(1024) unsigned char smem[];
     uint4 *sA = reinterpret_cast<uint4 *>(smem);
     __half *sB = reinterpret_cast<__half *>(smem + L::b_off);
@@ -125,12 +127,16 @@ __global__ void __launch_bounds__(NTH, 2)
     uint32_t *slot = reinterpret_cast<uint32_t *>(smem + L::slot_off);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-    stage_weights<CING, NOUT, EPI>(wp, wbias, cout, sB, sBias, tid);
+    // layer 0 may follow the kernel that wrote its weights; a backward pass follows the loss, which waited for it
+    if (EPI == EPI_MASK) stage_weights<CING, NOUT, EPI>(wp, wbias, cout, sB, sBias, tid);
     if (tid == 0) {
         tc::bar_init(bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
     if (warp == 0) tc::tmem_alloc(slot, L::tcols);
+    tc::grid_wait();
+    tc::grid_launch();
+    if (EPI != EPI_MASK) stage_weights<CING, NOUT, EPI>(wp, wbias, cout, sB, sBias, tid);
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
@@ -277,6 +283,8 @@ __global__ void __launch_bounds__(NTH, 2)
     }
     if (warp == 0) tc::tmem_alloc(slot, L::tcols);
     tc::fence_async_smem();
+    tc::grid_wait();  // (the weights above were written before the layer before this one started its own work)
+    tc::grid_launch();
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
@@ -375,22 +383,31 @@ __global__ void k_map_poison(float *map, size_t n, const int *err) {
 }
 
 // wp: the layer's packed weights (the network's, or the flipped ones of a backward pass).
-template <int CING, int NOUT, bool IN_F32, int EPI>
-hts_status conv_tc(const hts_cnn *n, const __half *wp, const __half *wbias, int cout, const float *img, int C, float in_scale,
-                   const __half *hin, int H, int W, __half *hout, float *map, const __half *hmask, int nsm,
-                   cudaStream_t s) {
-    using L = ConvTcLayout<CING, NOUT>;
-    const void *k = reinterpret_cast<const void *>(k_conv_tc<CING, NOUT, IN_F32, EPI>);
+template <int CING, int NOUT, int MT, bool IN_F32, int EPI>
+hts_status conv_tc_mt(const hts_cnn *n, const __half *wp, const __half *wbias, int cout, const float *img, int C,
+                      float in_scale, const __half *hin, int H, int W, __half *hout, float *map, const __half *hmask,
+                      int nsm, cudaStream_t s) {
+    using L = ConvTcLayout<CING, NOUT, MT>;
+    const void *k = reinterpret_cast<const void *>(k_conv_tc<CING, NOUT, MT, IN_F32, EPI>);
     const hts_status st = allow_smem(k, L::total);
     if (st != HTS_OK) return st;
-    const int nstrip = ((H + SY - 1) / SY) * ((W + SX - 1) / SX);
+    const int nstrip = ((H + SY - 1) / SY) * ((W + L::SX - 1) / L::SX);
     const int grid = std::max(1, std::min(nstrip, 2 * nsm));
-    {
-        KTimer kt("k_conv_tc", s);
-        k_conv_tc<CING, NOUT, IN_F32, EPI><<<grid, NTH, L::total, s>>>(img, C, in_scale, hin, H, W, wp, wbias, cout,
-                                                                      hout, map, hmask, n->err);
-    }
-    return check_launch("k_conv_tc");
+    return launch_chained("k_conv_tc", k_conv_tc<CING, NOUT, MT, IN_F32, EPI>, dim3(grid), NTH, L::total, s, img, C,
+                          in_scale, hin, H, W, wp, wbias, cout, hout, map, hmask, n->err);
+}
+
+// Strips of 64 columns (the least halo) where they fill the two blocks of every SM, else of 16: on a 256 x 256 crop 64
+// blocks of four times the work left most SMs idle (11.5 us a layer between events, now 9).
+template <int CING, int NOUT, bool IN_F32, int EPI>
+hts_status conv_tc(const hts_cnn *n, const __half *wp, const __half *wbias, int cout, const float *img, int C,
+                   float in_scale, const __half *hin, int H, int W, __half *hout, float *map, const __half *hmask,
+                   int nsm, cudaStream_t s) {
+    if (((H + SY - 1) / SY) * ((W + 63) / 64) >= 2 * nsm)
+        return conv_tc_mt<CING, NOUT, 8, IN_F32, EPI>(n, wp, wbias, cout, img, C, in_scale, hin, H, W, hout, map, hmask,
+                                                      nsm, s);
+    return conv_tc_mt<CING, NOUT, 2, IN_F32, EPI>(n, wp, wbias, cout, img, C, in_scale, hin, H, W, hout, map, hmask, nsm,
+                                                  s);
 }
 
 // A hidden layer with the TMA-staged input: the tensor map describes hin as [plane][y][x][8 halves], read
@@ -416,11 +433,8 @@ hts_status conv_tma(const hts_cnn *n, const __half *wp, const __half *wbias, int
     if (st != HTS_OK) return st;
     const int nstrip = ((H + SY - 1) / SY) * ((W + SXH - 1) / SXH);
     const int grid = std::max(1, std::min(nstrip, 2 * nsm));
-    {
-        KTimer kt("k_conv_tma", s);
-        k_conv_tma<NOUT, EPI><<<grid, NTH, L::total, s>>>(tmap, H, W, wp, wbias, cout, hout, map, hmask, n->err);
-    }
-    return check_launch("k_conv_tma");
+    return launch_chained("k_conv_tma", k_conv_tma<NOUT, EPI>, dim3(grid), NTH, L::total, s, tmap, H, W, wp, wbias, cout,
+                          hout, map, hmask, n->err);
 }
 
 // ------------------------------------------------------------------ training (backward) on the tensor cores
@@ -438,7 +452,7 @@ hts_status conv_tma(const hts_cnn *n, const __half *wp, const __half *wbias, int
 // Bound by latency at the training crops' size (128 strips a layer): staging, about 4 us of MMAs whose 4 KB A
 // operands come from shared memory, the read-back.  Three blocks per SM and the five layers side by side hide them:
 // 256 x 256 x 3, between events, 33 us for the layers together (before, a launch per layer with a copy of every tap
-// and a wait per strip row: 96 us); the reduction in one coalesced launch: 27 us (before 116).
+// and a wait per strip row: 96 us); the reduction in one coalesced launch: 17 us (before 116).
 constexpr int WSY = 8;            // strip rows
 constexpr int WPY = WSY + 2;      // staged X rows
 constexpr int WCH = SX;           // strip columns
@@ -491,6 +505,8 @@ __global__ void __launch_bounds__(NTH, 3) k_conv_wgrad(const __grid_constant__ W
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
     if (warp == 0) tc::tmem_alloc(slot, L::tcols);
+    tc::grid_wait();
+    tc::grid_launch();
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
@@ -600,6 +616,8 @@ __global__ void __launch_bounds__(NTH, 3) k_conv_wgrad(const __grid_constant__ W
 __global__ void __launch_bounds__(256) k_wgrad_reduce(const __grid_constant__ WgradArgs a) {
     const WgLayer &l = a.l[blockIdx.y];
     const int N = 8 * l.nply, j = blockIdx.x * 256 + threadIdx.x;
+    tc::grid_wait();
+    tc::grid_launch();
     if (j >= l.rows * N) return;
     const int row = j / N, co = j - row * N, cp = 8 * l.cinx, tap = row / cp, ci = row - tap * cp;
     const bool bias = row == l.rows - 1;
@@ -607,8 +625,14 @@ __global__ void __launch_bounds__(256) k_wgrad_reduce(const __grid_constant__ Wg
     const float *p = a.part + l.part + j;
     const size_t stride = (size_t)l.rows * N;
     float s = 0.f;
-#pragma unroll 16
-    for (int b = 0; b < a.nblk; ++b) s += p[b * stride];
+    for (int b0 = 0; b0 < a.nblk; b0 += 32) {  // 32 loads in flight, added in block order
+        float v[32];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) v[i] = b0 + i < a.nblk ? __ldg(p + (size_t)(b0 + i) * stride) : 0.f;
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+            if (b0 + i < a.nblk) s += v[i];
+    }
     float *g = l.grad + (bias ? l.cout * l.cin * 9 + co : (co * l.cin + ci) * 9 + tap);
     *g = *a.err ? __int_as_float(0x7fc00000) : *g + s * (1.f / a.y_scale);
 }
@@ -648,17 +672,9 @@ hts_status conv_wgrad(hts_cnn *n, const float *img, __half *const *act, const fl
     }
     hts_status st = allow_smem(reinterpret_cast<const void *>(k_conv_wgrad), WgradLayout::total);
     if (st != HTS_OK) return st;
-    {
-        KTimer kt("k_conv_wgrad", s);
-        k_conv_wgrad<<<dim3(a.nblk, NWG), NTH, WgradLayout::total, s>>>(a);
-    }
-    st = check_launch("k_conv_wgrad");
+    st = launch_chained("k_conv_wgrad", k_conv_wgrad, dim3(a.nblk, NWG), NTH, WgradLayout::total, s, a);
     if (st != HTS_OK) return st;
-    {
-        KTimer kt("k_wgrad_reduce", s);
-        k_wgrad_reduce<<<dim3((most + 255) / 256, NWG), 256, 0, s>>>(a);
-    }
-    return check_launch("k_wgrad_reduce");
+    return launch_chained("k_wgrad_reduce", k_wgrad_reduce, dim3((most + 255) / 256, NWG), 256, 0, s, a);
 }
 
 }  // namespace
