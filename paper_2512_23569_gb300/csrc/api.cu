@@ -475,9 +475,8 @@ hts_status denoise_run(const float *noisy, float *out, const Geom &g, float sigm
     if (sigma_ref && fallback_factor > 0) HTS_TRY(launch_learned_check(sigma_ref, g.nref, fallback_factor, w->st, s));
     float *mean_est = nullptr;
     if (fcn) {  // enhancement strategy: refined mean patch of every group (Eq. 24-25)
-        float *means = ra_buf, *refined = ra_buf + (size_t)g.nref * g.C * 64;
-        HTS_TRY(launch_group_means(noisy, g, w->idx, means, s));
-        HTS_TRY(fcn_refine_state(fcn, means, g.nref, w->st, b32, refined, s));
+        float *coords = ra_buf, *refined = ra_buf + (size_t)g.nref * g.C * 64;
+        HTS_TRY(fcn_refine_groups(fcn, noisy, g, w->idx, w->st, b32, coords, refined, s));
         mean_est = refined;
     }
     return launch_filter(noisy, g, w->idx, b64, b32, w->acc, w->wcount, w->redo, w->xlist, w->xskip, w->st, out,

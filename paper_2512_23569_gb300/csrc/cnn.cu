@@ -39,7 +39,6 @@
 
 #include "cnn_internal.h"
 #include "hts_internal.h"
-#include "tc_ptx.h"
 
 namespace hts {
 namespace {
@@ -205,8 +204,8 @@ __global__ void __launch_bounds__(256) k_loss(const float *__restrict__ outm, in
     __shared__ bool last;
     const int nref = nx * ny;
     double s = 0.0;
-    tc::grid_wait();
-    tc::grid_launch();
+    grid_wait();
+    grid_launch();
     for (int y = blockIdx.x; y < H; y += gridDim.x) {
         const int py = y - PS / 2;
         const bool row = py >= 0 && py <= H - PS && (py % step == 0 || py == H - PS);

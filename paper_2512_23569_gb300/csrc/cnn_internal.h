@@ -57,29 +57,6 @@ struct Geom;
 hts_status cnn_loss(hts_cnn *net, const float *map, int H, int W, const Geom &g, const float *target, float *dout,
                     cudaStream_t s);
 constexpr int LOSS_BLOCKS = 304;
-
-// Launches a kernel of the network's chains, overlapping the kernel before it on the stream (tc::grid_wait /
-// tc::grid_launch in the kernel) except inside a stream capture.  A layer of a 256 x 256 crop runs for 4 us, and its
-// launch, barrier and tensor-memory set-up and weights would follow the layer before one after the other.
-template <typename... P, typename... A>
-hts_status launch_chained(const char *name, void (*k)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s,
-                          A &&...args) {
-    {
-        KTimer kt(name, s);
-        cudaLaunchAttribute attr{};
-        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr.val.programmaticStreamSerializationAllowed = 1;
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = grid;
-        cfg.blockDim = dim3(threads);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = s;
-        cfg.attrs = &attr;
-        cfg.numAttrs = stream_capturing(s) ? 0 : 1;
-        cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);  // its error is check_launch's
-    }
-    return check_launch(name);
-}
 // One image's loss and gradient (added to net->grad) on the tensor cores: FP16 activations and input
 // gradients (loss scale 2^(floor(log2 N_ref) + 2)), FP32 accumulation of the weight gradients.
 hts_status cnn_grad_tc(hts_cnn *net, const float *img, int H, int W, const Geom &g, const float *target,

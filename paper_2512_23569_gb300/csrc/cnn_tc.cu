@@ -134,8 +134,8 @@ __global__ void __launch_bounds__(NTH, 2)
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
     if (warp == 0) tc::tmem_alloc(slot, L::tcols);
-    tc::grid_wait();
-    tc::grid_launch();
+    grid_wait();
+    grid_launch();
     if (EPI != EPI_MASK) stage_weights<CING, NOUT, EPI>(wp, wbias, cout, sB, sBias, tid);
     tc::fence_before();
     __syncthreads();
@@ -283,8 +283,8 @@ __global__ void __launch_bounds__(NTH, 2)
     }
     if (warp == 0) tc::tmem_alloc(slot, L::tcols);
     tc::fence_async_smem();
-    tc::grid_wait();  // (the weights above were written before the layer before this one started its own work)
-    tc::grid_launch();
+    grid_wait();  // (the weights above were written before the layer before this one started its own work)
+    grid_launch();
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
@@ -505,8 +505,8 @@ __global__ void __launch_bounds__(NTH, 3) k_conv_wgrad(const __grid_constant__ W
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
     if (warp == 0) tc::tmem_alloc(slot, L::tcols);
-    tc::grid_wait();
-    tc::grid_launch();
+    grid_wait();
+    grid_launch();
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
@@ -616,8 +616,8 @@ __global__ void __launch_bounds__(NTH, 3) k_conv_wgrad(const __grid_constant__ W
 __global__ void __launch_bounds__(256) k_wgrad_reduce(const __grid_constant__ WgradArgs a) {
     const WgLayer &l = a.l[blockIdx.y];
     const int N = 8 * l.nply, j = blockIdx.x * 256 + threadIdx.x;
-    tc::grid_wait();
-    tc::grid_launch();
+    grid_wait();
+    grid_launch();
     if (j >= l.rows * N) return;
     const int row = j / N, co = j - row * N, cp = 8 * l.cinx, tap = row / cp, ci = row - tap * cp;
     const bool bias = row == l.rows - 1;

@@ -14,9 +14,9 @@
 // reduce over the batch with a split of the reduction and a fixed-order sum
 // of the parts, so training is deterministic.
 //
-// Denoising (hts_denoise_ra): the mean patch of every group (k_group_means),
-// its coordinates, the network with the call's estimated sigma, the refined
-// patch back in pixels (k_coefs_to_patch), and the refined patches go to the
+// Denoising (hts_denoise_ra): the mean patch of every group, its coordinates
+// and features with the call's estimated sigma (k_group_features), the network,
+// the refined patch back in pixels (k_refined_patch), and the refined patches go to the
 // tensor-core filter, which drops each group's first Haar row and
 // adds the refined mean to every member's estimate instead (the same as
 // replacing that row by sqrt(K) times the refined mean's transform and not
@@ -56,7 +56,6 @@ struct hts_fcn {
     size_t cap_part = 0;
     float *part = nullptr;                // split-reduction parts, each a parameter vector
     double *loss = nullptr;               // accumulated loss
-    float *sig = nullptr;                 // the call's sigma for the features (denoising)
 };
 
 namespace hts {
@@ -320,9 +319,6 @@ __global__ void k_features(const float *__restrict__ coords, const float *__rest
     }
 }
 
-// sigma of the call (double in the state) as a float for the features.
-__global__ void k_state_sigma(const DevState *st, float *out) { *out = (float)st->sigma_hat; }
-
 __global__ void k_fcn_adam(float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
                            float *__restrict__ v, int n, float lr, float c1, float c2) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -368,128 +364,221 @@ __device__ void canon_column(float *re, float *im, int c) {
 
 // Basis slices of the FP32 device copy ([j][U/V][8][8][re/im]) in shared memory, columns in the
 // canonical phase (canon_column).
+struct MeanBasis {
+    float u0[64], v0[64], u1r[64], u1i[64], v1r[64], v1i[64];
+};
 template <int C>
-__device__ void load_bases(const float *__restrict__ b32, float (&u0)[64], float (&v0)[64], float (&u1r)[64],
-                           float (&u1i)[64], float (&v1r)[64], float (&v1i)[64]) {
+__device__ void load_bases(const float *__restrict__ b32, MeanBasis &b) {
     const int t = threadIdx.x;
-    u0[t] = b32[(0 * 64 + t) * 2];
-    v0[t] = b32[(1 * 64 + t) * 2];
-    if (C == 3) {
-        u1r[t] = b32[(2 * 64 + t) * 2];
-        u1i[t] = b32[(2 * 64 + t) * 2 + 1];
-        v1r[t] = b32[(3 * 64 + t) * 2];
-        v1i[t] = b32[(3 * 64 + t) * 2 + 1];
+    if (t < 64) {
+        b.u0[t] = b32[(0 * 64 + t) * 2];
+        b.v0[t] = b32[(1 * 64 + t) * 2];
+        if (C == 3) {
+            b.u1r[t] = b32[(2 * 64 + t) * 2];
+            b.u1i[t] = b32[(2 * 64 + t) * 2 + 1];
+            b.v1r[t] = b32[(3 * 64 + t) * 2];
+            b.v1i[t] = b32[(3 * 64 + t) * 2 + 1];
+        }
     }
     __syncthreads();
-    if (t < 8) canon_column(u0, nullptr, t);
-    else if (t < 16) canon_column(v0, nullptr, t - 8);
-    else if (C == 3 && t < 24) canon_column(u1r, u1i, t - 16);
-    else if (C == 3 && t < 32) canon_column(v1r, v1i, t - 24);
+    if (t < 8) canon_column(b.u0, nullptr, t);
+    else if (t < 16) canon_column(b.v0, nullptr, t - 8);
+    else if (C == 3 && t < 24) canon_column(b.u1r, b.u1i, t - 16);
+    else if (C == 3 && t < 32) canon_column(b.v1r, b.v1i, t - 24);
+    __syncthreads();
 }
 
-// Coordinates of patch r (one block of 64 threads per patch, thread = pixel / coefficient (a, b)):
-// the DFT along the channels, T = Phat V, S = U^H T (Eq. 19 without the Haar factor); out
-// [S^(1) | sqrt 2 Re S^(2) | sqrt 2 Im S^(2)] (orthonormal).
+// The transforms below take PB patches at a time per block of 64 PB threads, thread t of a patch = pixel / coefficient
+// (t >> 3, t & 7), and a block goes on to further patches, so that the bases are read and their phases fixed once.
+// Every thread of the block calls them (barriers).
+constexpr int PB = 4;
+struct PatchBuf {
+    float a0[64], ar[64], ai[64], b0[64], br[64], bi[64];
+};
+
+// Coordinates of the patch whose pixel values thread t holds in p (R, G, B or gray): the DFT along the channels,
+// T = Phat V, S = U^H T (Eq. 19 without the Haar factor); o = [S^(1) | sqrt 2 Re S^(2) | sqrt 2 Im S^(2)] (orthonormal).
 template <int C>
-__global__ void __launch_bounds__(64) k_mean_coefs(const float *__restrict__ means, const float *__restrict__ b32,
-                                                   float *__restrict__ coefs) {
-    __shared__ float u0[64], v0[64], u1r[64], u1i[64], v1r[64], v1i[64];
-    __shared__ float p0[64], pr[64], pi[64], t0[64], tr[64], ti[64];
-    const int t = threadIdx.x, r = blockIdx.x;
-    load_bases<C>(b32, u0, v0, u1r, u1i, v1r, v1i);
-    const float *m = means + (size_t)r * C * 64;
+__device__ __forceinline__ void patch_forward(const MeanBasis &b, PatchBuf &w, int t, const float (&p)[C],
+                                              float (&o)[C]) {
+    __syncthreads();  // the buffer's last readers are done
     if (C == 1) {
-        p0[t] = m[t];
+        w.a0[t] = p[0];
     } else {
-        const float R = m[t], G = m[64 + t], B = m[128 + t];
-        p0[t] = ((R + G) + B) * K3F;
-        pr[t] = (R - 0.5f * (G + B)) * K3F;
-        pi[t] = (B - G) * 0.5f;
+        const float R = p[0], G = p[C - 2], B = p[C - 1];
+        w.a0[t] = ((R + G) + B) * K3F;
+        w.ar[t] = (R - 0.5f * (G + B)) * K3F;
+        w.ai[t] = (B - G) * 0.5f;
     }
     __syncthreads();
     const int hi = t >> 3, lo = t & 7;
     {  // T[i][b] = sum_j Phat[i][j] V[j][b], thread (i, b) = (hi, lo)
         float a0 = 0.f, ar = 0.f, ai = 0.f;
         for (int j = 0; j < 8; ++j) {
-            a0 = fmaf(p0[hi * 8 + j], v0[j * 8 + lo], a0);
+            a0 = fmaf(w.a0[hi * 8 + j], b.v0[j * 8 + lo], a0);
             if (C == 3) {
-                const float xr = pr[hi * 8 + j], xi = pi[hi * 8 + j], yr = v1r[j * 8 + lo], yi = v1i[j * 8 + lo];
+                const float xr = w.ar[hi * 8 + j], xi = w.ai[hi * 8 + j], yr = b.v1r[j * 8 + lo], yi = b.v1i[j * 8 + lo];
                 ar = fmaf(xr, yr, fmaf(-xi, yi, ar));
                 ai = fmaf(xr, yi, fmaf(xi, yr, ai));
             }
         }
-        t0[t] = a0;
-        tr[t] = ar;
-        ti[t] = ai;
+        w.b0[t] = a0;
+        w.br[t] = ar;
+        w.bi[t] = ai;
     }
     __syncthreads();
     {  // S[a][b] = sum_i conj(U[i][a]) T[i][b], thread (a, b) = (hi, lo)
         float s0 = 0.f, sr = 0.f, si = 0.f;
         for (int i = 0; i < 8; ++i) {
-            s0 = fmaf(u0[i * 8 + hi], t0[i * 8 + lo], s0);
+            s0 = fmaf(b.u0[i * 8 + hi], w.b0[i * 8 + lo], s0);
             if (C == 3) {
-                const float ur = u1r[i * 8 + hi], ui = u1i[i * 8 + hi], xr = tr[i * 8 + lo], xi = ti[i * 8 + lo];
+                const float ur = b.u1r[i * 8 + hi], ui = b.u1i[i * 8 + hi], xr = w.br[i * 8 + lo], xi = w.bi[i * 8 + lo];
                 sr = fmaf(ur, xr, fmaf(ui, xi, sr));
                 si = fmaf(ur, xi, fmaf(-ui, xr, si));
             }
         }
-        float *o = coefs + (size_t)r * C * 64;
-        o[t] = s0;
+        o[0] = s0;
         if (C == 3) {
-            o[64 + t] = SQ2 * sr;
-            o[128 + t] = SQ2 * si;
+            o[C - 2] = SQ2 * sr;
+            o[C - 1] = SQ2 * si;
         }
     }
 }
 
-// Inverse of k_mean_coefs: Phat = U S V^H per slice, then the inverse DFT along the channels.
+// The inverse: Phat = U S V^H per slice, then the inverse DFT along the channels.
 template <int C>
-__global__ void __launch_bounds__(64) k_coefs_to_patch(const float *__restrict__ coefs, const float *__restrict__ b32,
-                                                       float *__restrict__ patches) {
-    __shared__ float u0[64], v0[64], u1r[64], u1i[64], v1r[64], v1i[64];
-    __shared__ float s0[64], sr[64], si[64], q0[64], qr[64], qi[64];
-    const int t = threadIdx.x, r = blockIdx.x;
-    load_bases<C>(b32, u0, v0, u1r, u1i, v1r, v1i);
-    const float *c = coefs + (size_t)r * C * 64;
-    s0[t] = c[t];
+__device__ __forceinline__ void patch_inverse(const MeanBasis &b, PatchBuf &w, int t, const float (&c)[C],
+                                              float (&o)[C]) {
+    __syncthreads();
+    w.a0[t] = c[0];
     if (C == 3) {
-        sr[t] = c[64 + t] * (1.f / SQ2);
-        si[t] = c[128 + t] * (1.f / SQ2);
+        w.ar[t] = c[C - 2] * (1.f / SQ2);
+        w.ai[t] = c[C - 1] * (1.f / SQ2);
     }
     __syncthreads();
     const int hi = t >> 3, lo = t & 7;
     {  // Q[a][j] = sum_b S[a][b] conj(V[j][b]), thread (a, j) = (hi, lo)
         float a0 = 0.f, ar = 0.f, ai = 0.f;
-        for (int b = 0; b < 8; ++b) {
-            a0 = fmaf(s0[hi * 8 + b], v0[lo * 8 + b], a0);
+        for (int k = 0; k < 8; ++k) {
+            a0 = fmaf(w.a0[hi * 8 + k], b.v0[lo * 8 + k], a0);
             if (C == 3) {
-                const float xr = sr[hi * 8 + b], xi = si[hi * 8 + b], yr = v1r[lo * 8 + b], yi = v1i[lo * 8 + b];
+                const float xr = w.ar[hi * 8 + k], xi = w.ai[hi * 8 + k], yr = b.v1r[lo * 8 + k], yi = b.v1i[lo * 8 + k];
                 ar = fmaf(xr, yr, fmaf(xi, yi, ar));
                 ai = fmaf(xi, yr, fmaf(-xr, yi, ai));
             }
         }
-        q0[t] = a0;
-        qr[t] = ar;
-        qi[t] = ai;
+        w.b0[t] = a0;
+        w.br[t] = ar;
+        w.bi[t] = ai;
     }
     __syncthreads();
     {  // Phat[i][j] = sum_a U[i][a] Q[a][j], thread (i, j) = (hi, lo); then the inverse channel DFT
         float f0 = 0.f, fr = 0.f, fi = 0.f;
         for (int a = 0; a < 8; ++a) {
-            f0 = fmaf(u0[hi * 8 + a], q0[a * 8 + lo], f0);
+            f0 = fmaf(b.u0[hi * 8 + a], w.b0[a * 8 + lo], f0);
             if (C == 3) {
-                const float ur = u1r[hi * 8 + a], ui = u1i[hi * 8 + a], xr = qr[a * 8 + lo], xi = qi[a * 8 + lo];
+                const float ur = b.u1r[hi * 8 + a], ui = b.u1i[hi * 8 + a], xr = w.br[a * 8 + lo], xi = w.bi[a * 8 + lo];
                 fr = fmaf(ur, xr, fmaf(-ui, xi, fr));
                 fi = fmaf(ur, xi, fmaf(ui, xr, fi));
             }
         }
-        float *o = patches + (size_t)r * C * 64;
         if (C == 1) {
-            o[t] = f0;
+            o[0] = f0;
         } else {
-            o[t] = (f0 + 2.f * fr) * K3F;
-            o[64 + t] = (f0 - fr - 1.7320508075688772f * fi) * K3F;
-            o[128 + t] = (f0 - fr + 1.7320508075688772f * fi) * K3F;
+            o[0] = (f0 + 2.f * fr) * K3F;
+            o[C - 2] = (f0 - fr - 1.7320508075688772f * fi) * K3F;
+            o[C - 1] = (f0 - fr + 1.7320508075688772f * fi) * K3F;
+        }
+    }
+}
+
+// Patches (n x C x 64) to coordinates, or back (INV).
+template <int C, bool INV>
+__global__ void __launch_bounds__(64 * PB) k_mean_coefs(const float *__restrict__ in, int n,
+                                                        const float *__restrict__ b32, float *__restrict__ out) {
+    __shared__ MeanBasis b;
+    __shared__ PatchBuf w[PB];
+    const int t = threadIdx.x & 63, sub = threadIdx.x >> 6;
+    load_bases<C>(b32, b);
+    for (int r0 = blockIdx.x * PB; r0 < n; r0 += gridDim.x * PB) {
+        const int r = r0 + sub;
+        const float *src = in + (size_t)min(r, n - 1) * C * 64 + t;
+        float x[C], y[C];
+#pragma unroll
+        for (int c = 0; c < C; ++c) x[c] = src[64 * c];
+        if (INV) patch_inverse<C>(b, w[sub], t, x, y);
+        else patch_forward<C>(b, w[sub], t, x, y);
+        if (r < n) {
+#pragma unroll
+            for (int c = 0; c < C; ++c) out[(size_t)r * C * 64 + 64 * c + t] = y[c];
+        }
+    }
+}
+
+// The network's input from the groups in one pass: the mean patch of every group (as k_group_means), its coordinates
+// (kept for the residual) and the features (as k_features) with the call's sigma.  Bound by L2 (K pixels read per value
+// kept); as kernels of their own the three read and wrote the values between them and fixed the bases' phases per
+// patch: 512 x 512 x 3, 81 us (between events), now 44.
+template <int C>
+__global__ void __launch_bounds__(64 * PB) k_group_features(const float *__restrict__ img, int H, int W,
+                                                            const int32_t *__restrict__ idx, int K, int nref,
+                                                            const float *__restrict__ b32, const DevState *st, int din,
+                                                            float rsqrt_k, float *__restrict__ coords,
+                                                            float *__restrict__ X) {
+    __shared__ MeanBasis b;
+    __shared__ PatchBuf w[PB];
+    const int t = threadIdx.x & 63, sub = threadIdx.x >> 6;
+    const size_t HW = (size_t)H * W, at = (size_t)(t >> 3) * W + (t & 7);
+    const float sg = (float)st->sigma_hat;
+    load_bases<C>(b32, b);
+    for (int r0 = blockIdx.x * PB; r0 < nref; r0 += gridDim.x * PB) {
+        const int r = r0 + sub;
+        const int32_t *grp = idx + (size_t)min(r, nref - 1) * K;
+        float m[C], o[C];
+#pragma unroll
+        for (int c = 0; c < C; ++c) m[c] = 0.f;
+#pragma unroll 8
+        for (int k = 0; k < K; ++k) {
+            const float *src = img + (size_t)grp[k] + at;
+#pragma unroll
+            for (int c = 0; c < C; ++c) m[c] += src[c * HW];
+        }
+#pragma unroll
+        for (int c = 0; c < C; ++c) m[c] = m[c] / (float)K;
+        patch_forward<C>(b, w[sub], t, m, o);
+        if (r < nref) {
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                coords[(size_t)r * C * 64 + 64 * c + t] = o[c];
+                const float x = o[c] / (sg * rsqrt_k);
+                X[(size_t)r * din + 64 * c + t] = x / (1.f + fabsf(x) * (1.f / SAT));
+            }
+            if (t < din - C * 64) X[(size_t)r * din + C * 64 + t] = t == 0 ? sg * (1.f / 255.f) : 0.f;
+        }
+    }
+}
+
+// The refined patch of every group in pixels: coordinates plus s times the network's output, then patch_inverse.
+template <int C>
+__global__ void __launch_bounds__(64 * PB) k_refined_patch(const float *__restrict__ coords,
+                                                           const float *__restrict__ res, int n,
+                                                           const float *__restrict__ b32, const DevState *st,
+                                                           float rsqrt_k, float *__restrict__ patches) {
+    __shared__ MeanBasis b;
+    __shared__ PatchBuf w[PB];
+    const int t = threadIdx.x & 63, sub = threadIdx.x >> 6;
+    const float sg = (float)st->sigma_hat;
+    load_bases<C>(b32, b);
+    for (int r0 = blockIdx.x * PB; r0 < n; r0 += gridDim.x * PB) {
+        const int r = r0 + sub;
+        const size_t o = (size_t)min(r, n - 1) * C * 64 + t;
+        float x[C], y[C];
+#pragma unroll
+        for (int c = 0; c < C; ++c) x[c] = coords[o + 64 * c] + sg * rsqrt_k * res[o + 64 * c];
+        patch_inverse<C>(b, w[sub], t, x, y);
+        if (r < n) {
+#pragma unroll
+            for (int c = 0; c < C; ++c) patches[o + 64 * c] = y[c];
         }
     }
 }
@@ -556,6 +645,9 @@ int nsm() {
     cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
     return n;
 }
+
+// Blocks of the patch kernels: eight per SM, as many as are resident.
+int patch_blocks(int n) { return std::max(1, std::min((n + PB - 1) / PB, 8 * nsm())); }
 
 template <bool BK, int EPI>
 hts_status gemm(const GemmArgs &g, cudaStream_t s) {
@@ -635,7 +727,6 @@ void free_fcn(hts_fcn *f) {
     for (float *p : f->dy) cudaFree(p);
     cudaFree(f->loss);
     cudaFree(f->lpart);
-    cudaFree(f->sig);
     delete f;
 }
 
@@ -661,38 +752,40 @@ hts_status launch_group_means(const float *img, const Geom &g, const int32_t *id
 hts_status launch_mean_transform(const float *in, int n, int C, const float *b32, bool inverse, float *out,
                                  cudaStream_t s) {
     if (n == 0) return HTS_OK;
+    const int nb = patch_blocks(n);
     KTimer kt(inverse ? "k_coefs_to_patch" : "k_mean_coefs", s);
     if (C == 1) {
-        if (inverse) k_coefs_to_patch<1><<<n, 64, 0, s>>>(in, b32, out);
-        else k_mean_coefs<1><<<n, 64, 0, s>>>(in, b32, out);
+        if (inverse) k_mean_coefs<1, true><<<nb, 64 * PB, 0, s>>>(in, n, b32, out);
+        else k_mean_coefs<1, false><<<nb, 64 * PB, 0, s>>>(in, n, b32, out);
     } else {
-        if (inverse) k_coefs_to_patch<3><<<n, 64, 0, s>>>(in, b32, out);
-        else k_mean_coefs<3><<<n, 64, 0, s>>>(in, b32, out);
+        if (inverse) k_mean_coefs<3, true><<<nb, 64 * PB, 0, s>>>(in, n, b32, out);
+        else k_mean_coefs<3, false><<<nb, 64 * PB, 0, s>>>(in, n, b32, out);
     }
     return check_launch(inverse ? "k_coefs_to_patch" : "k_mean_coefs");
 }
 
-// Refined mean patches (pixels) of the groups whose mean patches are in buf (n x C x 64; overwritten),
-// with the call's sigma from the state; result in out (n x C x 64).
-hts_status fcn_refine_state(hts_fcn *f, float *buf, int n, const DevState *st, const float *b32, float *out,
-                            cudaStream_t s) {
+// Refined mean patches (pixels) of the groups idx, with the call's sigma from the state, in out (N_ref x C x 64);
+// coords: scratch of the same size.
+hts_status fcn_refine_groups(hts_fcn *f, const float *img, const Geom &g, const int32_t *idx, const DevState *st,
+                             const float *b32, float *coords, float *out, cudaStream_t s) {
+    const int n = g.nref, nb = patch_blocks(n);
+    const float rk = 1.f / std::sqrt((float)f->K);
     HTS_TRY(ensure(f, n));
-    HTS_TRY(launch_mean_transform(buf, n, f->C, b32, false, out, s));  // coordinates in out
     {
-        KTimer kt("k_state_sigma", s);
-        k_state_sigma<<<1, 1, 0, s>>>(st, f->sig);
+        KTimer kt("k_group_features", s);
+        if (f->C == 1)
+            k_group_features<1><<<nb, 64 * PB, 0, s>>>(img, g.H, g.W, idx, g.K, n, b32, st, f->din, rk, coords, f->X);
+        else
+            k_group_features<3><<<nb, 64 * PB, 0, s>>>(img, g.H, g.W, idx, g.K, n, b32, st, f->din, rk, coords, f->X);
     }
-    HTS_TRY(check_launch("k_state_sigma"));
-    HTS_TRY(features(f, out, f->sig, 0, n, s));
+    HTS_TRY(check_launch("k_group_features"));
     HTS_TRY(forward(f, n, s));
-    const long total = (long)n * f->dout;
     {
-        KTimer kt("k_fcn_refine", s);
-        k_refine<<<(unsigned)std::min<long>((total + 255) / 256, 8192), 256, 0, s>>>(
-            out, f->act[NL - 1], f->sig, 0, f->dout, 1.f / std::sqrt((float)f->K), total, buf);
+        KTimer kt("k_refined_patch", s);
+        if (f->C == 1) k_refined_patch<1><<<nb, 64 * PB, 0, s>>>(coords, f->act[NL - 1], n, b32, st, rk, out);
+        else k_refined_patch<3><<<nb, 64 * PB, 0, s>>>(coords, f->act[NL - 1], n, b32, st, rk, out);
     }
-    HTS_TRY(check_launch("k_fcn_refine"));
-    return launch_mean_transform(buf, n, f->C, b32, true, out, s);  // refined patch in pixels
+    return check_launch("k_refined_patch");
 }
 
 }  // namespace hts
@@ -724,7 +817,6 @@ extern "C" hts_status hts_fcn_create(int C, int K, uint64_t seed, hts_fcn **out)
         if (st == HTS_OK) st = cu(dev_malloc(p, f->nparams * sizeof(float)), "cudaMalloc(fcn)");
     if (st == HTS_OK) st = cu(dev_malloc(&f->loss, sizeof(double)), "cudaMalloc(fcn)");
     if (st == HTS_OK) st = cu(cudaMemset(f->loss, 0, sizeof(double)), "cudaMemset");
-    if (st == HTS_OK) st = cu(dev_malloc(&f->sig, sizeof(float)), "cudaMalloc(fcn)");
     if (st != HTS_OK) {
         free_fcn(f);
         return st;

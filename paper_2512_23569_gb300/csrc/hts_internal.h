@@ -127,6 +127,35 @@ struct KTimer {
     ~KTimer();
 };
 
+// Launches that overlap the kernel before them on the stream (programmatic dependent launch; nothing happens without
+// the launch attribute): grid_wait returns when every earlier grid has completed and its writes are visible, and every
+// thread calls it before its first access to memory that those write; grid_launch, called after it, lets the next
+// grid's blocks start once every block has called it -- so whatever ran before this grid is complete when they do.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Launches a kernel that calls grid_wait, overlapping the kernel before it on the stream, except inside a stream
+// capture: its launch and set-up (2 to 3 us, as long as many of these kernels run) then hide behind that one's end.
+template <typename... P, typename... A>
+hts_status launch_chained(const char *name, void (*k)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s,
+                          A &&...args) {
+    {
+        KTimer kt(name, s);
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = grid;
+        cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = s;
+        cfg.attrs = &attr;
+        cfg.numAttrs = stream_capturing(s) ? 0 : 1;
+        cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);  // its error is check_launch's
+    }
+    return check_launch(name);
+}
+
 // ---- matching (match.cu)
 hts_status launch_match(const float *img, const Geom &g, double gamma_gcp, int32_t *idx, uint8_t *green,
                         int32_t *fallback_list, DevState *st, cudaStream_t s);
@@ -186,12 +215,12 @@ hts_status launch_filter_tc(const float *img, const Geom &g, const int32_t *idx,
                             int *wcount, DevState *st, const float *sigma_ref, int map_judged, double tau_scale,
                             const float *mean_est, cudaStream_t s, bool *used);
 // Enhancement strategy (fcn.cu): mean patch of every group (N_ref x C x 64,
-// channel-major) and its refinement by the network with the state's sigma in
-// the basis b32's coordinates (buf is overwritten; the refined patch in
-// pixels lands in out).
+// channel-major); and the groups' mean patches refined by the network with the
+// state's sigma in the basis b32's coordinates, in pixels (out; coords: scratch
+// of the same size).
 hts_status launch_group_means(const float *img, const Geom &g, const int32_t *idx, float *means, cudaStream_t s);
-hts_status fcn_refine_state(hts_fcn *f, float *buf, int n, const DevState *st, const float *b32, float *out,
-                            cudaStream_t s);
+hts_status fcn_refine_groups(hts_fcn *f, const float *img, const Geom &g, const int32_t *idx, const DevState *st,
+                             const float *b32, float *coords, float *out, cudaStream_t s);
 
 // Filter tile shape (k_filter_tile): ty x tx reference positions per tile,
 // ty = 0 for the non-local mode (no tile accumulators).  The launch uses, in

@@ -164,13 +164,6 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src, bool in) 
 }
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// Launches that overlap the kernel before them on the stream (programmatic dependent launch; nothing happens without
-// the launch attribute): grid_wait returns when every earlier grid has completed and its writes are visible, and is
-// called before the first access to memory that those write; grid_launch, called after it by every block, lets the
-// next grid's blocks start -- so whatever ran before this grid is complete when they do.
-__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // Brings the 128-byte line holding p (a valid global address) into L2; no register waits on it.
 __device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
