@@ -20,11 +20,15 @@
 // complex slice's real and imaginary parts lie in the same row) and writes
 // them as the inverse GEMMs' operand; the inverse (Eq. 21) is F0^T and F1^T,
 // the same shared-memory matrices read with the transpose bit (MN-major),
-// giving each Haar row's slice values.  One transposed pass per slice hands
-// a (group, pixel) pair to a thread, which applies the inverse Haar along
-// the group and adds the members' estimates to the tile's sums of that
-// slice; slice 1's pass runs while the tensor cores compute slice 2's
-// inverse.  The sums are kept per slice, and the inverse channel DFT is
+// now as the MMAs' A, so that a tensor-memory lane is a pixel of a slice and
+// its columns are the batch's Haar rows: the thread of a lane reads a (group,
+// pixel) pair's rows from its own lane, applies the inverse Haar along the
+// group and adds the members' estimates to the tile's sums of that slice;
+// slice 1's pass runs while the tensor cores compute slice 2's inverse.
+// (With the Haar rows as M the slices went through a transposed buffer in
+// shared memory, 34 KB and six of eleven block barriers per batch:
+// 3840 x 2160 x 3, sigma 2 to 28: 2870 -> 2670 us; 1021 x 771 x 3, sigma 30:
+// 335 -> 317 us.)  The sums are kept per slice, and the inverse channel DFT is
 // applied once per pixel when they are normalised (k_normalize_box): the
 // aggregation and the DFT are both linear.
 //
@@ -98,7 +102,6 @@ __device__ __forceinline__ void haar_inv_u(float (&x)[K]) {
 
 constexpr int NT = 512;   // 16 warps: warp w reads tensor-memory lanes 32 (w % 4) .. + 31, column quarter w / 4
 constexpr int MB = 128;   // Haar rows per batch (8 groups of K = 16) = MMA M
-constexpr int TS = MB + 4;  // row stride (floats) of the transposed buffer: conflict-free float4 reads
 constexpr long long SPIN = 1ll << 24;
 
 // The row operands of the two GEMMs (forward: the groups' Haar rows of raw pixels, inverse: the thresholded
@@ -139,19 +142,20 @@ struct FtcLayout {
     static constexpr int B_HALVES = (C == 3) ? F0_HALVES + 128 * 128 : F0_HALVES;
     static constexpr size_t a_bytes = (size_t)C * BLK_A;  // the row operand
     static constexpr size_t a_off = 0;
-    static constexpr size_t t_off = a_off + a_bytes;  // the transposed FP32 buffer [64][TS] of one slice
-    static constexpr size_t b_off = t_off + (size_t)64 * TS * 4;
-    static constexpr size_t basis_off = t_off;  // 6 x 64 FP32, only while the transforms are built
+    static constexpr size_t basis_off = a_off;  // 6 x 64 FP32, only while the transforms are built
+    static constexpr size_t b_off = a_off + a_bytes;
     static constexpr size_t misc_off = b_off + (size_t)B_HALVES * 2;
-    // misc: tau[2][32] float, off[2][MB] int, 4 mbarrier words (forward; inverse of slice 1; inverse of
-    // slices 2-3), tensor-memory slot, detail flags
-    static constexpr size_t job_off = misc_off + (size_t)2 * 32 * 4 + 2 * MB * 4 + 32 + 16;
+    // misc: tau[2][32] float, off[3][MB] int, 4 mbarrier words (forward; inverse of slice 1; inverse of
+    // slices 2-3), tensor-memory slot, detail flags [2]
+    static constexpr size_t job_off = misc_off + (size_t)2 * 32 * 4 + 3 * MB * 4 + 32 + 16;
     // then the tile's sums [C][RA] int32 (per slice) and its staged region [RA] of PXH FP16 values a pixel (RA =
     // rows x acc_stride(width)): R, G, B and a pad, so that a pixel is one 8-byte load; one value for gray
     static constexpr int PXH = (C == 3) ? 4 : 1;
     static constexpr size_t acc_off = job_off + 256;
     static constexpr size_t bytes(int rh, int rw) { return acc_off + (size_t)rh * acc_stride(rw) * (C * 4 + PXH * 2); }
-    static constexpr uint32_t tcols = (C == 3) ? 256 : 64;
+    // the forward GEMMs fill columns 0 .. 64 C - 1 (a lane per Haar row), the inverse ones columns 0 .. 127
+    // (slice 1) and 128 .. 255 (slices 2-3), a column per Haar row
+    static constexpr uint32_t tcols = (C == 3) ? 256 : 128;
 };
 // a tile of one reference fits with the largest window (MAX_WIN)
 static_assert(FtcLayout<3>::bytes(MAX_WIN - 1 + PS, MAX_WIN - 1 + PS) <= 227 * 1024, "every window has a tile");
@@ -191,10 +195,10 @@ struct FtcBatch {
 //  3. threshold: a thread per row (tensor-memory lane) keeps or drops its coefficients against the level's
 //     threshold (modulus for the complex slice, both parts in the same lane), rescales the kept ones by
 //     2^-l and writes them as the inverse GEMMs' row operand (FP16);
-//  4. inverse GEMMs with F0^T, then F1^T (two commits): the rows' slice values, still in the Haar domain;
-//  5. per slice, once its inverse has completed: tensor memory -> transposed FP32 buffer; a thread per
-//     (group, pixel) pair applies the unnormalised inverse Haar and adds the K members' estimates of that
-//     pixel to the tile's sums of the slice.
+//  4. inverse GEMMs with F0^T, then F1^T (two commits): D[pixel][row], slice values still in the Haar domain;
+//  5. per slice, once its inverse has completed: a thread per (group, pixel) pair reads the pair's rows from its
+//     lane, applies the unnormalised inverse Haar and adds the K members' estimates of that pixel to the tile's
+//     sums of the slice.
 template <int C, int K, bool BATCH>
 __global__ void __launch_bounds__(NT, 1) k_filter_tc(const __grid_constant__ FtcArgs a0,
                                                      const __grid_constant__ FtcBatch bt) {
@@ -208,14 +212,13 @@ __global__ void __launch_bounds__(NT, 1) k_filter_tc(const __grid_constant__ Ftc
     constexpr int LOGK = (K == 8) ? 3 : (K == 16) ? 4 : 5;
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char *sA = smem + L::a_off;
-    float *sT = reinterpret_cast<float *>(smem + L::t_off);
     __half *sB = reinterpret_cast<__half *>(smem + L::b_off);
     float *sBas = reinterpret_cast<float *>(smem + L::basis_off);
     float *sTau = reinterpret_cast<float *>(smem + L::misc_off);  // [2][32] groups' thresholds
-    int *sOff = reinterpret_cast<int *>(sTau + 64);  // [2][MB] members' patch origins in the tile region (-1: none)
-    uint64_t *bar = reinterpret_cast<uint64_t *>(sOff + 2 * MB);  // [3], 8-byte aligned
+    int *sOff = reinterpret_cast<int *>(sTau + 64);  // [3][MB] members' patch origins in the tile region (-1: none)
+    uint64_t *bar = reinterpret_cast<uint64_t *>(sOff + 3 * MB);  // [3], 8-byte aligned
     uint32_t *slot = reinterpret_cast<uint32_t *>(bar + 4);
-    unsigned *sDet = slot + 1;  // bit 2 g + (slice > 0): group g of the batch kept a Haar detail coefficient
+    unsigned *sDet = slot + 1;  // [2] bit 2 g + (slice > 0): group g of the batch kept a Haar detail coefficient
     int *accs = reinterpret_cast<int *>(smem + L::acc_off);
     FtcArgs *sjob = reinterpret_cast<FtcArgs *>(smem + L::job_off);
     const FtcArgs &a = BATCH ? *sjob : a0;  // the current job's arguments
@@ -272,62 +275,86 @@ __global__ void __launch_bounds__(NT, 1) k_filter_tc(const __grid_constant__ Ftc
     tc::fence_after();
     const uint32_t tbase = *slot;
     const uint32_t idf0 = tc::idesc_f16(MB, 64, false), idf1 = tc::idesc_f16(MB, 128, false);  // B K-major
-    const uint32_t idi0 = idf0 | (1u << 16), idi1 = idf1 | (1u << 16);  // inverse: B transposed (MN-major)
+    const uint32_t idi0 = idf0 | (1u << 15), idi1 = idf1 | (1u << 15);  // inverse: A = F^T (MN-major), B K-major
     const int q = warp & 3, wq = warp >> 2;  // tensor-memory lane quarter, column quarter
     const uint32_t tlane = (uint32_t)(32 * q) << 16;
     uint32_t phase = 0;  // parity of the batches done: every barrier completes once per batch
     bool ok = true;
 
-    // A K step kk of the row operand: columns 16 kk .. 16 kk + 15, two core matrices at (kk % 4) * 2 * LBO_A
-    // in 64-column block kk / 4.
-    auto a_desc = [&](uint32_t a0, int kk) { return tc::sdesc(a0 + (kk >> 2) * BLK_A + (kk & 3) * 2 * LBO_A, LBO_A, SBO_A); };
+    // K step kk of the row operand from 8-row group rg on: columns 16 kk .. 16 kk + 15, two core matrices at
+    // (kk % 4) * 2 * LBO_A in 64-column block kk / 4.
+    auto a_desc = [&](uint32_t a0, int kk, int rg) {
+        return tc::sdesc(a0 + (kk >> 2) * BLK_A + (kk & 3) * 2 * LBO_A + rg * SBO_A, LBO_A, SBO_A);
+    };
     // Issues the MMAs of the forward GEMMs (commit on bar[0]) or of the inverse ones (slice 1's commit on
     // bar[1], then slices 2-3's on bar[2]), after every thread's shared-memory writes; thread 0 only.
-    // Forward B = F: K = pixels, core matrices 128 B apart along K, (64 or 128) * 16 B along N (coefficients).
-    // Inverse B = F^T read in place: K = coefficients ((64 or 128) * 16 B apart: LBO), N = pixels (128 B
-    // apart: SBO), the MN-major convention.
+    // Forward: A = the Haar rows (M = 128), B = F: K = pixels, core matrices 128 B apart along K, (64 or 128) * 16 B
+    // along N (coefficients).
+    // Inverse: A = F^T read in place (M = pixels, 128 B apart: SBO; K = coefficients, (64 or 128) * 16 B apart: LBO;
+    // the MN-major convention), B = the thresholded rows (N = Haar rows).  D[pixel][Haar row]: a lane per pixel of
+    // a slice, so that one thread reads all the Haar rows of a (group, pixel) pair from its own lane.  Slices 2-3: the
+    // 128 lanes are Re's 64 pixels, then Im's.  Slice 1 has 64 pixels for 128 lanes: rows 0-63 of the batch go to
+    // lanes 0-63 of columns 0-63, rows 64-127 to lanes 64-127 of columns 64-127.  The other lanes of the two are
+    // never read: their A rows are whatever lies in shared memory 1 KB beside F0 (in the row operand before it; in
+    // F1 or the words after it).
     auto issue = [&](bool inverse) {
         tc::fence_after();
         const uint32_t a0 = tc::su32(sA), f0 = tc::su32(sB), f1 = f0 + L::F0_HALVES * 2;
+        if (!inverse) {
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-            const uint64_t bd = inverse ? tc::sdesc(f0 + kk * 2 * 1024, 1024, 128) : tc::sdesc(f0 + kk * 256, 128, 1024);
-            tc::mma_f16(tbase, a_desc(a0, kk), bd, inverse ? idi0 : idf0, kk > 0 ? 1u : 0u);
-        }
-        if (inverse) tc::mma_commit(&bar[1]);
-        if constexpr (C == 3) {
+            for (int kk = 0; kk < 4; ++kk)
+                tc::mma_f16(tbase, a_desc(a0, kk, 0), tc::sdesc(f0 + kk * 256, 128, 1024), idf0, kk > 0 ? 1u : 0u);
+            if constexpr (C == 3) {
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk) {
-                const uint64_t bd =
-                    inverse ? tc::sdesc(f1 + kk * 2 * 2048, 2048, 128) : tc::sdesc(f1 + kk * 256, 128, 2048);
-                tc::mma_f16(tbase + 64, a_desc(a0, 4 + kk), bd, inverse ? idi1 : idf1, kk > 0 ? 1u : 0u);
+                for (int kk = 0; kk < 8; ++kk)
+                    tc::mma_f16(tbase + 64, a_desc(a0, 4 + kk, 0), tc::sdesc(f1 + kk * 256, 128, 2048), idf1,
+                                kk > 0 ? 1u : 0u);
             }
-            if (inverse) tc::mma_commit(&bar[2]);
+            tc::mma_commit(&bar[0]);
+        } else {
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf)
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk)
+                    tc::mma_f16(tbase + 64 * hf, tc::sdesc(f0 - 1024 * hf + kk * 2 * 1024, 1024, 128),
+                                a_desc(a0, kk, 8 * hf), idi0, kk > 0 ? 1u : 0u);
+            tc::mma_commit(&bar[1]);
+            if constexpr (C == 3) {
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk)
+                    tc::mma_f16(tbase + 128, tc::sdesc(f1 + kk * 2 * 2048, 2048, 128), a_desc(a0, 4 + kk, 0), idi1,
+                                kk > 0 ? 1u : 0u);
+                tc::mma_commit(&bar[2]);
+            }
         }
-        if (!inverse) tc::mma_commit(&bar[0]);
     };
-    // Every thread: the row operand written, then thread 0 issues the GEMMs.
-    auto launch_stage = [&](bool inverse) {
+    // A wait for MMAs gives up on its own; the whole block learns of it at the next barrier (meanwhile the thread
+    // works on values that are thrown away, at addresses that do not depend on them).
+    bool bad = false;
+    auto wait_bar = [&](int i) {
+        if (!tc::bar_wait(&bar[i], phase, SPIN)) bad = true;
+        tc::fence_after();
+    };
+    // Once a wait has given up: error 2, and thread 0 waits (bounded) for the MMAs that the last issue of parity
+    // ph left in flight, so that the memory can be released.
+    auto give_up = [&](bool inverse, uint32_t ph) {
+        if (tid == 0) {
+            for (int j = inverse ? 1 : 0; j < (inverse ? (C == 3 ? 3 : 2) : 1); ++j) tc::bar_wait(&bar[j], ph, SPIN);
+            atomicExch(&a.st->error, 2);
+        }
+        ok = false;
+    };
+    // Every thread: the row operand written, then thread 0 issues the GEMMs; false if a wait before gave up.
+    auto launch_stage = [&](bool inverse) -> bool {
         tc::fence_async_smem();
         tc::fence_before();
-        __syncthreads();
-        if (tid == 0) issue(inverse);
-    };
-    // Waits for barrier i of this batch; false (error 2 recorded) if the wait gave up, after thread 0 has
-    // waited (bounded) for every MMA this batch issued, so that the memory can be released.
-    auto wait_bar = [&](int i) -> bool {
-        const bool done = tc::bar_wait(&bar[i], phase, SPIN);
-        if (__syncthreads_or(!done)) {
-            if (tid == 0) {
-                for (int j = i; j < (i == 0 ? 1 : (C == 3 ? 3 : 2)); ++j) tc::bar_wait(&bar[j], phase, SPIN);
-                atomicExch(&a.st->error, 2);
-            }
+        if (__syncthreads_or(bad)) {
+            give_up(!inverse, inverse ? phase : phase ^ 1u);
             return false;
         }
-        tc::fence_after();
+        if (tid == 0) issue(inverse);
         return true;
     };
-
     // pair slot i of this thread: group g, pixel p (patch row p >> 3, column p & 7), half h of the group's
     // members (K = 32).  A warp covers 32 consecutive pixels of one group (4 patch rows: 4 coalesced 32-byte
     // segments per member); for K = 32 16 pixels of both halves, the partner half in lane ^ 16.
@@ -538,6 +565,92 @@ __global__ void __launch_bounds__(NT, 1) k_filter_tc(const __grid_constant__ Ftc
                 }
             }
         };
+        // Inverse Haar along the group axis (Eq. 21) and aggregation: slice c of pixel 32 (q % 2) + lane for the 16 Haar
+        // rows from rb on of batch b (two groups of K = 8, one of 16, half of one of 32), whose column in this lane is
+        // tcol + row; member offsets in buffer buf.
+        const int ap = 32 * (q & 1) + lane;              // the patch's pixel
+        const int app = (ap >> 3) * rwp + (ap & 7);      // its place in the region beside the patch's origin
+        auto aggregate = [&](int rb, uint32_t tcol, int c, int b, int buf, unsigned det) {
+            int *dst = acc_v + c * RP + app;
+            const int h = (K == 32) ? (rb >> 4) & 1 : 0;
+#pragma unroll
+            for (int gi = 0; gi < 16 / KM; ++gi) {
+                const int g = rb / K + gi;
+                const int4 *offp = reinterpret_cast<const int4 *>(sOff + MB * buf + g * K + h * KM);
+                float mu = 0.f;  // first Haar row replaced (Eq. 24-25): the refined mean joins every member
+                if (ra) {
+                    const int lg = b * GPB + g;
+                    const int gy = gy0 + lg / a.tx, gx = gx0 + lg % a.tx;
+                    if (lg < gpt && gy <= gy1 && gx <= gx1) {
+                        const float *mp = a.mean_est + (size_t)(gy * a.nx + gx) * (C * 64) + ap;
+                        // slice c of the refined mean's pixel
+                        if (C == 1) {
+                            mu = __ldg(mp);
+                        } else {
+                            const float r = __ldg(mp), gg = __ldg(mp + 64), bl = __ldg(mp + 128);
+                            mu = c == 0 ? K3F * (r + (gg + bl)) : c == 1 ? K23F * fmaf(-0.5f, gg + bl, r) : K12F * (bl - gg);
+                        }
+                    }
+                }
+                // No detail coefficient of the group's slice was kept (the rule where the members match to within
+                // the noise): the butterflies would add zeros, and every member gets the first row's value.  A
+                // warp holds one group, so it takes this way as a whole.
+                if (!(det >> (2 * g + (c > 0 ? 1 : 0)) & 1u)) {
+                    uint32_t z = tc::tmem_ld1(tcol + (uint32_t)(g * K));
+                    tc::tmem_wait_ld(z);
+                    float x0 = __uint_as_float(z);
+                    if (ra) x0 += mu;
+                    const int fx = fix8(x0);
+                    if (fx != 0) {  // (chroma slices thresholded away)
+#pragma unroll
+                        for (int j4 = 0; j4 < KM / 4; ++j4) {
+                            const int4 o4 = offp[j4];
+                            const int o[4] = {o4.x, o4.y, o4.z, o4.w};
+#pragma unroll
+                            for (int j = 0; j < 4; ++j)
+                                if (o[j] >= 0 && HTS_IN_BOUNDS(o[j] + app < RP, &a.st->error)) atomicAdd(dst + o[j], fx);
+                        }
+                    }
+                    continue;
+                }
+                float x[KM];
+                if constexpr (K == 8) {
+                    uint32_t v[8];
+                    tc::tmem_ld8(tcol + (uint32_t)(g * K), v);
+                    tc::tmem_wait_ld(v);
+#pragma unroll
+                    for (int r = 0; r < 8; ++r) x[r] = __uint_as_float(v[r]);
+                } else if constexpr (K == 16) {
+                    uint32_t v[16];
+                    tc::tmem_ld16(tcol + (uint32_t)(g * K), v);
+                    tc::tmem_wait_ld(v);
+#pragma unroll
+                    for (int r = 0; r < 16; ++r) x[r] = __uint_as_float(v[r]);
+                } else {
+                    uint32_t v[32];
+                    tc::tmem_ld32(tcol + (uint32_t)(g * K), v);
+                    tc::tmem_wait_ld(v);
+                    const float z0 = __uint_as_float(v[0]), z1 = __uint_as_float(v[1]);
+                    x[0] = h ? (z0 - z1) : (z0 + z1);  // the top level: this half's sum
+#pragma unroll
+                    for (int r = 1; r < KM; ++r) x[r] = __uint_as_float(h ? v[grow(r, 1)] : v[grow(r, 0)]);
+                }
+                haar_inv_u<KM>(x);
+                if (ra) {
+#pragma unroll
+                    for (int j = 0; j < KM; ++j) x[j] += mu;
+                }
+#pragma unroll
+                for (int j4 = 0; j4 < KM / 4; ++j4) {
+                    const int4 o4 = offp[j4];
+                    const int o[4] = {o4.x, o4.y, o4.z, o4.w};
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (o[j] >= 0 && HTS_IN_BOUNDS(o[j] + app < RP, &a.st->error))
+                            atomicAdd(dst + o[j], fix8(x[4 * j4 + j]));
+                }
+            }
+        };
         int posreg = -1;
         float sigreg = 0.f;
         bool pvalid = false, svalid = false;
@@ -553,20 +666,18 @@ __global__ void __launch_bounds__(NT, 1) k_filter_tc(const __grid_constant__ Ftc
         }
         __syncthreads();
         for (int b = 0; b < nbatch; ++b) {
-            const int cur = b & 1;
+            const int cur = b & 1;                   // thresholds, detail flags
+            const int cur3 = b % 3, nxt3 = (b + 1) % 3;  // offsets: read until the batch's last aggregation, no barrier after
             const float *bTau = sTau + 32 * cur;
-            if (tid == 0) *sDet = 0u;  // read last before the previous batch's last barrier
-            commit(cur);
+            if (tid == 0) sDet[cur] = 0u;  // read last in the batch before the previous one
+            commit(cur3);
             if (b + 1 < nbatch) {  // the next batch's thresholds and member offsets (read after the next barrier)
                 if (tid < GPB) sTau[32 * (cur ^ 1) + tid] = tau_from(sigreg, svalid);
-                if (tid < MB) member_off(pvalid ? posreg : -1, cur ^ 1);
+                if (tid < MB) member_off(pvalid ? posreg : -1, nxt3);
             }
             // ---- forward transform (Eq. 19) of the Haar rows: D[row] = [S0 | sqrt2 Re S1 | sqrt2 Im S1]
-            launch_stage(false);
-            if (!wait_bar(0)) {
-                ok = false;
-                break;
-            }
+            if (!launch_stage(false)) break;
+            wait_bar(0);
             if (b + 2 < nbatch) {  // the positions and noise levels of the batch after next
                 if (tid < MB) posreg = member_pos(b + 2, pvalid);
                 if (tid < GPB) sigreg = sig_of(b + 2, svalid);
@@ -632,119 +743,29 @@ __global__ void __launch_bounds__(NT, 1) k_filter_tc(const __grid_constant__ Ftc
                     *reinterpret_cast<uint4 *>(rowp + 2 * BLK_A + (2 * wq + 1) * LBO_A) = ip[1];
                 }
                 det = __reduce_or_sync(0xffffffffu, det);
-                if (lane == 0 && det) atomicOr(sDet, det);
+                if (lane == 0 && det) atomicOr(sDet + cur, det);
             }
-            // ---- inverse transform (Eq. 21): E[row] = the slices' values of the group's thresholded Haar rows,
-            //      slice 1 first (its own commit), so that its aggregation overlaps the rest
-            launch_stage(true);
-            // ---- per slice: inverse Haar along the group axis and aggregation of the members' estimates
-            int offs[PPT][KM];  // this thread's members' patch origins in the region (-1: empty slot)
-#pragma unroll
-            for (int i = 0; i < PPT; ++i) {
-                int g, p, h;
-                slot_of(i, g, p, h);
-#pragma unroll
-                for (int j = 0; j < KM; ++j) {
-                    const int o = sOff[MB * cur + g * K + h * KM + j];
-                    offs[i][j] = o >= 0 ? o + (p >> 3) * rwp + (p & 7) : -1;
-                }
-            }
+            // ---- inverse transform (Eq. 21): the slices' values of the groups' thresholded Haar rows, slice 1 first
+            //      (its own commit), so that its aggregation overlaps the rest; then, per slice, the inverse Haar along
+            //      the group axis and the aggregation of the members' estimates
+            if (!launch_stage(true)) break;
+            const unsigned det = sDet[cur];
+            wait_bar(1);
+            aggregate(64 * (q >> 1) + 16 * wq, tbase + tlane, 0, b, cur3, det);
+            if constexpr (C == 3) {
+                wait_bar(2);
 #pragma unroll 1
-            for (int c = 0; c < C; ++c) {
-                if (c < 2 && !wait_bar(1 + c)) {  // slice c's inverse has completed (slices 2 and 3 together)
-                    ok = false;
-                    break;
-                }
-                {
-                    uint32_t v[16];
-                    tc::tmem_ld16(tbase + tlane + (uint32_t)(64 * c + 16 * wq), v);
-                    tc::tmem_wait_ld();
-                    const int m = 32 * q + lane;
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) sT[(16 * wq + j) * TS + m] = __uint_as_float(v[j]);
-                }
-                __syncthreads();
-#pragma unroll
-                for (int i = 0; i < PPT; ++i) {
-                    int g, p, h;
-                    slot_of(i, g, p, h);
-                    const float *colp = sT + p * TS + g * K;
-                    float mu = 0.f;  // first Haar row replaced (Eq. 24-25): the refined mean joins every member
-                    if (ra) {
-                        const int lg = b * GPB + g;
-                        const int gy = gy0 + lg / a.tx, gx = gx0 + lg % a.tx;
-                        if (lg < gpt && gy <= gy1 && gx <= gx1) {
-                            const float *mp = a.mean_est + (size_t)(gy * a.nx + gx) * (C * 64) + p;
-                            // slice c of the refined mean's pixel p
-                            if (C == 1) {
-                                mu = __ldg(mp);
-                            } else {
-                                const float r = __ldg(mp), gg = __ldg(mp + 64), bl = __ldg(mp + 128);
-                                mu = c == 0 ? K3F * (r + (gg + bl)) : c == 1 ? K23F * fmaf(-0.5f, gg + bl, r) : K12F * (bl - gg);
-                            }
-                        }
-                    }
-                    int *dst = acc_v + c * RP;
-                    // No detail coefficient of the group's slice was kept (the rule where the members match to within
-                    // the noise): the butterflies would add zeros, and every member gets the first row's value.  A
-                    // warp holds one group, so it takes this way as a whole.  (With the region's 8-byte pixels 20 % of
-                    // the warp instructions: 3840 x 2160 x 3, sigma 2 to 28: 3190 -> 2870 us; 1021 x 771 x 3, sigma
-                    // 30: 372 -> 335.  Barriers between the phases, 16 warps per SM in step, bind it now.)
-                    if (!(*sDet >> (2 * g + (c > 0 ? 1 : 0)) & 1u)) {
-                        float x0 = colp[0];
-                        if (ra) x0 += mu;
-                        const int fx = fix8(x0);
-                        if (fx != 0) {  // (chroma slices thresholded away)
-#pragma unroll
-                            for (int j = 0; j < KM; ++j)
-                                if (offs[i][j] >= 0 && HTS_IN_BOUNDS(offs[i][j] < RP, &a.st->error))
-                                    atomicAdd(dst + offs[i][j], fx);
-                        }
-                        continue;
-                    }
-                    float x[KM];
-                    if (TPP == 1) {
-#pragma unroll
-                        for (int r = 0; r < KM; r += 4) {
-                            const float4 t4 = *reinterpret_cast<const float4 *>(colp + r);
-                            x[r] = t4.x;
-                            x[r + 1] = t4.y;
-                            x[r + 2] = t4.z;
-                            x[r + 3] = t4.w;
-                        }
-                    } else {
-                        const float2 z = *reinterpret_cast<const float2 *>(colp);
-                        x[0] = h ? (z.x - z.y) : (z.x + z.y);  // the top level: this half's sum
-                        x[1] = colp[grow(1, h)];
-                        const float2 u = *reinterpret_cast<const float2 *>(colp + grow(2, h));
-                        x[2] = u.x;
-                        x[3] = u.y;
-#pragma unroll
-                        for (int r = 4; r < KM; r += 4) {
-                            const float4 t4 = *reinterpret_cast<const float4 *>(colp + grow(r, h));
-                            x[r] = t4.x;
-                            x[r + 1] = t4.y;
-                            x[r + 2] = t4.z;
-                            x[r + 3] = t4.w;
-                        }
-                    }
-                    haar_inv_u<KM>(x);
-                    if (ra) {
-#pragma unroll
-                        for (int j = 0; j < KM; ++j) x[j] += mu;
-                    }
-#pragma unroll
-                    for (int j = 0; j < KM; ++j)
-                        if (offs[i][j] >= 0 && HTS_IN_BOUNDS(offs[i][j] < RP, &a.st->error))
-                            atomicAdd(dst + offs[i][j], fix8(x[j]));
-                }
-                tc::fence_before();
-                __syncthreads();
+                for (int t = 0; t < 2; ++t)
+                    aggregate(32 * wq + 16 * t, tbase + tlane + 128u, 1 + (q >> 1), b, cur3, det);
             }
-            if (!ok) break;
             phase ^= 1u;
         }
         if (!ok) break;
+        tc::fence_before();
+        if (__syncthreads_or(bad)) {
+            give_up(true, phase ^ 1u);
+            break;
+        }
         // flush the tile's sums (per slice) to the image-wide int64 sums
         for (int e = tid; e < rh * rw; e += NT) {
             const int yy = e / rw, xx = e - yy * rw;
