@@ -24,7 +24,8 @@
 // candidate's index, so equal distances keep the lower index first; ~0 for a
 // candidate outside the reference's window) and drops key i into bin i (K = 32:
 // bin i mod 16), a sorted list of T slots, through a branch-free min / max network -- every
-// lane and every warp does the same work in every run.  The smallest key a
+// lane and every warp does the same work in every run.  The index bits that are the
+// bin's number (the half-runs start at multiples of 32) join the keys after the runs.  The smallest key a
 // full bin pushed out is remembered.  A ninth warp issues the MMAs into two
 // accumulators of 256 columns: a run goes into an accumulator once all eight
 // warps have loaded the run before from it (mbarriers, no block-wide barrier
@@ -281,6 +282,7 @@ __global__ void __launch_bounds__(NT, 1) k_match_tc(const __grid_constant__ TcAr
     int *abort_flag = reinterpret_cast<int *>(tbar + 1);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(abort_flag + 1);
     int *item_slot = reinterpret_cast<int *>(tmem_slot + 1);  // the block's current work item
+    unsigned *rn_max = reinterpret_cast<unsigned *>(item_slot + 1);  // largest finite row norm of the item (bits)
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const bool cw = warp < NWC;              // a reading warp
@@ -313,7 +315,10 @@ __global__ void __launch_bounds__(NT, 1) k_match_tc(const __grid_constant__ TcAr
         // on two SMs and blocks that drew passes without references move on at once.  The fence orders this
         // thread's earlier shared-memory accesses before the next item's TMA writes into the same area.
         tc::fence_async_smem();
-        if (tid == 0) *item_slot = atomicAdd(BATCH ? bt.queue : &a0.st->mtc_next, 1);
+        if (tid == 0) {
+            *item_slot = atomicAdd(BATCH ? bt.queue : &a0.st->mtc_next, 1);
+            *rn_max = 0u;
+        }
         __syncthreads();
         int item = *item_slot;
         __syncthreads();
@@ -442,6 +447,7 @@ __global__ void __launch_bounds__(NT, 1) k_match_tc(const __grid_constant__ TcAr
                 }
             }
             __syncthreads();
+            unsigned nmax = 0u;  // largest finite row norm (bits)
             for (int qi = tid; qi < nq; qi += NT) {
                 const int y = qi / Wq, x = qi - y * Wq;
                 uint4 w = make_uint4(0u, 0u, 0u, 0u);
@@ -458,15 +464,23 @@ __global__ void __launch_bounds__(NT, 1) k_match_tc(const __grid_constant__ TcAr
                 }
                 Q[qi] = w;
                 rn[qi] = n2;  // squared norm of the BF16 row-8 vector
+                if (__float_as_uint(n2) < 0x7f800000u) nmax = max(nmax, __float_as_uint(n2));
             }
+            nmax = __reduce_max_sync(FULLM, nmax);
+            if (lane == 0) atomicMax(rn_max, nmax);
             __syncthreads();
+            // Distances are formed times a power of two that brings the item's largest below 1 (at most four times
+            // eight row norms: 2^5), so that the fused multiply-add's saturation is their clamp at 0: their order and
+            // the keys' mantissas are those of the distances themselves.
+            const float scale = __int_as_float(max(1, min(254, 248 - (int)(*rn_max >> 23))) << 23);
+            const float m2s = -2.f * scale;
             for (int p = tid; p < ncand + CH; p += NT) {
                 float e2 = 0.f;
                 if (p < ncand) {
 #pragma unroll
                     for (int u = 0; u < PS; ++u) e2 += rn[p + u * Wq];
                 }
-                E[p] = e2;
+                E[p] = e2 * scale;
             }
             // A: row j = reference j, element 8u+v; core matrix (j/8, u) at (j/8)*1024 + u*128
             for (int e = tid; e < NR * PS; e += NT) {
@@ -515,7 +529,7 @@ __global__ void __launch_bounds__(NT, 1) k_match_tc(const __grid_constant__ TcAr
             for (int g = 0; g < NBIN; ++g)
 #pragma unroll
                 for (int t = 0; t < T; ++t) bn[g][t] = 0xffffffffu;
-            uint32_t ev = 0xffffffffu;  // smallest key a full bin pushed out
+            uint32_t ev = 0xffffffffu;  // smallest key a full bin pushed out, without the bin's bits: never above it
             if (!cw) {  // the issuing warp: run c goes into its accumulator once run c - NBUF was loaded by all
                 if (lane == 0) {
                     int issued = 0;
@@ -574,23 +588,31 @@ __global__ void __launch_bounds__(NT, 1) k_match_tc(const __grid_constant__ TcAr
                     if (lane == 0) tc::bar_arrive(&empty[b]);  // this warp is done with accumulator b
                     if (act && __any_sync(FULLM, vm != 0u)) {
                         const float4 *E4 = reinterpret_cast<const float4 *>(E + pb);
+                        // Bound by the pipe of logic, select and min / max operations, 9.5 of 11.5 a key (K <= 16) since
+                        // the clamp went into the multiply-add, the column's bits (the bin's number) out of the key
+                        // and the pushed-out keys into three-way minima; 14 operations before: 3840 x 2160 x 3, K = 16,
+                        // win 31: 2561 -> 2469 us, 1536 x 2048 x 3: 1018 -> 981 us.
+                        const uint32_t pbh[2] = {(uint32_t)pb, (uint32_t)(pb + NBIN % 32)};
 #pragma unroll
                         for (int i4 = 0; i4 < 8; ++i4) {
                             const float4 e4 = E4[i4];
                             const float evl[4] = {e4.x, e4.y, e4.z, e4.w};
+                            uint32_t out[4];  // the key each bin pushes out
 #pragma unroll
                             for (int l = 0; l < 4; ++l) {
                                 const int i = 4 * i4 + l;
-                                const float d = fmaf(-2.f, __uint_as_float(v[i]), a2 + evl[l]);
-                                uint32_t key = (__float_as_uint(fmaxf(d, 0.f)) & him) | (uint32_t)(pb + i);
+                                const float d = __saturatef(fmaf(m2s, __uint_as_float(v[i]), a2 + evl[l]));
+                                uint32_t key = (__float_as_uint(d) & him) | pbh[i / NBIN];
                                 key = (vm & (1u << i)) ? key : 0xffffffffu;
                                 uint32_t *bb = bn[i % NBIN];
-                                ev = min(ev, max(bb[T - 1], key));
+                                out[l] = max(bb[T - 1], key);
                                 // every slot from the old bin alone: no dependent chain
 #pragma unroll
                                 for (int t = T - 1; t > 0; --t) bb[t] = max(bb[t - 1], min(bb[t], key));
                                 bb[0] = min(bb[0], key);
                             }
+                            ev = __vimin3_u32(ev, out[0], out[1]);
+                            ev = __vimin3_u32(ev, out[2], out[3]);
                         }
                     }
                     rx += CH;
@@ -616,7 +638,8 @@ __global__ void __launch_bounds__(NT, 1) k_match_tc(const __grid_constant__ TcAr
 #pragma unroll
                 for (int g = 0; g < NBIN; ++g)
 #pragma unroll
-                    for (int s = 0; s < TP; ++s) v[g * TP + s] = s < T ? bn[g][s] : 0xffffffffu;
+                    for (int s = 0; s < TP; ++s)  // the bin's number back into the key (~0 stays)
+                        v[g * TP + s] = s < T ? (bn[g][s] | (uint32_t)g) : 0xffffffffu;
                 smallest_sorted<NBIN * TP, TP, LS>(v);
 #pragma unroll
                 for (int t = 0; t < LH; ++t) fk[(hh * LH + t) * NR + m] = v[t];
