@@ -98,8 +98,25 @@ __device__ __forceinline__ int cover_count(int i, int n, int step) {
     return c;
 }
 
+// The line pair (y + a, y + b) with a, b >= step is the pair (a - step, b - step) of the next grid line, so at step 4..7
+// (a - step < step; a smaller step would chain parents, a larger one has none) block bl's partial sum of such a "derived"
+// entry is, bit for bit, block bl + 1's of its parent wherever the lines of block bl, each moved on by one, are those of
+// block bl + 1 and all on the step: 222 of 300 entries are left to sum (colour, step 4).
+__device__ __forceinline__ bool cov_shared(int bl, int nb, int n, int nlines, int step) {
+    if (step < 4 || step >= PS || bl + 1 >= nb) return false;
+    const int last_reg = (n - PS) / step;  // the last line on the step
+    const int last = bl + (nlines - 1 - bl) / nb * nb, last1 = bl + 1 + (nlines - 2 - bl) / nb * nb;  // the blocks' last lines
+    return last1 == last + 1 && last1 <= last_reg;
+}
+
 // blockIdx.y = side (0: row sums along image rows, 1: column sums along image columns); block b of a
-// side takes grid lines b, b + nb, ... (nb = nb_r or nb_c); thread t < PER takes entry t of its side.
+// side takes grid lines b, b + nb, ... (nb = nb_r or nb_c); a thread takes an entry of its side (the last warps only
+// stage where the derived entries are left to the next block).  Bound by FP32 issue: ten operations a product and two
+// 16-byte loads per four where the chunk's cover counts are one power of two (all but a line's ends): that scales the
+// double-float sum exactly.  Elsewhere the count is a third load and one more operation, as it was everywhere.
+// 1024 x 1024 x 3, both sides: 114 -> 97 us; hts_denoise_learned at 3840 x 2160 x 3, where the sums share the SMs with
+// the matching: 8205 -> 8062 us.  Only steps that keep every bit of the sums are open here: near-equal eigenvalues turn
+// 1e-15 of the largest into 1e-6 of an eigenvector, which the FP16 transforms of the tensor-core filter show.
 template <int C>
 __global__ void __launch_bounds__(CovCfg<C>::THREADS) k_cov(const float *__restrict__ img, int H, int W, int step,
                                                             int ny, int nx, int nb_r, int nb_c,
@@ -113,9 +130,22 @@ __global__ void __launch_bounds__(CovCfg<C>::THREADS) k_cov(const float *__restr
     const int nb = side == 0 ? nb_r : nb_c;
     if ((int)blockIdx.x >= nb) return;  // the whole block
     const int t = threadIdx.x;
-    const bool valid = t < PER;
+    // thread -> entry: every one, or those with a < step or b < step (a triangle's first rows; of a square the first
+    // rows, then the first columns of the others)
+    int ent = t, nent = PER;
+    if (cov_shared(blockIdx.x, nb, side == 0 ? H : W, side == 0 ? ny : nx, step)) {
+        const int ns = 8 * step - step * (step - 1) / 2, na = 64 - (8 - step) * (8 - step);
+        nent = CovCfg<C>::NSYM * ns + CovCfg<C>::NASY * na;
+        if (t < CovCfg<C>::NSYM * ns) {
+            ent = t / ns * 36 + t % ns;
+        } else {
+            const int u = t - CovCfg<C>::NSYM * ns, q = u / na, e = u - q * na, r = e - 8 * step;
+            ent = CovCfg<C>::NSYM * 36 + 64 * q + (r < 0 ? e : (step + r / step) * 8 + r % step);
+        }
+    }
+    const bool valid = t < nent;
     int m = 0, t0 = 0, t1 = 0, a = 0, b = 0;
-    if (valid) task_of(side * PER + t, PER, CovCfg<C>::NSYM, m, t0, t1, a, b);
+    if (valid) task_of(side * PER + ent, PER, CovCfg<C>::NSYM, m, t0, t1, a, b);
     const size_t HW = (size_t)H * W;
     const int nlines = side == 0 ? ny : nx;
     const int len = side == 0 ? W : H;
@@ -125,44 +155,65 @@ __global__ void __launch_bounds__(CovCfg<C>::THREADS) k_cov(const float *__restr
         for (int p0 = 0; p0 < len; p0 += COV_CH) {
             const int np = min(COV_CH, len - p0);
             if (side == 0) {  // rows base .. base + 7 of every channel, columns p0 .. p0 + np - 1
-                for (int e = t; e < NL * COV_CH; e += blockDim.x) {
+#pragma unroll 4
+                for (int e = t; e < NL * COV_CH; e += CovCfg<C>::THREADS) {
                     const int ln = e / COV_CH, q = e - ln * COV_CH;
                     const int c = ln >> 3, off = ln & 7;
                     sl[ln][q] = q < np ? __ldg(img + c * HW + (size_t)(base + off) * W + p0 + q) : 0.f;
                 }
             } else {  // columns base .. base + 7 of every channel, rows p0 .. p0 + np - 1
-                for (int e = t; e < NL * COV_CH; e += blockDim.x) {
+#pragma unroll 4
+                for (int e = t; e < NL * COV_CH; e += CovCfg<C>::THREADS) {
                     const int q = e / NL, ln = e - q * NL;
                     const int c = ln >> 3, off = ln & 7;
                     sl[ln][q] = q < np ? __ldg(img + c * HW + (size_t)(p0 + q) * W + base + off) : 0.f;
                 }
             }
-            for (int q = t; q < COV_CH; q += blockDim.x) sw[q] = q < np ? (float)cover_count(p0 + q, len, step) : 0.f;
-            __syncthreads();
+            const int w0 = cover_count(p0, len, step);
+            bool same = (w0 & (w0 - 1)) == 0;  // the chunk's counts are one power of two
+            for (int q = t; q < COV_CH; q += CovCfg<C>::THREADS) {
+                const int cnt = q < np ? cover_count(p0 + q, len, step) : 0;
+                same = same && (q >= np || cnt == w0);
+                sw[q] = (float)cnt;
+            }
+            const bool uniform = __syncthreads_and(same);
             if (valid) {
                 const float4 *X = reinterpret_cast<const float4 *>(sl[t0 * PS + a]);
                 const float4 *Y = reinterpret_cast<const float4 *>(sl[t1 * PS + b]);
-                const float4 *Wt = reinterpret_cast<const float4 *>(sw);
                 float hi = 0.f, lo = 0.f;
-                for (int q4 = 0; q4 < (np + 3) / 4; ++q4) {
-                    const float4 x = X[q4], y = Y[q4], w = Wt[q4];
-                    df_add(hi, lo, __fmul_rn(x.x, w.x), y.x);
-                    df_add(hi, lo, __fmul_rn(x.y, w.y), y.y);
-                    df_add(hi, lo, __fmul_rn(x.z, w.z), y.z);
-                    df_add(hi, lo, __fmul_rn(x.w, w.w), y.w);
+                if (uniform) {
+#pragma unroll 2
+                    for (int q4 = 0; q4 < (np + 3) / 4; ++q4) {
+                        const float4 x = X[q4], y = Y[q4];
+                        df_add(hi, lo, x.x, y.x);
+                        df_add(hi, lo, x.y, y.y);
+                        df_add(hi, lo, x.z, y.z);
+                        df_add(hi, lo, x.w, y.w);
+                    }
+                    hi = __fmul_rn(hi, (float)w0);
+                    lo = __fmul_rn(lo, (float)w0);
+                } else {
+                    const float4 *Wt = reinterpret_cast<const float4 *>(sw);
+                    for (int q4 = 0; q4 < (np + 3) / 4; ++q4) {
+                        const float4 x = X[q4], y = Y[q4], w = Wt[q4];
+                        df_add(hi, lo, __fmul_rn(x.x, w.x), y.x);
+                        df_add(hi, lo, __fmul_rn(x.y, w.y), y.y);
+                        df_add(hi, lo, __fmul_rn(x.z, w.z), y.z);
+                        df_add(hi, lo, __fmul_rn(x.w, w.w), y.w);
+                    }
                 }
                 acc += (double)hi + (double)lo;
             }
             __syncthreads();
         }
     }
-    if (valid) partials[((size_t)(side == 0 ? 0 : nb_r) + blockIdx.x) * PER + t] = acc;
+    if (valid) partials[((size_t)(side == 0 ? 0 : nb_r) + blockIdx.x) * PER + ent] = acc;
 }
 
 // Sum of the blocks' partial sums, one warp per entry, fixed reduction tree.
 template <int C>
-__global__ void __launch_bounds__(256) k_cov_sum(const double *__restrict__ partials, int nb_r, int nb_c,
-                                                 double *__restrict__ totals) {
+__global__ void __launch_bounds__(256) k_cov_sum(const double *__restrict__ partials, int H, int W, int step,
+                                                 int ny, int nx, int nb_r, int nb_c, double *__restrict__ totals) {
     constexpr int NT = CovCfg<C>::NT, PER = CovCfg<C>::PER;
     const int lane = threadIdx.x & 31;
     const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -170,8 +221,18 @@ __global__ void __launch_bounds__(256) k_cov_sum(const double *__restrict__ part
     const int side = t / PER, e = t - side * PER;
     const int nblocks = side == 0 ? nb_r : nb_c;
     const double *part = partials + (size_t)(side == 0 ? 0 : nb_r) * PER + e;
+    int m, t0, t1, a, b;
+    task_of(t, PER, CovCfg<C>::NSYM, m, t0, t1, a, b);
+    // a derived entry: where its block left it to the next block's parent (a - step, b - step), the offset to that
+    auto in_tri = [](int i, int j) { return i * 8 - i * (i - 1) / 2 + (j - i); };
+    const bool derived = a >= step && b >= step;
+    const int next = PER - (t0 == t1 ? in_tri(a, b) - in_tri(a - step, b - step) : 9 * step);
     double sum = 0.0;
-    for (int bl = lane; bl < nblocks; bl += 32) sum += part[(size_t)bl * PER];
+#pragma unroll 4
+    for (int bl = lane; bl < nblocks; bl += 32) {
+        const bool other = derived && cov_shared(bl, nblocks, side == 0 ? H : W, side == 0 ? ny : nx, step);
+        sum += part[(size_t)bl * PER + (other ? next : 0)];
+    }
 #pragma unroll
     for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(FULL, sum, o);
     if (lane == 0) totals[t] = sum;
@@ -634,7 +695,7 @@ hts_status launch_basis_c(const float *img, const Geom &g, double *partials, dou
     if (hts_status st = check_launch("k_cov"); st != HTS_OK) return st;
     {
         KTimer kt("k_cov_sum", s);
-        k_cov_sum<C><<<(NT * 32 + 255) / 256, 256, 0, s>>>(partials, nb_r, nb_c, totals);
+        k_cov_sum<C><<<(NT * 32 + 255) / 256, 256, 0, s>>>(partials, g.H, g.W, g.step, g.ny, g.nx, nb_r, nb_c, totals);
     }
     if (hts_status st = check_launch("k_cov_sum"); st != HTS_OK) return st;
     {
