@@ -685,10 +685,17 @@ CONV_KERNELS = ("k_conv_tc", "k_conv_tma")
 
 def _kernel_rooflines(kernels, H, W, C, K, win, step, green):
     """Roofline of each main kernel of a step: the tensor-core matcher (issued BF16 MMA flops) and filter
-    (algorithmic transform flops) against the dense BF16/FP16 peak, the network forward and the normalisation
-    (algorithmic bytes) against the measured HBM bandwidth."""
+    (algorithmic transform flops) against the dense BF16/FP16 peak, the FP32 matcher (algorithmic flops; it shares
+    part of them between references) against the FP32 pipes, the network forward and the normalisation (algorithmic
+    bytes) against the measured HBM bandwidth."""
     peaks = _peaks()
     out = {}
+    if "k_match" in kernels:
+        peak = 152 * 128 * 2 * 2.07e9 / 1e12  # SMs x FP32 lanes x FMA x the highest SM clock
+        work = algorithmic_work(H, W, C, K, win, step)["k_match"]
+        ach = work["flops"] / (kernels["k_match"]["ms_per_launch"] / 1e3) / 1e12
+        out["k_match"] = {"kernel": "k_match", "bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
+                          "frac": ach / peak, "traffic": None, "algorithmic": work["per"]}
     for k in ("k_match_tc", "k_filter_tc"):
         if k in kernels:
             out[k] = _tc_roofline(k, kernels[k]["ms_per_launch"], H, W, C, K, win, step, green)
