@@ -1,0 +1,45 @@
+"""Rules of the CUDA sources that no run can show to be kept, read from the sources."""
+
+import glob
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2512_23569_gb300", "csrc")
+
+
+def _source(name):
+    with open(os.path.join(CSRC, name)) as f:
+        return re.sub(r"//[^\n]*", "", f.read())
+
+
+def _functions(src, qualifier):
+    """name -> (parameters, body) of the functions declared with `qualifier`."""
+    out = {}
+    for m in re.finditer(qualifier + r"\b", src):
+        n = re.compile(r"(\w+)\s*\(").search(src, m.end())
+        while n.group(1) in ("__launch_bounds__", "__align__"):
+            n = re.compile(r"(\w+)\s*\(").search(src, src.index(")", n.end()))
+        depth, i = 1, n.end()
+        while depth:
+            depth += {"(": 1, ")": -1}.get(src[i], 0)
+            i += 1
+        params = src[n.end():i - 1]
+        b = re.compile(r"[;{]").search(src, i)
+        if b.group() == ";":
+            continue  # a declaration
+        depth, j = 1, b.end()
+        while depth:
+            depth += {"{": 1, "}": -1}.get(src[j], 0)
+            j += 1
+        p, q = out.get(n.group(1), ("", ""))
+        out[n.group(1)] = (p + params, q + src[b.end():j])
+    return out
+
+
+def test_tensor_memory_loads_start_from_a_converged_warp():
+    loads = {k: body for k, (_, body) in _functions(_source("tc_ptx.h"), "__device__").items() if "tcgen05.ld." in body}
+    assert len(loads) >= 4
+    for name, body in loads.items():
+        sync = body.find("__syncwarp();")
+        assert 0 <= sync < body.index("tcgen05.ld."), name
+
