@@ -222,10 +222,11 @@ __global__ void __launch_bounds__(NTH, 2)
             uint32_t r[32];
             if (EPI == EPI_MAP) {
                 r[0] = tc::tmem_ld1(taddr);
+                tc::tmem_wait_ld(r[0]);
             } else {
                 tc::tmem_ld32(taddr, r);
+                tc::tmem_wait_ld(r);
             }
-            tc::tmem_wait_ld();
             epilogue_store<NOUT, EPI>(r, sBias, H, W, oy, ox, hout, map, hmask);
         }
         tc::fence_before();
@@ -351,10 +352,11 @@ __global__ void __launch_bounds__(NTH, 2)
             uint32_t r[32];
             if (EPI == EPI_MAP) {
                 r[0] = tc::tmem_ld1(taddr);
+                tc::tmem_wait_ld(r[0]);
             } else {
                 tc::tmem_ld32(taddr, r);
+                tc::tmem_wait_ld(r);
             }
-            tc::tmem_wait_ld();
             epilogue_store<NOUT, EPI>(r, sBias, H, W, oy, ox, hout, map, hmask);
         }
         tc::fence_before();
@@ -590,7 +592,7 @@ __global__ void __launch_bounds__(NTH, 3) k_conv_wgrad(const __grid_constant__ W
         for (int t = warp >> 2; t < 4; t += NTH / 128) {
             uint32_t v[32];
             tc::tmem_ld32(tbase + ((uint32_t)(32 * q) << 16) + (uint32_t)(t * 32), v);
-            tc::tmem_wait_ld();
+            tc::tmem_wait_ld(v);
             int orow = -1;
             if (t < 3) {
                 if (ky < 3) orow = ((ky * 3 + t) * cinx + gp) * 8 + ch;  // (tap, ci)

@@ -697,7 +697,7 @@ __global__ void __launch_bounds__(NT, 1) k_filter_tc(const __grid_constant__ Ftc
                 {
                     uint32_t v[16];
                     tc::tmem_ld16(tbase + tlane + (uint32_t)(16 * wq), v);
-                    tc::tmem_wait_ld();
+                    tc::tmem_wait_ld(v);
                     __align__(16) __half2 hv[8];
                     bool any = false;
 #pragma unroll
@@ -716,7 +716,8 @@ __global__ void __launch_bounds__(NT, 1) k_filter_tc(const __grid_constant__ Ftc
                     uint32_t vr[16], vi[16];
                     tc::tmem_ld16(tbase + tlane + (uint32_t)(64 + 16 * wq), vr);
                     tc::tmem_ld16(tbase + tlane + (uint32_t)(128 + 16 * wq), vi);
-                    tc::tmem_wait_ld();
+                    tc::tmem_wait_ld(vr);
+                    tc::tmem_wait_ld(vi);
                     const float t2c = 2.f * t2;
                     __align__(16) __half2 hr[8], hi[8];
                     bool any = false;

@@ -114,7 +114,7 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t base, uint32_t ncols) {
 
 // Tensor-memory loads by one whole warp (.sync.aligned: every lane executes the instruction together, so the warp is
 // brought together first: its lanes may come from a poll that each left on its own or from a store that only some
-// made).
+// made).  The registers hold the values only after tmem_wait_ld of them.
 // 32 lanes x 32 consecutive 32-bit columns: register j of lane l = column j of lane (quarter + l).
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
     __syncwarp();
@@ -151,9 +151,8 @@ __device__ __forceinline__ uint32_t tmem_ld1(uint32_t taddr) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr));
     return r;
 }
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-// The same wait, with the 32 destination registers of the loads it completes as operands, so that no use of
-// them is scheduled before it (for code that works between a load and its wait).
+// The wait for a warp's loads, with the destination registers of a load it completes as operands, so that no use of
+// them is scheduled before it (two loads: a wait for each, the second one done at once).
 __device__ __forceinline__ void tmem_wait_ld(uint32_t (&r)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;"
                  : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),

@@ -43,3 +43,7 @@ def test_tensor_memory_loads_start_from_a_converged_warp():
         sync = body.find("__syncwarp();")
         assert 0 <= sync < body.index("tcgen05.ld."), name
 
+
+def test_tensor_memory_waits_name_their_registers():
+    for path in glob.glob(os.path.join(CSRC, "*.*")):
+        assert not re.search(r"\btmem_wait_ld\(\s*\)", _source(os.path.basename(path))), path
