@@ -197,9 +197,9 @@ __global__ void k_reduce_grad(const float *__restrict__ part, int ntiles, int ne
 // so that the zeros and the gradient are one coalesced write (a block of 1024 threads over all patches
 // and its memset took two launches and 13 us on a 256 x 256 crop, this 10 between events).  The last block to finish adds the blocks' parts in
 // block order.
-__global__ void __launch_bounds__(256) k_loss(const float *__restrict__ outm, int H, int W, int step, int nx, int ny,
-                                              const float *__restrict__ target, float *__restrict__ dout,
-                                              double *lpart, double *loss) {
+__global__ void __launch_bounds__(256) k_loss(const float *outm, int H, int W, int step, int nx, int ny,
+                                              const float *target, float *__restrict__ dout, double *lpart,
+                                              double *loss) {
     __shared__ double red[8];
     __shared__ bool last;
     const int nref = nx * ny;

@@ -54,10 +54,10 @@ constexpr int EPI_RELU = 0, EPI_MAP = 1, EPI_MASK = 2;
 // The layer's weights B[tap][g][n][k] = w[n][8 g + k][tap], laid out so in global memory, and its biases, into shared
 // memory (gathering them from [n][ci][tap] took 2-byte loads with four divisions each: half of a small layer's time).
 template <int CING, int NOUT, int EPI>
-__device__ __forceinline__ void stage_weights(const __half *__restrict__ wp, const __half *__restrict__ wbias, int cout,
-                                              __half *sB, float *sBias, int tid) {
+__device__ __forceinline__ void stage_weights(const __half *wp, const __half *wbias, int cout, __half *sB,
+                                              float *sBias, int tid) {
     for (int e = tid; e < 9 * CING * NOUT; e += NTH)
-        reinterpret_cast<uint4 *>(sB)[e] = __ldg(reinterpret_cast<const uint4 *>(wp) + e);
+        reinterpret_cast<uint4 *>(sB)[e] = reinterpret_cast<const uint4 *>(wp)[e];
     if (EPI != EPI_MASK)
         for (int n = tid; n < NOUT; n += NTH) sBias[n] = n < cout ? __half2float(wbias[n]) : 0.f;
 }
@@ -114,9 +114,9 @@ struct ConvTcLayout {
 // epilogue (EPI_RELU, EPI_MAP, EPI_MASK with the activation planes hmask).
 template <int CING, int NOUT, int MT, bool IN_F32, int EPI>
 __global__ void __launch_bounds__(NTH, 2)
-    k_conv_tc(const float *__restrict__ img, int C, float in_scale, const __half *__restrict__ hin, int H, int W,
-              const __half *__restrict__ wp, const __half *__restrict__ wbias, int cout, __half *__restrict__ hout,
-              float *__restrict__ map, const __half *__restrict__ hmask, int *err) {
+    k_conv_tc(const float *img, int C, float in_scale, const __half *hin, int H, int W, const __half *wp,
+              const __half *wbias, int cout, __half *__restrict__ hout, float *__restrict__ map, const __half *hmask,
+              int *err) {
     using L = ConvTcLayout<CING, NOUT, MT>;
     constexpr int SX = L::SX, PX = L::PX;
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(NTH, 2)
                 const int y = y0 - 1 + py, x = x0 - 1 + px;
                 const bool in = e < PY * PX && y >= 0 && y < H && x >= 0 && x < W;
 #pragma unroll
-                for (int c = 0; c < 3; ++c) v[i][c] = (in && c < C) ? __ldg(img + c * HW + (size_t)y * W + x) : 0.f;
+                for (int c = 0; c < 3; ++c) v[i][c] = (in && c < C) ? img[c * HW + (size_t)y * W + x] : 0.f;
             }
 #pragma unroll
             for (int i = 0; i < NE; ++i) {
@@ -264,9 +264,8 @@ struct ConvTmaLayout {
 
 template <int NOUT, int EPI>
 __global__ void __launch_bounds__(NTH, 2)
-    k_conv_tma(const __grid_constant__ CUtensorMap tmap, int H, int W, const __half *__restrict__ wp,
-               const __half *__restrict__ wbias, int cout, __half *__restrict__ hout, float *__restrict__ map,
-               const __half *__restrict__ hmask, int *err) {
+    k_conv_tma(const __grid_constant__ CUtensorMap tmap, int H, int W, const __half *wp, const __half *wbias, int cout,
+               __half *__restrict__ hout, float *__restrict__ map, const __half *hmask, int *err) {
     using L = ConvTmaLayout<NOUT>;
     extern __shared__ __align__(1024) unsigned char smem[];
     __half *sB = reinterpret_cast<__half *>(smem + L::b_off);
@@ -630,7 +629,7 @@ __global__ void __launch_bounds__(256) k_wgrad_reduce(const __grid_constant__ Wg
     for (int b0 = 0; b0 < a.nblk; b0 += 32) {  // 32 loads in flight, added in block order
         float v[32];
 #pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] = b0 + i < a.nblk ? __ldg(p + (size_t)(b0 + i) * stride) : 0.f;
+        for (int i = 0; i < 32; ++i) v[i] = b0 + i < a.nblk ? p[(size_t)(b0 + i) * stride] : 0.f;
 #pragma unroll
         for (int i = 0; i < 32; ++i)
             if (b0 + i < a.nblk) s += v[i];

@@ -131,6 +131,9 @@ struct KTimer {
 // the launch attribute): grid_wait returns when every earlier grid has completed and its writes are visible, and every
 // thread calls it before its first access to memory that those write; grid_launch, called after it, lets the next
 // grid's blocks start once every block has called it -- so whatever ran before this grid is complete when they do.
+// Such a kernel's lifetime begins before the kernel before it has ended, so its input is not constant for that
+// lifetime: no __ldg and no const __restrict__ (which allow loads through the read-only path, and loads moved above
+// the wait) in these kernels, only plain loads, copies to shared memory and TMA.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

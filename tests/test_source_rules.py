@@ -47,3 +47,24 @@ def test_tensor_memory_loads_start_from_a_converged_warp():
 def test_tensor_memory_waits_name_their_registers():
     for path in glob.glob(os.path.join(CSRC, "*.*")):
         assert not re.search(r"\btmem_wait_ld\(\s*\)", _source(os.path.basename(path))), path
+
+
+def test_overlapping_kernels_read_nothing_as_constant():
+    """Kernels launched over the end of the one before (launch_chained): that one still writes their input after they
+    have begun, so neither they nor the functions they call read it as data constant for their lifetime."""
+    seen = set()
+    for name in ("cnn.cu", "cnn_tc.cu"):
+        src = _source(name)
+        chained = set(re.findall(r"launch_chained\(\s*\"\w+\",\s*(\w+)", src))
+        funcs = _functions(src, "__global__")
+        helpers = _functions(src, "__device__")
+        for k in chained:
+            params, body = funcs[k]
+            assert "grid_wait();" in body, k
+            for h, (hp, hb) in helpers.items():
+                if re.search(r"\b%s\s*(<[^;{}]*>)?\(" % h, body):
+                    params, body = params + "," + hp, body + hb
+            assert "__ldg" not in body, k
+            assert not re.search(r"const[^,]*\*\s*__restrict__", params), k
+            seen.add(k)
+    assert {"k_conv_tc", "k_conv_tma", "k_conv_wgrad", "k_wgrad_reduce", "k_loss"} <= seen
