@@ -173,10 +173,7 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs &g, int m0, int n0, int
     float4 bias = make_float4(0.f, 0.f, 0.f, 0.f);
     if ((EPI == EPI_BIAS || EPI == EPI_BIAS_RELU || EPI == EPI_LOSS) && gn < g.N)
         bias = *reinterpret_cast<const float4 *>(g.bias + gn);
-    // EPI_LOSS: sum of squared errors, a double-float (FP64 runs at a 64th of the rate), and in FP64 what FP32
-    // squares could not hold
-    float ls = 0.f, lc = 0.f;
-    double ld = 0.0;
+    double ls = 0.0;  // EPI_LOSS: sum of squared errors
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         const int gm = m0 + ty * 8 + i;
@@ -206,14 +203,7 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs &g, int m0, int n0, int
             for (int j = 0; j < 4; ++j) {
                 const float e = r[j] - (g.clean[o + j] - g.noisy[o + j]) / unit;
                 r[j] = 2.f * e / g.total;
-                if (fabsf(e) > 1e-12f && fabsf(e) < 1e12f) {
-                    const float p = __fmul_rn(e, e), pe = __fmaf_rn(e, e, -p);  // e^2 = p + pe exactly
-                    const float s = __fadd_rn(ls, p), t = __fsub_rn(s, ls);
-                    lc = __fadd_rn(lc, __fadd_rn(__fadd_rn(__fsub_rn(ls, __fsub_rn(s, t)), __fsub_rn(p, t)), pe));
-                    ls = s;
-                } else {
-                    ld += (double)e * e;
-                }
+                ls = fma((double)e, (double)e, ls);  // (the product is exact)
             }
         }
         *reinterpret_cast<float4 *>(g.out + o) = make_float4(r[0], r[1], r[2], r[3]);
@@ -225,7 +215,7 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs &g, int m0, int n0, int
     }
     if (EPI == EPI_LOSS) {
         __shared__ double red[GT / 32];
-        double s = ((double)ls + (double)lc) + ld;
+        double s = ls;
 #pragma unroll
         for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         if ((tid & 31) == 0) red[tid >> 5] = s;
