@@ -728,13 +728,24 @@ hts_status launch_cells(const MatchArgs &a, cudaStream_t s) {
         return ((size_t)(a.C == 3 ? 2 : 1) * (4 * (nry + 1) + 2 * a.R) * c.cols + (size_t)CX * c.ncp) * sizeof(float) +
                (size_t)(threads / 32) * CandList::LIST;
     };
-    // rows per tile: more share cells (n rows of references need n + 1 cell rows) but fill the SMs unevenly: the
-    // least work of the fullest SM, in thousands of warp instructions (a cell row 1.4 per warp, a row of references
-    // settled 4, the staging 2 per 3000 values)
+    int dev = 0, nsm = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    // rows per tile: more share cells (n rows of references need n + 1 cell rows) but leave fewer blocks, and an SM
+    // needs its 16 resident warps (the registers' limit) to hide a block's latencies: the work of a block, in thousands
+    // of warp instructions (a cell row 1.4 per warp, a row of references settled 4, the staging 2 per 3000 values), times
+    // the blocks of an SM and half a round of resident ones for the uneven end, or one round where they are fewer (no
+    // uneven end where only two are resident and all are: 512 x 512 x 3, win 31, seven rows a tile 150 us, four 169).
+    // With the blocks counted as if an SM ran them one by one, small windows (two to four warps a block) got tiles
+    // whose blocks left the SMs idle: 301 x 417 gray, K = 16, win 9: 104 us, now 46; 512 x 640 x 3, K = 32, win 15:
+    // 311 us, now 167.  Over 96 x 128 to 768 x 1024, K = 4 to 32 and windows 5 to 31 the choice is 2 % off the best.
+    const double resident = 512.0 / threads;
     double best = 0.0;
     for (int n = 8; n >= 1; --n) {
         const long blocks = (long)c.ntx * ((c.ry + n - 1) / n);
-        const double w = (double)((blocks + 151) / 152) *
+        const double per_sm = (double)blocks / nsm;
+        const double round = resident <= 2.0 && per_sm <= resident ? resident : std::max(resident, per_sm + 0.5 * resident);
+        const double w = round *
                          ((n + 1) * 1.4 * (threads / 32) + n * 4.0 +
                           (a.C == 3 ? 2 : 1) * (4 * (n + 1) + 2 * a.R) * c.cols * (2.0 / 3000.0));
         if (best == 0.0 || w < best) {
