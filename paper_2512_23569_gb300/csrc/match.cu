@@ -1,7 +1,8 @@
 // Grouping step of Haar-tSVD (Eq. 9, Alg. 1 step 1) on sm_103a.
 //
 // At the default grid step k_match_cells (below) shares the squared differences
-// of neighbouring references; for other steps and windows above 31, k_match:
+// of neighbouring references; for other steps, windows above 31 and grids too
+// small for it (cells_faster), k_match:
 //
 // A block of four warps takes a 2x2 block of reference patches and stages the
 // union of their search regions of the matching planes in shared memory
@@ -1036,12 +1037,25 @@ hts_status launch_direct(const MatchArgs &a, cudaStream_t s) {
     return check_launch("k_match");
 }
 
+// Whether the cell matcher takes a call at step 4 (windows whose offsets fit a block's threads: R <= 15).  Its blocks
+// settle rows of eight references in turn, so small grids leave it few warps, and a small window's distances, which
+// it halves, are the smaller part; the lines lie where a reference per warp (k_match) took as long (us, cells / k_match,
+// both with k_match_fallback; K = 16 where not given): 96 x 128 x 3 (713 references), win 15: 67 / 53; 203 x 317 x 3
+// (3950): 77 / 66, gray 44 / 46; 301 x 417 x 3 (7800): 76 / 86; 203 x 317 x 3, win 19: 68 / 73; 96 x 128 gray, win 21:
+// 38 / 40, colour 63 / 58; 512 x 640 gray (20193), K = 8, win 5: 83 / 71; 1080 x 1920 (128851), win 5: 0.83 to 0.89 of
+// k_match's time on gray, the same on colour.  At K = 32 k_match leaves most references of a wide window to the
+// exhaustive pass (96 x 128 gray, win 31: 41 / 543).
+inline bool cells_faster(int K, int C, int R, int nref) {
+    int R4;
+    if ((2 * R + 1) * cell_groups(R, &R4) > CT || (C == 3 && R <= 2)) return false;
+    int need = R <= 3 ? 40000 : R <= 7 ? 7000 : R <= 9 || C == 3 ? 3000 : 500;
+    if (K == 32 && R >= 13) need = 500;
+    return nref >= (K == 2 ? 2 * need : need);
+}
+
 template <int K>
 hts_status launch_k(const MatchArgs &a, cudaStream_t s) {
-    // the cells are cut for step 4, and a window's offsets have to fit a block's threads (R <= 15); at any image size
-    // they are the faster (96 x 128 gray, where each cell row serves one row of references: 38 us against 39)
-    int R4;
-    const bool cells = a.step == 4 && (2 * a.R + 1) * cell_groups(a.R, &R4) <= CT;
+    const bool cells = a.step == 4 && cells_faster(K, a.C, a.R, a.nref);
     const hts_status st = cells ? launch_cells<K>(a, s) : launch_direct<K>(a, s);
     if (st != HTS_OK) return st;
     {
