@@ -817,7 +817,8 @@ __global__ void __launch_bounds__(128) k_match_fallback(MatchArgs a) {
                 const int oi = __shfl_xor_sync(FULL, bi, o);
                 if (od < bd || (od == bd && oi < bi)) { bd = od; bi = oi; }
             }
-            if (lane == 0) out[1 + j] = bi;
+            // no candidate left with a distance (NaN pixels): the reference itself, a valid patch
+            if (lane == 0) out[1 + j] = bi == 0x7fffffff ? yr * a.W + xr : bi;
             if (il[0] == bi && dl[0] == bd) {
 #pragma unroll
                 for (int q = 0; q < L - 1; ++q) { dl[q] = dl[q + 1]; il[q] = il[q + 1]; }
