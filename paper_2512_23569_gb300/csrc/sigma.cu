@@ -422,11 +422,12 @@ __global__ void __launch_bounds__(VNT) k_vote(const float *__restrict__ img, int
             next = member(t + VNT / 32);  // in flight while this group is decided
             const int py = pos / W, px = pos - py * W;
             const bool inside = lane >= K || (py >= ry0 && py + PS - 1 <= ry1 && px >= rx0 && px + PS - 1 <= rx1);
-            const bool staged = __all_sync(FULL, inside);
-            const int mine = staged ? (py - ry0) * rs + (px - rx0) : pos;
-            if (staged && !HTS_IN_BOUNDS(lane >= K || mine + (C - 1) * (int)plane + (PS - 1) * rs + PS - 1 < C * (int)plane,
-                                         &st->error))
-                continue;  // (the check build: the staged region would be overrun)
+            const int at = (py - ry0) * rs + (px - rx0);
+            // (the check build: a group that would overrun the staged region reads the image, the whole warp together)
+            const bool staged = __all_sync(
+                FULL, inside && HTS_IN_BOUNDS(lane >= K || at + (C - 1) * (int)plane + (PS - 1) * rs + PS - 1 < C * (int)plane,
+                                              &st->error));
+            const int mine = staged ? at : pos;
             __syncwarp();
             if (lane < K) s_off[warp][lane] = mine;
             __syncwarp();

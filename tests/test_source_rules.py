@@ -68,3 +68,11 @@ def test_overlapping_kernels_read_nothing_as_constant():
             assert not re.search(r"const[^,]*\*\s*__restrict__", params), k
             seen.add(k)
     assert {"k_conv_tc", "k_conv_tma", "k_conv_wgrad", "k_wgrad_reduce", "k_loss"} <= seen
+
+
+def test_the_votes_bounds_check_keeps_the_warp_together():
+    """The check build's test is made by each lane for its own member: a lane that fails it may not leave the others to
+    the warp's barriers that follow."""
+    _, body = _functions(_source("sigma.cu"), "__global__")["k_vote"]
+    assert body.count("HTS_IN_BOUNDS") == len(re.findall(r"__all_sync\(\s*FULL,[^;]*HTS_IN_BOUNDS", body)) > 0
+    assert "continue;" not in body
