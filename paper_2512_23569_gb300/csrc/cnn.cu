@@ -674,7 +674,7 @@ extern "C" hts_status hts_cnn_log_sigma_map(hts_cnn *net, const float *img, int 
     HTS_TRY(check_net(net, img, H, W));
     if (!map_out) return report(HTS_EINVAL, "NULL pointer");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    HTS_TRY(cnn_ensure_infer(net, H, W, 1));
+    HTS_TRY(cnn_ensure_h16(net, H, W));
     return cnn_forward_tc_into(net, img, H, W, net->h16[0], net->h16[1], map_out, s);
 }
 

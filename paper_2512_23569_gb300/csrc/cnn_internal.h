@@ -42,16 +42,15 @@ struct hts_cnn {
 namespace hts {
 
 // Tensor-core forward pass (cnn_tc.cu): the log-sigma map of img (device,
-// planar C x H x W, [0, 255]) in net->map (H x W, FP32).  Hidden
-// activations are rounded to FP16 (8-channel planes, net->h16), the network
-// input x / 255 too; FP16 weights, FP32 accumulation in tensor memory.
-// cnn_ensure_infer sizes net->h16, net->map and net->rows first.
-hts_status cnn_forward_tc(hts_cnn *net, const float *img, int H, int W, cudaStream_t s);
-hts_status cnn_ensure_infer(hts_cnn *net, int H, int W, int nx);
-// The same forward into caller-owned buffers: h0, h1 (H * W * 32 halves each)
-// and map (H * W floats); only the weights and the error flag are the net's.
+// planar C x H x W, [0, 255]) in map (H x W, FP32).  Hidden activations are
+// rounded to FP16 (8-channel planes, in h0 and h1: H * W * 32 halves each), the
+// network input x / 255 too; FP16 weights, FP32 accumulation in tensor memory.
+// Only the weights and the error flag are the net's.
 hts_status cnn_forward_tc_into(hts_cnn *net, const float *img, int H, int W, __half *h0, __half *h1, float *map,
                                cudaStream_t s);
+// The net's own buffers: its activations h16; those, its map and its rows (for nx reference columns).
+hts_status cnn_ensure_h16(hts_cnn *net, int H, int W);
+hts_status cnn_ensure_infer(hts_cnn *net, int H, int W, int nx);
 struct Geom;
 // Training loss (added to net->loss) of the map over the reference patches and its gradient map (dout, every pixel).
 hts_status cnn_loss(hts_cnn *net, const float *map, int H, int W, const Geom &g, const float *target, float *dout,

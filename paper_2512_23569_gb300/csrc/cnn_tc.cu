@@ -694,23 +694,21 @@ hts_status grow_buf(T *&p, size_t &cap, size_t need) {
     return HTS_OK;
 }
 
-hts_status cnn_ensure_infer(hts_cnn *n, int H, int W, int nx) {
+hts_status cnn_ensure_h16(hts_cnn *n, int H, int W) {
     const size_t px = (size_t)H * W;
-    if (px * 32 > n->cap_h16 || !n->h16[1]) {
-        size_t c0 = 0;
-        hts_status st = grow_buf(n->h16[0], c0, px * 32);
-        size_t c1 = 0;
-        if (st == HTS_OK) st = grow_buf(n->h16[1], c1, px * 32);
-        n->cap_h16 = st == HTS_OK ? px * 32 : 0;
-        if (st != HTS_OK) return st;
-    }
-    const hts_status st = grow_buf(n->map, n->cap_map, px);
-    if (st != HTS_OK) return st;
-    return grow_buf(n->rows, n->cap_rows, (size_t)H * nx);
+    if (px * 32 <= n->cap_h16 && n->h16[1]) return HTS_OK;
+    size_t c0 = 0;
+    hts_status st = grow_buf(n->h16[0], c0, px * 32);
+    size_t c1 = 0;
+    if (st == HTS_OK) st = grow_buf(n->h16[1], c1, px * 32);
+    n->cap_h16 = st == HTS_OK ? px * 32 : 0;
+    return st;
 }
 
-hts_status cnn_forward_tc(hts_cnn *n, const float *img, int H, int W, cudaStream_t s) {
-    return cnn_forward_tc_into(n, img, H, W, n->h16[0], n->h16[1], n->map, s);
+hts_status cnn_ensure_infer(hts_cnn *n, int H, int W, int nx) {
+    hts_status st = cnn_ensure_h16(n, H, W);
+    if (st == HTS_OK) st = grow_buf(n->map, n->cap_map, (size_t)H * W);
+    return st == HTS_OK ? grow_buf(n->rows, n->cap_rows, (size_t)H * nx) : st;
 }
 
 hts_status cnn_forward_tc_into(hts_cnn *n, const float *img, int H, int W, __half *h0, __half *h1, float *map,
@@ -772,7 +770,7 @@ hts_status cnn_train_ensure(hts_cnn *n, int H, int W, int nsm) {
     return grow_buf(n->tr_part, n->tr_cap_part, (size_t)nsm * WG_PART);
 }
 
-// One image's loss and gradient on the tensor cores: the forward of cnn_forward_tc keeping every layer's
+// One image's loss and gradient on the tensor cores: the forward of cnn_forward_tc_into keeping every layer's
 // FP16 activations, the loss gradient map 2 (out - target) / N_ref times the loss scale 2^(floor(log2 N_ref)
 // + 2) (so (4, 8] times the error, well inside FP16's range) rounded to FP16, then from the last layer down the
 // gradient of the layer input (the forward kernels with the flipped, transposed weights, times the ReLU mask of
