@@ -970,18 +970,31 @@ __global__ void __launch_bounds__(RW * 32) k_match_rescue(MatchArgs a) {
             m = nless = 0;
             int cap = PMAX;  // of the candidates at T
             if (pass == 1) {
-                unsigned lo = 0u, hi = T;  // count(<= hi) >= L
+                // lo <= the L-th distance <= hi, both among the distances (so that ties, the common case, take few
+                // rounds: bisecting the bits took 31), until the list holds all up to hi, or lo and hi meet
+                unsigned lo = __shfl_sync(FULL, A, 0), hi = T;
                 while (lo < hi) {
                     const unsigned mid = lo + (hi - lo) / 2;
                     int n = 0;
-                    for (int i = 0; i < nch; ++i) n += db[32 * i + lane] <= mid ? 1 : 0;
-                    if (__reduce_add_sync(FULL, n) >= L) hi = mid;
-                    else lo = mid + 1;
+                    unsigned below = 0u, above = NONE;
+#pragma unroll 8
+                    for (int i = 0; i < nch; ++i) {
+                        const unsigned v = db[32 * i + lane];
+                        n += v <= mid ? 1 : 0;
+                        below = max(below, v <= mid ? v : 0u);
+                        above = min(above, v <= mid ? NONE : v);
+                    }
+                    n = __reduce_add_sync(FULL, n);
+                    if (n >= L) hi = __reduce_max_sync(FULL, below);
+                    else lo = __reduce_min_sync(FULL, above);
+                    if (n >= L && n <= PMAX) break;
                 }
                 T = hi;
                 int n = 0;
+#pragma unroll 8
                 for (int i = 0; i < nch; ++i) n += db[32 * i + lane] < T ? 1 : 0;
-                cap = L - __reduce_add_sync(FULL, n);  // fewer than L lie below
+                n = __reduce_add_sync(FULL, n);
+                if (n < L) cap = L - n;  // else the list holds them all
             }
             for (int i = 0; i < nch; ++i) {
                 const int e = 32 * i + lane;

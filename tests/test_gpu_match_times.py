@@ -33,3 +33,23 @@ def test_a_smaller_window_takes_no_longer(H, W, C, K, win, wide):
     _, noisy = synth.make_config_image(H, W, C, 20.0, 7 * H + W)
     x = torch.from_numpy(np.ascontiguousarray(noisy, dtype=np.float32)).cuda()
     assert _match_us(hts, x, K=K, win=win) <= _match_us(hts, x, K=K, win=wide)
+
+
+@pytest.mark.parametrize("C,win,step,noise,share", [(1, 31, 4, 1, 0.32), (3, 45, 2, 0, 0.19)])
+def test_the_exhaustive_pass_over_a_few_references_stays_short(C, win, step, noise, share):
+    """Some dozens of the references, ties among their candidates, against the tensor-core matching of all of them."""
+    from paper_2512_23569_gb300 import build, hts
+
+    build.build()
+    img = synth.make_config_image(400, 400, C, 20.0, 5)[noise]
+    x = torch.from_numpy(np.ascontiguousarray(img, dtype=np.float32)).cuda()
+    p = hts.params(K=16, win=win, step=step, precision=1)
+    hts.match(x, p=p)
+    assert 0 < hts.last_stats()["match_fallback"] < 100
+    times = []
+    for _ in range(7):
+        hts.profile_begin()
+        hts.match(x, p=p)
+        r = hts.profile_end()
+        times.append([r[k][0] for k in ("k_match_rescue", "k_match_tc")])
+    assert min(t[0] for t in times) <= share * min(t[1] for t in times)
