@@ -194,9 +194,9 @@ __global__ void k_reduce_grad(const float *__restrict__ part, int ntiles, int ne
 
 // Loss over the reference patches: mean of (out[centre] - target)^2 added to *loss; dout = 2 (out - target) / N_ref at
 // the patch centres, zero elsewhere.  Bound by its launch and one pass over the map: a block takes rows of the image,
-// so that the zeros and the gradient are one coalesced write (a block of 1024 threads over all patches
-// and its memset took two launches and 13 us on a 256 x 256 crop, this 10 between events).  The last block to finish adds the blocks' parts in
-// block order.
+// so that the zeros and the gradient are one coalesced write (a block of 1024 threads over all patches and its memset
+// took two launches and 13 us on a 256 x 256 crop, this 10 between events).  The last block to finish adds the blocks'
+// parts in a fixed order: 32 strided chains, then a tree.
 __global__ void __launch_bounds__(256) k_loss(const float *outm, int H, int W, int step, int nx, int ny,
                                               const float *target, float *__restrict__ dout, double *lpart,
                                               double *loss) {

@@ -1196,7 +1196,13 @@ hts_status launch_match_rescue(const float *img, const Geom &g, int32_t *idx, co
         const hts_status st0 = allow_smem(fn, smem);
         if (st0 != HTS_OK) return st0;
     }
-    const int blocks = 4 * 152;  // as many as are resident
+    int dev = 0, nsm = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    // four blocks an SM: resident together at windows up to 31 (44 KB of shared memory each); wider ones take fewer at
+    // a time, down to one at 63 (149 KB), where the pass still takes no longer than with a block per reference
+    // (400 x 400, step 1, win 63, 1187 references: 118 us, 147)
+    const int blocks = 4 * nsm;
     {
         KTimer kt("k_match_rescue", s);
         switch (g.K) {
