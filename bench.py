@@ -80,7 +80,9 @@ def _grid(n, step, ps=8):
 
 def algorithmic_work(H, W, C, K, win, step):
     """Algorithmic flops / bytes per launch of the main kernels: distances 3 flop x 64 px per candidate
-    pair, the filter's projections and Haar transforms per group, the normalisation's bytes per pixel."""
+    pair (at step 4 the squared differences are summed in 4 x 4 cells that the four references around one
+    share: 3 flop x 16 px and 3 additions of cell sums), the filter's projections and Haar transforms per
+    group, the normalisation's bytes per pixel."""
     ys, xs = _grid(H, step), _grid(W, step)
     R = (win - 1) // 2
     cy = [min(H - 8, y + R) - max(0, y - R) + 1 for y in ys]
@@ -96,9 +98,10 @@ def algorithmic_work(H, W, C, K, win, step):
         streams = 64
     haar = streams * 4 * (K - 1)
     per_group = 2 * (K * patch + haar)  # forward + inverse
+    per_pair, per_text = (64 * 3, "3 flop x 64 px per candidate pair") if step != 4 else (
+        16 * 3 + 3, "3 flop x 16 px and 3 additions per candidate pair (4 x 4 cells shared by four references)")
     return {
-        "k_match": {"flops": pairs * 64 * 3, "unit": "TFLOP/s", "per": "3 flop x 64 px per candidate pair",
-                    "units": pairs},
+        "k_match": {"flops": pairs * per_pair, "unit": "TFLOP/s", "per": per_text, "units": pairs},
         "k_filter": {"flops": nref * per_group, "unit": "TFLOP/s",
                      "per": "%d flop per group (8x8 projections fwd+inv, Haar fwd+inv)" % per_group,
                      "units": nref},
@@ -685,13 +688,13 @@ CONV_KERNELS = ("k_conv_tc", "k_conv_tma")
 
 def _kernel_rooflines(kernels, H, W, C, K, win, step, green):
     """Roofline of each main kernel of a step: the tensor-core matcher (issued BF16 MMA flops) and filter
-    (algorithmic transform flops) against the dense BF16/FP16 peak, the FP32 matcher (algorithmic flops; it shares
-    part of them between references) against the FP32 pipes, the network forward and the normalisation (algorithmic
+    (algorithmic transform flops) against the dense BF16/FP16 peak, the FP32 matcher (algorithmic flops) against
+    the FP32 pipes, the network forward and the normalisation (algorithmic
     bytes) against the measured HBM bandwidth."""
     peaks = _peaks()
     out = {}
     if "k_match" in kernels:
-        peak = 152 * 128 * 2 * 2.07e9 / 1e12  # SMs x FP32 lanes x FMA x the highest SM clock
+        peak = FP32_PEAK_TFLOPS
         work = algorithmic_work(H, W, C, K, win, step)["k_match"]
         ach = work["flops"] / (kernels["k_match"]["ms_per_launch"] / 1e3) / 1e12
         out["k_match"] = {"kernel": "k_match", "bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s",

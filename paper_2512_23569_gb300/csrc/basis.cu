@@ -47,7 +47,10 @@ __device__ __forceinline__ void pair_of(int p, int &a, int &b) {
 // I_t(y + a, col) I_t'(y + b, col), m_X(col) = number of grid positions x
 // with x <= col <= x + 7 (1 or 2 at step 4): one weighted dot product of two
 // image rows per grid row instead of one 8-term product per patch (and the
-// same along columns for N).  Multiplying by m_X (an integer <= 8) is exact.
+// same along columns for N).  Multiplying by m_X is exact where it is a power
+// of two; a count of 3, 5, 6 or 7 (beside a last grid position off the step,
+// or at steps 1 to 3) rounds the pixel's value once in FP32, which moves the
+// eigenvalues by about 1e-9 of the largest.
 // k_cov_sum adds the blocks' partial sums in FP64 in block order and forms
 // the Fourier-slice covariances C_row^(j) = (1/c) sum_{t,t'} w^{j(t-t')} M_tt',
 // C_col^(j) = (1/c) sum_{t,t'} w^{j(t'-t)} N_tt', w = exp(-2 pi i / c).
