@@ -431,8 +431,8 @@ __global__ void __launch_bounds__(MW * 32) k_match(MatchArgs a) {
 // warp minima), the candidates under it, then as k_match; the few references whose order FP64 decides wait for the
 // end of the tile, where they do not hold up a row.  Bound by issue (58-64 % active, 16 warps per SM) and, below
 // 1000 tiles, by the uneven filling of the SMs.  Measured against a reference per warp (k_match): 768 x 1024 gray,
-// K = 32, win 21: 191 us (562); 512 x 512 x 3, K = 16, win 31, beside the basis chain: 162 us (260); 1021 x 771 x 3:
-// 365 us (683).
+// K = 32, win 21: 184 us (562); 512 x 512 x 3, K = 16, win 31, beside the basis chain: 151 us (260); 1021 x 771 x 3:
+// 352 us (683).
 // Tiles are cut where the grid is: the last row / column of references, where H - 8 / W - 8 is no multiple of 4, are
 // tiles of their own.
 // Error: a term passes 2 roundings (difference, squared), at most 16 of the cell's chain and 2 of the cells' sums,

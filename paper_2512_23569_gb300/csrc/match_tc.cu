@@ -588,10 +588,13 @@ __global__ void __launch_bounds__(NT, 1) k_match_tc(const __grid_constant__ TcAr
                     if (lane == 0) tc::bar_arrive(&empty[b]);  // this warp is done with accumulator b
                     if (act && __any_sync(FULLM, vm != 0u)) {
                         const float4 *E4 = reinterpret_cast<const float4 *>(E + pb);
-                        // Bound by the pipe of logic, select and min / max operations, 9.5 of 11.5 a key (K <= 16) since
-                        // the clamp went into the multiply-add, the column's bits (the bin's number) out of the key
-                        // and the pushed-out keys into three-way minima; 14 operations before: 3840 x 2160 x 3, K = 16,
-                        // win 31: 2561 -> 2469 us, 1536 x 2048 x 3: 1018 -> 981 us.
+                        // 9.5 of the 11.5 operations a key (K <= 16) are logic, selects or min / max, which issue at
+                        // half rate: the clamp is the multiply-add's, the column's bits (the bin's number) join the
+                        // key after the runs and the pushed-out keys go through three-way minima.  Taking those out of
+                        // 14 gave 2561 -> 2469 us at 3840 x 2160 x 3, K = 16, win 31, and 1018 -> 981 us at 1536 x 2048 x
+                        // 3.  Not a full pipe, though: there that pipe is busy in 46 % of the cycles and issue in 41 %
+                        // (2.25 warps a scheduler, 14 % of the slots, of which the longest stalls are fixed latencies
+                        // and shared memory; 44 of 80 M shared wavefronts are the re-rank's bank conflicts).
                         const uint32_t pbh[2] = {(uint32_t)pb, (uint32_t)(pb + NBIN % 32)};
 #pragma unroll
                         for (int i4 = 0; i4 < 8; ++i4) {
