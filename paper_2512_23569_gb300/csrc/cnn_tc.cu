@@ -217,6 +217,7 @@ __global__ void __launch_bounds__(NTH, 2)
         const int q = warp & 3, m = 32 * q + lane;
         const int oy = y0 + (m >> 3);
         for (int j = warp >> 2; j < MT; j += 2) {
+            tc::converge();
             const int ox = x0 + 8 * j + (m & 7);
             const uint32_t taddr = tbase + ((uint32_t)(32 * q) << 16) + (uint32_t)(j * NOUT);
             uint32_t r[32];
@@ -346,6 +347,7 @@ __global__ void __launch_bounds__(NTH, 2)
         const int q = warp & 3, m = 32 * q + lane;
         const int oy = y0 + (m >> 3);
         for (int j = warp >> 2; j < MTH; j += 2) {
+            tc::converge();
             const int ox = x0 + 8 * j + (m & 7);
             const uint32_t taddr = tbase + ((uint32_t)(32 * q) << 16) + (uint32_t)(j * NOUT);
             uint32_t r[32];
@@ -589,6 +591,7 @@ __global__ void __launch_bounds__(NTH, 3) k_conv_wgrad(const __grid_constant__ W
         const int q = warp & 3, row = 32 * q + lane, gr = row >> 3, ch = row & 7;
         const int ky = gr / cinx, gp = gr - ky * cinx;
         for (int t = warp >> 2; t < 4; t += NTH / 128) {
+            tc::converge();
             uint32_t v[32];
             tc::tmem_ld32(tbase + ((uint32_t)(32 * q) << 16) + (uint32_t)(t * 32), v);
             tc::tmem_wait_ld(v);

@@ -575,6 +575,7 @@ __global__ void __launch_bounds__(NT, 1) k_filter_tc(const __grid_constant__ Ftc
             const int h = (K == 32) ? (rb >> 4) & 1 : 0;
 #pragma unroll
             for (int gi = 0; gi < 16 / KM; ++gi) {
+                tc::converge();  // each lane left the poll, or the atomics of the group before, by itself
                 const int g = rb / K + gi;
                 const int4 *offp = reinterpret_cast<const int4 *>(sOff + MB * buf + g * K + h * KM);
                 float mu = 0.f;  // first Haar row replaced (Eq. 24-25): the refined mean joins every member
@@ -694,6 +695,7 @@ __global__ void __launch_bounds__(NT, 1) k_filter_tc(const __grid_constant__ Ftc
                 const float sc = (ra && k == 0) ? 0.f : __int_as_float((127 - l) << 23);  // 2^-l; RA: row 0 replaced
                 unsigned char *rowp = sA + (m >> 3) * SBO_A + ((m & 7) << 4);
                 unsigned det = 0u;  // kept a detail coefficient: slice 1, slices 2-3
+                tc::converge();
                 {
                     uint32_t v[16];
                     tc::tmem_ld16(tbase + tlane + (uint32_t)(16 * wq), v);
@@ -716,8 +718,7 @@ __global__ void __launch_bounds__(NT, 1) k_filter_tc(const __grid_constant__ Ftc
                     uint32_t vr[16], vi[16];
                     tc::tmem_ld16(tbase + tlane + (uint32_t)(64 + 16 * wq), vr);
                     tc::tmem_ld16(tbase + tlane + (uint32_t)(128 + 16 * wq), vi);
-                    tc::tmem_wait_ld(vr);
-                    tc::tmem_wait_ld(vi);
+                    tc::tmem_wait_ld(vr, vi);
                     const float t2c = 2.f * t2;
                     __align__(16) __half2 hr[8], hi[8];
                     bool any = false;

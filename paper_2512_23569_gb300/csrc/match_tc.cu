@@ -568,6 +568,7 @@ __global__ void __launch_bounds__(NT, 1) k_match_tc(const __grid_constant__ TcAr
                     uint32_t vm = 0u;  // candidates pb .. pb+31 inside the window, without the reference
                     if (act) {
                         tc::fence_after();
+                        tc::converge();
                         tc::tmem_ld32(tbase + ((uint32_t)(32 * q) << 16) + b * RUNC + q * CH + 32 * hh, v);
                         if (mine) {
                             for (int y = ry, rs = pb - rx; rs <= pb + 31 && y <= rq.wy1; ++y, rs += Wq) {

@@ -36,12 +36,35 @@ def _functions(src, qualifier):
     return out
 
 
+def _loop_before(src, pos):
+    """The text from the start of the innermost loop body around `pos` up to it."""
+    depth = 0
+    for i in range(pos, -1, -1):
+        if src[i] == "}":
+            depth += 1
+        elif src[i] == "{":
+            if depth == 0:
+                head = src[max(0, i - 200):i].rstrip()
+                if re.search(r"\b(for|while) \([^{}]*\)$", head):
+                    return src[i:pos]
+            else:
+                depth -= 1
+    raise AssertionError("no loop")
+
+
 def test_tensor_memory_loads_start_from_a_converged_warp():
-    loads = {k: body for k, (_, body) in _functions(_source("tc_ptx.h"), "__device__").items() if "tcgen05.ld." in body}
-    assert len(loads) >= 4
-    for name, body in loads.items():
-        sync = body.find("__syncwarp();")
-        assert 0 <= sync < body.index("tcgen05.ld."), name
+    """tcgen05.ld is .sync.aligned: in the loop body that makes it, the warp is converged before it and after the
+    last poll, which its lanes leave one by one."""
+    calls = 0
+    for path in glob.glob(os.path.join(CSRC, "*.cu")):
+        src = _source(os.path.basename(path))
+        assert "tcgen05.ld." not in src  # only through the helpers
+        for m in re.finditer(r"tc::tmem_ld\d+\(", src):
+            before = _loop_before(src, m.start())
+            at = before.rfind("tc::converge();")
+            assert at >= 0 and not re.search(r"bar_wait|wait_bar\(", before[at:]), (path, src[m.start() - 80:m.end()])
+            calls += 1
+    assert calls >= 10
 
 
 def test_tensor_memory_waits_name_their_registers():
