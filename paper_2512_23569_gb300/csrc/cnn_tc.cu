@@ -56,8 +56,14 @@ constexpr int EPI_RELU = 0, EPI_MAP = 1, EPI_MASK = 2;
 template <int CING, int NOUT, int EPI>
 __device__ __forceinline__ void stage_weights(const __half *wp, const __half *wbias, int cout, __half *sB,
                                               float *sBias, int tid) {
-    for (int e = tid; e < 9 * CING * NOUT; e += NTH)
-        reinterpret_cast<uint4 *>(sB)[e] = reinterpret_cast<const uint4 *>(wp)[e];
+    constexpr int NV = 9 * CING * NOUT, NE = (NV + NTH - 1) / NTH;
+    uint4 v[NE];  // every load in flight before the first store
+#pragma unroll
+    for (int i = 0; i < NE; ++i)
+        if (tid + i * NTH < NV) v[i] = reinterpret_cast<const uint4 *>(wp)[tid + i * NTH];
+#pragma unroll
+    for (int i = 0; i < NE; ++i)
+        if (tid + i * NTH < NV) reinterpret_cast<uint4 *>(sB)[tid + i * NTH] = v[i];
     if (EPI != EPI_MASK)
         for (int n = tid; n < NOUT; n += NTH) sBias[n] = n < cout ? __half2float(wbias[n]) : 0.f;
 }
