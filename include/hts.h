@@ -206,7 +206,8 @@ typedef struct {
  * streams) and synchronises; later calls with the same signature reuse the
  * graph (updating it in place when pointers or sigma values change) and are
  * asynchronous.  The output equals hts_denoise's on each image, bit for bit,
- * whatever the tuning chose.  Up to 4 signatures are kept per process (least
+ * whatever the tuning chose (a plain-form image whose list of coefficients for
+ * FP64 decisions overflows, at very low noise, repeats to FP32 rounding only).  Up to 4 signatures are kept per process (least
  * recently used dropped, hts_shutdown frees all).  Calls are serialised
  * across host threads. */
 hts_status hts_denoise_batch(const hts_image *imgs, int n, const hts_params *p, void *stream);
@@ -281,7 +282,7 @@ hts_status hts_cnn_sigma_refs(hts_cnn *net, const float *img, int H, int W, cons
  * gradients accumulated in FP32.  hts_cnn_set_train_fp16(net, 0) selects
  * the FP32 kernels instead (FP32 activations and gradients); either setting
  * keeps FP32 master parameters and FP32 Adam state.  If a bounded wait of a
- * training kernel gives up, the layer's gradient becomes NaN. */
+ * training kernel gives up, every gradient of that image's step becomes NaN. */
 hts_status hts_cnn_set_train_fp16(hts_cnn *net, int on);
 int hts_cnn_train_fp16(const hts_cnn *net); /* 1: tensor-core training (default), 0: FP32, -1 for NULL */
 hts_status hts_cnn_zero_grad(hts_cnn *net, void *stream);
