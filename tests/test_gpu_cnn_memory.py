@@ -1,6 +1,8 @@
 """Device memory of the noise-map network's calls: log_sigma_map writes the caller's map, so the network allocates its
 two FP16 activation buffers (32 channels each) and nothing per pixel besides."""
 
+import gc
+
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -18,6 +20,7 @@ def test_the_noise_map_call_allocates_its_activations_only():
     net = hts.Cnn(1, seed=1)
     out = torch.empty(H, W, device="cuda")  # the map's place in torch's pool
     del out
+    gc.collect()
     torch.cuda.synchronize()
     before = torch.cuda.mem_get_info()[0]
     net.log_sigma_map(x)
